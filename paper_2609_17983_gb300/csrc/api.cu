@@ -7,11 +7,13 @@
 // attention -> O GEMM (+residual) -> RMSNorm -> gate/up GEMM -> SwiGLU ->
 // down GEMM (+residual).
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdlib>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -167,6 +169,8 @@ struct Rows {
   int max_pos = 0;                           // largest position among the rows
   const int4 *blocks = nullptr;              // attention query blocks (device)
   int n_blocks = 0, n_splits = 1, max_block_rows = 0;
+  const int4 *pairs = nullptr;               // two-tile kernel: pairs of blocks (device)
+  int n_pairs = 0;
   const CUtensorMap *tm_kv = nullptr;        // TMA view of the single document's pages
   const CUtensorMap *tmaps = nullptr;        // device [docs]: TMA views of a batch's pages
   bool tc5 = false;                          // attention on tcgen05 (set by plan_attention)
@@ -180,44 +184,131 @@ bool use_tc_attention(const kvr_model *m) {
   return m->dims.dtype == KVR_DTYPE_BF16 && (m->dims.dh == 64 || m->dims.dh == 128);
 }
 
+// Modelled time of an attention launch, in units of 0.1 us: CTAs of `per_page`
+// a 64-key page and `fixed` besides, ctas[i] of the key range pages[i] (longest
+// first), each range in `splits` parts.  One wave ends with its longest CTA;
+// more are dealt to the SMs as these fall free, longest first, so they end
+// about half a CTA after the mean.  A split pass also runs the combine.
+struct AttnCost {
+  int per_page, fixed;
+};
+constexpr AttnCost COST_TILE{10, 35}, COST_PAIR{11, 60};  // a pair's pages come two at a time
+constexpr int COST_COMBINE = 50;
+int attn_cost(const AttnCost &c, const std::vector<int> &pages, int heads, int splits, int sms) {
+  long long total = 0;
+  int longest = 0;
+  for (int np : pages) {
+    const int cta = c.per_page * ((np + splits - 1) / splits) + c.fixed;
+    total += (long long)cta * heads * splits;
+    longest = std::max(longest, cta);
+  }
+  const bool one_wave = (long long)pages.size() * heads * splits <= sms;
+  const int end = one_wave ? longest : std::max<int>(longest, (int)(total / sms) + longest / 2);
+  return end + (splits > 1 ? COST_COMBINE : 0);
+}
+
+// Key splits of the two-tile kernel's pairs: those that fill one wave, one or
+// two more, or none, whichever ends first.
+int pair_splits(const kvr_model *m, const std::vector<int> &pages, int &cost) {
+  const int ctas = (int)pages.size() * m->dims.G;
+  const int wave = std::max(1, m->num_sms / ctas);
+  const int longest = *std::max_element(pages.begin(), pages.end());
+  const int most = std::min((longest + 1) / 2, 64);
+  int best = 1;
+  cost = attn_cost(COST_PAIR, pages, m->dims.G, 1, m->num_sms);
+  for (int s = std::max(2, std::min(wave, most)); s <= std::min(most, wave + 2); ++s)
+    if (const int c = attn_cost(COST_PAIR, pages, m->dims.G, s, m->num_sms); c < cost)
+      best = s, cost = c;
+  return best;
+}
+
 // Query blocks for the tensor-core attention: consecutive rows of one
 // document (rows of a document are in ascending position order), at most
-// rows_per_block rows; and a key split count giving about two CTAs per SM.
+// rows_per_block rows; and a key split count giving about one wave of CTAs.
+// With the two-tile kernel the blocks are its tiles, and a table of pairs of
+// one document's tiles follows them, longest key range first (the last wave
+// then holds the shortest CTAs).
 kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32_t *rowdoc) {
   r.tc5 = false;
+  r.pairs = nullptr;
+  r.n_pairs = 0;
   if (!use_tc_attention(m) || r.M <= 0) return KVR_OK;
   const Dims &dm = m->dims;
   const int grp = dm.H / dm.G;
-  // the tcgen05 kernel (query blocks of up to 128 query vectors) when every
+  // the tcgen05 kernels (query blocks of up to 128 query vectors) when every
   // document has a TMA view of its pages, else the mma.sync kernel
   r.tc5 = m->use_tc5 && (rowdoc ? r.tmaps != nullptr : r.tm_kv != nullptr) &&
           attn_tc5_rows_per_block(grp) > 0;
   const int qb = r.tc5 ? attn_tc5_rows_per_block(grp) : attn_tc_rows_per_block(grp);
   std::vector<int32_t> b;
+  std::vector<std::array<int32_t, 4>> pairs;  // (first tile, tiles, kmax, doc)
   int max_chunks = 0, max_rows = 0;
-  for (int i = 0; i < r.M;) {
-    int doc = rowdoc ? rowdoc[i] : 0;
-    int e = i;
-    while (e < r.M && (rowdoc ? rowdoc[e] : 0) == doc) ++e;
-    // the document's rows in equal blocks of at most qb rows
-    const int nbd = (e - i + qb - 1) / qb, per = (e - i + nbd - 1) / nbd;
-    for (int j0 = i; j0 < e; j0 += per) {
-      const int j1 = std::min(e, j0 + per);
-      const int kmax = pos[j1 - 1];
-      max_rows = std::max(max_rows, j1 - j0);
-      b.insert(b.end(), {j0, j1 - j0, kmax, doc});
-      max_chunks = std::max(max_chunks, kmax / KVR_PAGE + 1);
+  // a document's rows in equal blocks of at most qb rows (`pair`: in whole pairs)
+  auto cut = [&](bool pair) {
+    b.clear();
+    pairs.clear();
+    max_chunks = max_rows = 0;
+    for (int i = 0; i < r.M;) {
+      int doc = rowdoc ? rowdoc[i] : 0;
+      int e = i;
+      while (e < r.M && (rowdoc ? rowdoc[e] : 0) == doc) ++e;
+      int nbd = (e - i + qb - 1) / qb;
+      if (pair && nbd > 1) nbd += nbd & 1;
+      const int per = (e - i + nbd - 1) / nbd;
+      for (int j0 = i; j0 < e; j0 += per) {
+        const int j1 = std::min(e, j0 + per);
+        const int kmax = pos[j1 - 1], tile = (int)b.size() / 4;
+        max_rows = std::max(max_rows, j1 - j0);
+        b.insert(b.end(), {j0, j1 - j0, kmax, doc});
+        max_chunks = std::max(max_chunks, kmax / KVR_PAGE + 1);
+        if (pair && ((j0 - i) / per) % 2 == 0)
+          pairs.push_back({tile, 1, kmax, doc});
+        else if (pair)
+          pairs.back()[1] = 2, pairs.back()[2] = kmax;
+      }
+      i = e;
     }
-    i = e;
+    return (int)b.size() / 4;
+  };
+  auto one_wave = [&](int nb) {
+    const int target = m->num_sms * (r.tc5 ? attn_tc5_ctas_per_sm(dm.dh) : 1), ctas = nb * dm.G;
+    const int s = r.tc5 ? std::max(1, target / ctas)  // one wave: no straggler CTAs
+                        : std::max(1, (target + ctas - 1) / ctas);
+    return std::min(std::min(s, max_chunks), 64);  // the combine merges <= 64 splits
+  };
+  // The two-tile kernel halves the time per tile and page, but its CTAs are
+  // half as many and twice as long: it is taken where the model says that its
+  // launch ends first (never with one or two tiles, whose CTAs it would
+  // leave alone on their SMs).
+  int nb = cut(false), splits = one_wave(nb);
+  if (r.tc5 && r.M > 2 * qb) {
+    std::vector<int> pages;
+    for (int t = 0; t < nb; ++t) pages.push_back(b[4 * t + 2] / KVR_PAGE + 1);
+    const int tile_cost = attn_cost(COST_TILE, pages, dm.G, splits, m->num_sms);
+    nb = cut(true);
+    pages.clear();
+    for (const auto &x : pairs) pages.push_back(x[2] / KVR_PAGE + 1);
+    int pair_cost = 0;
+    const int ps = pair_splits(m, pages, pair_cost);
+    if (pair_cost <= tile_cost) {
+      splits = ps;
+      std::stable_sort(pairs.begin(), pairs.end(),
+                       [](const auto &x, const auto &y) { return x[2] > y[2]; });
+    } else {
+      nb = cut(false);
+    }
   }
-  int nb = (int)b.size() / 4;
   if (nb > m->max_blocks) return fail(KVR_E_UNSUPPORTED, "too many attention blocks (%d)", nb);
-  // about one wave: as many CTAs as fit on the SMs at once
-  const int target = m->num_sms * (r.tc5 ? attn_tc5_ctas_per_sm(dm.dh) : 1);
-  int splits = r.tc5 ? std::max(1, target / (nb * dm.G))  // one wave: no straggler CTAs
-                     : std::max(1, (target + nb * dm.G - 1) / (nb * dm.G));
-  splits = std::min(std::min(splits, max_chunks), 64);  // the combine merges <= 64 splits
   while (splits > 1 && attn_tc_ws_floats(splits, nb, dm.G, dm.dh) > m->attn_ws_floats) --splits;
+  if (!pairs.empty()) {
+    // split ranges come from the pair's last key: the combine takes it from the tiles
+    if (splits > 1)
+      for (const auto &x : pairs)
+        for (int t = 0; t < x[1]; ++t) b[4 * (x[0] + t) + 2] = x[2];
+    for (const auto &x : pairs) b.insert(b.end(), x.begin(), x.end());
+    r.pairs = m->blocks_d + nb;
+    r.n_pairs = (int)pairs.size();
+  }
   KVR_TRY(stage_h2d(m, (int32_t *)m->blocks_d, b.data(), b.size()));
   r.blocks = m->blocks_d;
   r.n_blocks = nb;
@@ -283,10 +374,17 @@ kvr_status attention(kvr_model *m, const Rows &r, int l) {
     Prof pr(m, P_ATTN, kv_bytes);
     if (r.tc5) {
       static const CUtensorMap unused{};  // a batch's views come from r.tmaps
-      const char *e = launch_attention_tc5(
-          m->qb, r.pos, r.blocks, r.n_blocks, r.n_splits, dm, l, r.single.pages, r.single.table,
-          r.tm_kv ? *r.tm_kv : unused, m->attn_ws_o, m->attn_ws_ml, m->attn, m->dev_flag,
-          m->stream, r.tmaps ? r.views : nullptr, r.tmaps);
+      const CUtensorMap &tm = r.tm_kv ? *r.tm_kv : unused;
+      const KVView *views = r.tmaps ? r.views : nullptr;
+      const char *e =
+          r.pairs ? launch_attention_pair(m->qb, r.pos, r.blocks, r.n_blocks, r.pairs, r.n_pairs,
+                                          r.n_splits, dm, l, r.single.table, tm, m->attn_ws_o,
+                                          m->attn_ws_ml, m->attn, m->dev_flag, m->stream, views,
+                                          r.tmaps)
+                  : launch_attention_tc5(m->qb, r.pos, r.blocks, r.n_blocks, r.n_splits, dm, l,
+                                         r.single.pages, r.single.table, tm, m->attn_ws_o,
+                                         m->attn_ws_ml, m->attn, m->dev_flag, m->stream, views,
+                                         r.tmaps);
       if (!e)
         e = launch_attention_combine(r.blocks, r.n_blocks, r.max_block_rows, r.n_splits, dm,
                                      m->attn_ws_o, m->attn_ws_ml, m->attn, m->stream,
@@ -465,7 +563,8 @@ kvr_status run_pass(kvr_model *m, const Rows &r, bool kv_only) {
 kvr_status run_pass_graph(kvr_model *m, kvr_cache *c, const Rows &r) {
   if (!m->use_graphs || m->prof || m->stream == nullptr) return run_pass(m, r, true);
   for (auto &g : c->graphs)
-    if (g.M == r.M && g.nb == r.n_blocks && g.ns == r.n_splits && g.rows_out == r.rows_out) {
+    if (g.M == r.M && g.nb == r.n_blocks && g.np == r.n_pairs && g.ns == r.n_splits &&
+        g.rows_out == r.rows_out) {
       cudaError_t e = cudaGraphLaunch(g.exec, m->stream);
       if (e != cudaSuccess) return fail(KVR_E_CUDA, "graph launch: %s", cudaGetErrorString(e));
       m->launches += g.kernels;
@@ -486,7 +585,8 @@ kvr_status run_pass_graph(kvr_model *m, kvr_cache *c, const Rows &r) {
   e = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return fail(KVR_E_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-  c->graphs.push_back({r.M, r.n_blocks, r.n_splits, r.rows_out, m->launches - l0, exec});
+  c->graphs.push_back(
+      {r.M, r.n_blocks, r.n_pairs, r.n_splits, r.rows_out, m->launches - l0, exec});
   e = cudaGraphLaunch(exec, m->stream);
   if (e != cudaSuccess) return fail(KVR_E_CUDA, "graph launch: %s", cudaGetErrorString(e));
   return KVR_OK;
@@ -925,7 +1025,7 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
         (unsigned *)dev_alloc((size_t)(dm.L + 1) * gemm_chain_bar_words() * sizeof(unsigned));
     if (!m->chain_bar) return bail(fail(KVR_E_NOMEM, "chain counters"));
     // positions and tokens of a pass, plus the tables of a 256-document batch
-    m->stage_cap = std::max<size_t>(R * 4, P) + 4096 +
+    m->stage_cap = std::max<size_t>(R * 8, P) + 4096 +
                    256 * (sizeof(CUtensorMap) + sizeof(KVView) + sizeof(void *)) / 4;
     if (cudaMallocHost(&m->stage_h, m->stage_cap * sizeof(int32_t)) != cudaSuccess)
       return bail(fail(KVR_E_NOMEM, "pinned staging"));
@@ -993,7 +1093,7 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
   if (use_tc_attention(m)) {
     m->max_blocks = dm.max_rows + 256;
     m->attn_ws_floats = (size_t)16 << 20;  // 64 MB of split-KV partials
-    m->blocks_d = (int4 *)dev_alloc((size_t)m->max_blocks * sizeof(int4));
+    m->blocks_d = (int4 *)dev_alloc((size_t)2 * m->max_blocks * sizeof(int4));
     m->attn_ws_o = (float *)dev_alloc(m->attn_ws_floats * sizeof(float));
     m->attn_ws_ml = (float2 *)dev_alloc(m->attn_ws_floats / dm.dh * sizeof(float2));
     if (!m->blocks_d || !m->attn_ws_o || !m->attn_ws_ml)
@@ -1917,6 +2017,7 @@ kvr_status kvr_linear(kvr_model *m, const char *name, int32_t layer, const void 
 
 static cudaError_t trace_attach_all(const TraceBuf &b) {
   cudaError_t e = trace_attach_rows(b);
+  if (e == cudaSuccess) e = trace_attach_attn_pair(b);
   if (e == cudaSuccess) e = trace_attach_gemm(b);
   if (e == cudaSuccess) e = trace_attach_attn(b);
   if (e == cudaSuccess) e = trace_attach_attn5(b);

@@ -293,7 +293,7 @@ struct kvr_cache {
   std::vector<int32_t> tokens_h;
   bool poisoned = false;
   struct Graph {
-    int M, nb, ns;
+    int M, nb, np, ns;
     const void *rows_out;  // kvr_repair_read's row buffer, or null
     int64_t kernels;
     cudaGraphExec_t exec;
@@ -404,6 +404,7 @@ cudaError_t trace_attach_rows(const TraceBuf &b);
 cudaError_t trace_attach_gemm(const TraceBuf &b);
 cudaError_t trace_attach_attn(const TraceBuf &b);
 cudaError_t trace_attach_attn5(const TraceBuf &b);
+cudaError_t trace_attach_attn_pair(const TraceBuf &b);
 cudaError_t trace_attach_select(const TraceBuf &b);
 
 // ---- programmatic dependent launch (PDL) ----
@@ -588,6 +589,17 @@ const char *launch_attention_tc5(const void *q, const int32_t *pos, const int4 *
                                  float *ws_o, float2 *ws_ml, void *out, int *dev_flag,
                                  cudaStream_t s, const KVView *views = nullptr,
                                  const CUtensorMap *tmaps = nullptr);
+
+// The same over many rows: the blocks are tiles of at most
+// attn_tc5_rows_per_block(grp) rows, and each CTA takes a pair (device int4:
+// first tile, tiles 1 or 2, kmax of the pair, doc).  With n_splits > 1 the
+// tiles of a pair carry the pair's kmax.
+const char *launch_attention_pair(const void *q, const int32_t *pos, const int4 *blocks,
+                                  int n_blocks, const int4 *pairs, int n_pairs, int n_splits,
+                                  const Dims &dm, int layer, const int32_t *table,
+                                  const CUtensorMap &tm_kv, float *ws_o, float2 *ws_ml, void *out,
+                                  int *dev_flag, cudaStream_t s, const KVView *views = nullptr,
+                                  const CUtensorMap *tmaps = nullptr);
 
 // ---- kernels: selectors ----
 // The keys of a simple policy (EditLocal, Structural, Random,

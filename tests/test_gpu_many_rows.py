@@ -1,0 +1,77 @@
+"""The kernels of passes with many rows at the sizes where they can go wrong,
+against the oracle: two query tiles per CTA in the attention (odd tile counts,
+ragged tiles, split and unsplit key ranges, several documents)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2609_17983_gb300 import synth
+
+try:
+    from paper_2609_17983_gb300 import kvrepair as kv
+except ImportError as _e:  # pragma: no cover
+    kv, _IMPORT_ERROR = None, _e
+
+pytestmark = pytest.mark.gpu
+TOL = 2e-2  # bf16 path, as everywhere
+
+
+def rel(a, b):
+    return float(np.abs(a - b).max() / np.abs(b).max())
+
+
+def small_cfg(**over):
+    return synth.preset("tiny", dtype="bf16", d_model=512, ffn=512, **over)
+
+
+def loaded(model, cfg, n, seed):
+    doc = synth.document(seed, n, cfg["vocab"])
+    k, v = synth.kv_rows(seed, n, cfg["n_layers"], cfg["n_kv_heads"], cfg["head_dim"], "bf16",
+                         std=0.45)
+    to = lambda x: np.ascontiguousarray(synth.bf16_bits_to_f32(x).transpose(1, 0, 2, 3))  # noqa: E731
+    return model.load_cache(doc, k, v), oracle.Cache(to(k), to(v), doc.copy())
+
+
+def check_rows(cfg, cache, ref, P):
+    gk, gv = cache.read(P)
+    for l in range(cfg["n_layers"]):
+        assert rel(gk[:, l], ref.k[l, P]) <= TOL and rel(gv[:, l], ref.v[l, P]) <= TOL, l
+
+
+# (heads, kv heads, head_dim, n, rows, how): a key range split over CTAs with
+# whole and with odd pairs of ragged tiles (7 heads a kv head: tiles of 126
+# vectors), and one CTA per pair over many waves
+@pytest.mark.parametrize("H,G,dh,n,rows,how", [(8, 2, 128, 2300, 1100, "window"),
+                                               (14, 2, 64, 2300, 701, "scatter"),
+                                               (32, 8, 64, 2400, 2400, "window")])
+def test_attention_pairs_of_tiles(H, G, dh, n, rows, how):
+    cfg = small_cfg(n_heads=H, n_kv_heads=G, head_dim=dh)
+    W = synth.weights(cfg, 0)
+    model = kv.Model(cfg, None, seed=0, max_context=4096, max_rows=4096)
+    cache, ref = loaded(model, cfg, n, 11)
+    A = (np.arange(n - rows, n) if how == "window" else
+         np.sort(np.random.default_rng(1).permutation(np.arange(200, n))[:rows]))
+    none = np.zeros(0, np.int32)
+    cache.repair(none, 0, A)
+    ref = oracle.repair(cfg, W, ref, none, 0, A)
+    check_rows(cfg, cache, ref, A)
+    model.close()
+
+
+def test_attention_pairs_of_several_documents():
+    cfg = small_cfg(n_heads=8, n_kv_heads=2, head_dim=128)
+    W = synth.weights(cfg, 0)
+    model = kv.Model(cfg, None, seed=0, max_context=4096, max_rows=4096)
+    docs = [loaded(model, cfg, n, 20 + n) for n in (2300, 1501, 700)]
+    rng = np.random.default_rng(2)
+    reqs, want = [], []
+    for (cache, ref), rows in zip(docs, (900, 601, 20)):  # odd tile counts, a lone tile
+        s = 100
+        new = synth.edit_tokens(3, ref.tokens[s:s + 5], cfg["vocab"])
+        A = np.sort(rng.permutation(np.arange(s + 5, cache.n))[:rows])
+        reqs.append((cache, [(s, new)], A))
+        want.append(oracle.repair(cfg, W, ref, new, s, A))
+    model.repair_batch(reqs)
+    for (cache, edits, A), ref in zip(reqs, want):
+        check_rows(cfg, cache, ref, np.concatenate([np.arange(100, 105), A]))
+    model.close()
