@@ -482,7 +482,7 @@ void launch_cache_scatter_raw(KVView v, int dtype, int p0, int n_pos, const void
 void launch_rows_copy(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
                       void *buf, bool to_buf, cudaStream_t s);
 void launch_transplant(KVView dst, KVView src, int dtype, const int32_t *pos, int n_pos,
-                       cudaStream_t s);
+                       int32_t *tok_dst, const int32_t *tok_src, cudaStream_t s);
 void launch_row_logprob(const float *logits, int rows, int V, const int32_t *target, float *out,
                         cudaStream_t s);
 

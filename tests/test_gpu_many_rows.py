@@ -1,6 +1,7 @@
 """The kernels of passes with many rows at the sizes where they can go wrong,
 against the oracle: two query tiles per CTA in the attention (odd tile counts,
-ragged tiles, split and unsplit key ranges, several documents)."""
+ragged tiles, split and unsplit key ranges, several documents), vector row
+kernels."""
 import numpy as np
 import pytest
 
@@ -74,4 +75,18 @@ def test_attention_pairs_of_several_documents():
     model.repair_batch(reqs)
     for (cache, edits, A), ref in zip(reqs, want):
         check_rows(cfg, cache, ref, np.concatenate([np.arange(100, 105), A]))
+    model.close()
+
+
+@pytest.mark.parametrize("vocab", [1024, 1021])
+def test_answer_logprob_row_widths(vocab):
+    # rows on 16-byte boundaries, and rows that are not
+    cfg = synth.preset("tiny", vocab=vocab)
+    W = synth.weights(cfg, 0)
+    model = kv.Model(cfg, None, seed=0, max_context=256, max_rows=256)
+    doc = synth.document(5, 100, vocab)
+    prompt, answer = synth.fill_tokens(6, 7, vocab, 13), synth.fill_tokens(7, 5, vocab, 13)
+    got = model.answer_logprob(model.prefill(doc), prompt, answer)
+    want = oracle.answer_logprob(cfg, W, oracle.prefill(cfg, W, doc), prompt, answer)
+    assert abs(got - want) <= 1e-4 * abs(want)  # the fp32 path's tolerance
     model.close()
