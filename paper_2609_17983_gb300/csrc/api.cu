@@ -2016,6 +2016,7 @@ static cudaError_t trace_attach_all(const TraceBuf &b) {
   cudaError_t e = trace_attach_rows(b);
   if (e == cudaSuccess) e = trace_attach_attn_pair(b);
   if (e == cudaSuccess) e = trace_attach_gemm(b);
+  if (e == cudaSuccess) e = trace_attach_gemm_pair(b);
   if (e == cudaSuccess) e = trace_attach_attn(b);
   if (e == cudaSuccess) e = trace_attach_attn5(b);
   if (e == cudaSuccess) e = trace_attach_select(b);

@@ -280,12 +280,12 @@ __global__ void __launch_bounds__(ROPE_HEADS * 64) k_rope_scatter(const RopeArgs
   }
 }
 
-// Hundreds of rows and more: four rotated pairs per thread (16-byte loads, 8- or
+// Many rows: four rotated pairs per thread (16-byte loads, 8- or
 // 16-byte stores), and without a split view ROPE_RPB rows at a time, all their
 // loads in flight together.  One pair per thread, 2-byte stores: 75 us for 4096
 // rows of a 6144-wide projection (100 MB read, 50 MB written, 2.0 TB/s).
 constexpr int ROPE_RPB = 4, ROPE_THREADS = 256;
-constexpr int ROPE_MANY = 128;  // rows from which it is taken
+constexpr int ROPE_MANY = 64;  // rows from which it is taken (40 rows: equal; 64 rows: 9.9 -> 8.2 us)
 template <typename T, int RPB>
 __global__ void __launch_bounds__(ROPE_THREADS) k_rope_rows(const RopeArgs a) {
   TraceScope ts(TK_ROPE);

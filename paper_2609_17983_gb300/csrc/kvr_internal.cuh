@@ -402,6 +402,7 @@ struct TraceScope {
 #endif
 cudaError_t trace_attach_rows(const TraceBuf &b);
 cudaError_t trace_attach_gemm(const TraceBuf &b);
+cudaError_t trace_attach_gemm_pair(const TraceBuf &b);
 cudaError_t trace_attach_attn(const TraceBuf &b);
 cudaError_t trace_attach_attn5(const TraceBuf &b);
 cudaError_t trace_attach_attn_pair(const TraceBuf &b);
@@ -546,6 +547,11 @@ struct ChainStep {
 size_t gemm_chain_bar_words();
 const char *launch_gemm_chain(const ChainStep *steps, int n, const TcWorkspace &ws, unsigned *bar,
                               cudaStream_t s, SplitView *last_defer);
+// Many rows (k_gemm_pair.cu): pairs of CTAs on 256-feature tiles; Y is always
+// complete.  launch_gemm_tc hands them over.
+bool gemm_pair_takes(int M, int N, int K, int epi);
+const char *launch_gemm_pair(const GemmArgs &g, const CUtensorMap &tmW, int epi, void *out2,
+                             int ld2, const TcWorkspace &ws, cudaStream_t s);
 const char *launch_gemm_tc(const GemmArgs &g, const CUtensorMap &tmW, int epi, void *out2,
                            int ld2, const TcWorkspace &ws, cudaStream_t s,
                            SplitView *defer = nullptr);

@@ -1,6 +1,8 @@
 """The kernels of passes with many rows at the sizes where they can go wrong,
-against the oracle: two query tiles per CTA in the attention (odd tile counts,
-ragged tiles, split and unsplit key ranges, several documents), vector row
+against the oracle and float64 products: two query tiles per CTA in the
+attention (odd tile counts, ragged tiles, split and unsplit key ranges,
+several documents), pairs of CTAs per tile in the GEMM (ragged token tiles, a
+feature count that is an odd multiple of 128, few K blocks), vector row
 kernels."""
 import numpy as np
 import pytest
@@ -76,6 +78,30 @@ def test_attention_pairs_of_several_documents():
     for (cache, edits, A), ref in zip(reqs, want):
         check_rows(cfg, cache, ref, np.concatenate([np.arange(100, 105), A]))
     model.close()
+
+
+@pytest.mark.parametrize("M", [961, 1537])
+def test_gemm_pairs_of_ctas(M):
+    # 7040, 4224 and 8576 output features: odd multiples of 128, so the last
+    # feature tile is half empty; 66 and 67 K blocks (the last unit of two is
+    # short), ragged token tiles, tiles split over clusters; a sample of rows
+    cfg = synth.preset("llama8b", n_layers=1, d_model=4224, n_heads=33, n_kv_heads=11, ffn=4288,
+                       vocab=1024)
+    m = kv.Model(cfg, None, seed=0, max_context=256, max_rows=2048)
+    f64 = lambda b: synth.bf16_bits_to_f32(b).astype(np.float64)  # noqa: E731
+    x, xd = (synth.tensor(M, t, (M, k), "bf16", std=1.0) for t, k in ((5, 4224), (6, 4288)))
+    at = np.unique(np.concatenate([np.arange(0, M, 61), np.arange(M - 5, M)]))
+    wqkv = np.concatenate([m.read_tensor(n, 0) for n in ("wq", "wk", "wv")])
+    # fp32 sums of exact products: 1e-3 as for the other GEMMs; SwiGLU rounds to bf16
+    for name, w, y in (("wqkv", wqkv, x), ("wo", m.read_tensor("wo", 0), x),
+                       ("wd", m.read_tensor("wd", 0), xd)):
+        got = kv.kvr_linear(m.h, name, 0, y, w.shape[0])[at]
+        assert rel(got, f64(y[at]) @ f64(w).T) <= 1e-3, name
+    g = f64(x[at]) @ f64(m.read_tensor("wg", 0)).T
+    u = f64(x[at]) @ f64(m.read_tensor("wu", 0)).T
+    got = kv.kvr_linear(m.h, "wgu", 0, x, 4288)[at]
+    assert rel(got, g / (1.0 + np.exp(-g)) * u) <= 1e-2
+    m.close()
 
 
 @pytest.mark.parametrize("vocab", [1024, 1021])

@@ -553,9 +553,8 @@ def test_8b_shape_two_layer_parity(shape, chain, monkeypatch):
 
 
 def test_8b_shape_prefill_many_rows_parity():
-    # a prefill chunk of 600 rows: enough for the GEMMs' grouped data-parallel
-    # tiling (whole tiles per CTA, a ragged last token tile) where it fills
-    # the SMs (the QKV projection here), stream-K elsewhere; every row's K/V
+    # a prefill chunk of 600 rows: the gate/up and down GEMMs on pairs of CTAs,
+    # stream-K over several ragged token tiles for the others; every row's K/V
     # at both layers against the oracle's prefill
     cfg = synth.preset("llama8b", n_layers=2)
     n = 600
