@@ -4,7 +4,7 @@
 // layer-major pass of the repair operator R (Sec. 3, Eq. 1) on the model's
 // stream: embedding gather of the rows, then per layer RMSNorm -> QKV GEMM ->
 // RoPE at the original positions + K/V scatter of all rows -> scattered-query
-// attention -> O GEMM (+residual) -> RMSNorm -> gate/up GEMM -> SwiGLU ->
+// attention -> O GEMM (+residual) -> RMSNorm -> gate/up GEMM (SwiGLU) ->
 // down GEMM (+residual).
 #include <algorithm>
 #include <array>
@@ -128,8 +128,8 @@ kvr_status stage_h2d(kvr_model *m, int32_t *dst_dev, const int32_t *src, size_t 
 // ------------------------------------------------------------ GEMM dispatch
 
 // Y (+)= X W^T through the tensor-core kernel when the weight has a TMA
-// descriptor, else the FFMA kernel.  epi selects the epilogue; for SwiGLU
-// the FFMA path writes gate/up to m->gu and runs the SwiGLU kernel.
+// descriptor, else the FFMA kernel.  epi selects the epilogue (SwiGLU goes to
+// m->act).
 // defer: split tiles of the tensor-core GEMM are left to the kernel that
 // next reads Y, which must take *defer (ws null when Y is complete).
 kvr_status gemm(kvr_model *m, int cls, const void *X, const void *W, const CUtensorMap *tm,
@@ -145,14 +145,8 @@ kvr_status gemm(kvr_model *m, int cls, const void *X, const void *W, const CUten
     if (e) return fail(KVR_E_CUDA, "tensor-core GEMM (M=%d N=%d K=%d): %s", M, N, K, e);
     return launch_check(m, 1);
   }
-  if (epi == GEMM_EPI_SWIGLU) {
-    GemmArgs g{X, W, nullptr, m->gu, M, N, K, K, N, dm.dtype, 0};
-    launch_gemm_simt(g, m->stream);
-    launch_swiglu(m->gu, M, N / 2, m->act, dm.dtype, m->stream);
-    return launch_check(m, 2);
-  }
   GemmArgs g{X, W, bias, Y, M, N, K, K, N, dm.dtype, epi == GEMM_EPI_ACCUM};
-  launch_gemm_simt(g, m->stream);
+  launch_gemm_simt(g, epi == GEMM_EPI_SWIGLU ? m->act : nullptr, m->num_sms, m->stream);
   return launch_check(m, 1);
 }
 
@@ -399,8 +393,8 @@ kvr_status attention(kvr_model *m, const Rows &r, int l) {
       if (e) return fail(KVR_E_CUDA, "attention: %s", e);
       KVR_TRY(launch_check(m, r.n_splits > 1 ? 2 : 1));
     } else {
-      launch_attention_simt(m->q, r.pos, r.M, dm, l, r.views, r.rowdoc, r.single, m->attn,
-                            m->stream);
+      launch_attention_simt(m->q, r.pos, r.M, dm, l, r.views, r.rowdoc, r.single,
+                            (float *)m->attn, m->stream);
       KVR_TRY(launch_check(m, 1));
     }
   }
@@ -989,7 +983,7 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
   {
     size_t R = dm.max_rows, P = dm.max_ctx + KVR_QUERY_RESERVE;
     size_t sz[] = {R * 4,          R * 4,          R * d * 4,        R * d * es,  R * Nq * 4,
-                   R * HD * 4,     R * HD * es,    R * 2 * F * 4,    R * F * es,
+                   R * HD * 4,     R * HD * es,    R * F * es,
                    (size_t)KVR_QUERY_RESERVE * V * 4,
                    P * 4,          P * 8,          P * 4,            256,         R * HD * 2};
     size_t tot = 0;
@@ -997,8 +991,8 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
     m->ws_block = dev_alloc(tot);
     if (!m->ws_block) return bail(fail(KVR_E_NOMEM, "workspace: %zu bytes", tot));
     char *p = (char *)m->ws_block;
-    void *ptrs[15];
-    for (int i = 0; i < 15; ++i) {
+    void *ptrs[14];
+    for (int i = 0; i < 14; ++i) {
       ptrs[i] = p;
       p += al(sz[i]);
     }
@@ -1009,14 +1003,13 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
     m->qkv = (float *)ptrs[4];
     m->q = (float *)ptrs[5];
     m->attn = ptrs[6];
-    m->gu = (float *)ptrs[7];
-    m->act = ptrs[8];
-    m->logits = (float *)ptrs[9];
-    m->scores = (float *)ptrs[10];
-    m->keys = (unsigned long long *)ptrs[11];
-    m->sel_out = (int32_t *)ptrs[12];
-    m->sel_count = (int32_t *)ptrs[13];
-    m->qb = ptrs[14];
+    m->act = ptrs[7];
+    m->logits = (float *)ptrs[8];
+    m->scores = (float *)ptrs[9];
+    m->keys = (unsigned long long *)ptrs[10];
+    m->sel_out = (int32_t *)ptrs[11];
+    m->sel_count = (int32_t *)ptrs[12];
+    m->qb = ptrs[13];
     m->dev_flag = (int *)dev_alloc(256);
     if (!m->dev_flag) return bail(fail(KVR_E_NOMEM, "flag"));
     cudaMemset(m->dev_flag, 0, 256);

@@ -1,6 +1,6 @@
 // k_rows.cu -- per-row kernels of the repair pass: seeded weight init,
 // embedding gather, RMSNorm, RoPE + K/V scatter into the paged cache,
-// SwiGLU, and cache row readback / save / restore.
+// and cache row readback / save / restore.
 #include "kvr_internal.cuh"
 
 namespace kvr {
@@ -362,19 +362,6 @@ __global__ void __launch_bounds__(ROPE_THREADS) k_rope_rows(const RopeArgs a) {
 }
 
 template <typename T>
-__global__ void k_swiglu(const float *gu, int M, int F, T *act) {
-  size_t total = (size_t)M * F;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    size_t m = e / F;
-    int f = (int)(e % F);
-    size_t base = m * 2 * F + (size_t)(f / GU_BLOCK) * 2 * GU_BLOCK + f % GU_BLOCK;
-    float g = gu[base], u = gu[base + GU_BLOCK];
-    st(act, e, g / (1.0f + expf(-g)) * u);
-  }
-}
-
-template <typename T>
 __global__ void k_cache_gather(KVView v, const int32_t *pos, int n_pos, int l0, int nl, int G,
                                int dh, float *k_out, float *v_out) {
   size_t total = (size_t)n_pos * nl * G * dh;
@@ -641,15 +628,6 @@ void launch_rope_scatter(const float *qkv, const float2 *rope, const int32_t *po
     go((__nv_bfloat16 *)nullptr);
   else
     go((float *)nullptr);
-}
-
-void launch_swiglu(const float *gu, int M, int F, void *act, int dtype, cudaStream_t s) {
-  if (M <= 0) return;
-  size_t n = (size_t)M * F;
-  if (dtype == KVR_DTYPE_BF16)
-    k_swiglu<<<grid_for(n, 256), 256, 0, s>>>(gu, M, F, (__nv_bfloat16 *)act);
-  else
-    k_swiglu<<<grid_for(n, 256), 256, 0, s>>>(gu, M, F, (float *)act);
 }
 
 void launch_cache_gather(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,

@@ -16,7 +16,7 @@
 //            a block table maps logical page -> physical page.
 //   activations (per model workspace, max_rows R): residual h fp32 [R][d],
 //            normed rows a [R][d], qkv fp32 [R][Nqkv], q fp32 [R][H*dh],
-//            attention output [R][H*dh], gate/up fp32 [R][2F], act [R][F].
+//            attention output [R][H*dh], act [R][F].
 #pragma once
 
 #include <cuda.h>
@@ -237,7 +237,7 @@ struct kvr_model {
   void *ws_block = nullptr;
   int32_t *pos_d = nullptr;  // [R] positions of the rows of a pass
   int32_t *rowdoc_d = nullptr;  // [R] batch: document of each row
-  float *h = nullptr, *qkv = nullptr, *q = nullptr, *gu = nullptr, *logits = nullptr;
+  float *h = nullptr, *qkv = nullptr, *q = nullptr, *logits = nullptr;
   void *qb = nullptr;  // bf16 post-RoPE q for the tensor-core attention
   void *a = nullptr, *attn = nullptr, *act = nullptr;
   float *scores = nullptr;     // [max_ctx + reserve] selector scores
@@ -471,7 +471,6 @@ void launch_rope_scatter(const float *qkv, const float2 *rope, const int32_t *po
                          const Dims &dm, int layer, const KVView *views, const int32_t *rowdoc,
                          KVView single, float *q_out, void *qb_out, float qscale, bool write_kv,
                          cudaStream_t s, const SplitView *sv = nullptr, void *rows_out = nullptr);
-void launch_swiglu(const float *gu, int M, int F, void *act, int dtype, cudaStream_t s);
 void launch_cache_gather(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
                          int G, int dh, float *k_out, float *v_out, cudaStream_t s);
 // The same gather in the cache's element type (no widening).
@@ -498,7 +497,9 @@ struct GemmArgs {
   int dtype;       // operands: KVR_DTYPE_F32 or KVR_DTYPE_BF16
   int accumulate;  // 1: Y += result
 };
-void launch_gemm_simt(const GemmArgs &g, cudaStream_t s);
+// FFMA GEMM; act (optional): W's rows are interleaved gate/up and the SwiGLU of
+// their products goes to act [M][N / 2] in the model dtype instead of Y.
+void launch_gemm_simt(const GemmArgs &g, void *act, int num_sms, cudaStream_t s);
 
 // Tensor-core GEMM (bf16, N % 128 == 0, K % 64 == 0).  Epilogues:
 enum { GEMM_EPI_STORE = 0, GEMM_EPI_ACCUM = 1, GEMM_EPI_SWIGLU = 2 };
@@ -558,9 +559,9 @@ const char *launch_gemm_tc(const GemmArgs &g, const CUtensorMap &tmW, int epi, v
 
 // ---- kernels: attention ----
 // o[i] = softmax(q_i K[0..pos_i]^T / sqrt(dh)) V[0..pos_i] for every row i,
-// GQA head h -> kv head h / (H/G).  q fp32 [M][H*dh]; out [M][H*dh] in dtype.
+// GQA head h -> kv head h / (H/G).  fp32 model; q, out [M][H*dh].
 void launch_attention_simt(const float *q, const int32_t *pos, int M, const Dims &dm, int layer,
-                           const KVView *views, const int32_t *rowdoc, KVView single, void *out,
+                           const KVView *views, const int32_t *rowdoc, KVView single, float *out,
                            cudaStream_t s);
 
 // Tensor-core attention (bf16 cache, head_dim 64 or 128).  blocks: device
