@@ -222,21 +222,26 @@ int pair_splits(const kvr_model *m, const std::vector<int> &pages, int &cost) {
 // With the two-tile kernel the blocks are its tiles, and a table of pairs of
 // one document's tiles follows them, longest key range first (the last wave
 // then holds the shortest CTAs).
-kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32_t *rowdoc) {
-  r.tc5 = false;
-  r.pairs = nullptr;
-  r.n_pairs = 0;
-  if (!use_tc_attention(m) || r.M <= 0) return KVR_OK;
+// force_splits > 0: that split count, one tile per CTA.
+struct AttnPlan {
+  std::vector<int32_t> b;                     // blocks: (row0, nrows, kmax, doc)
+  std::vector<std::array<int32_t, 4>> pairs;  // (first tile, tiles, kmax, doc)
+  int nb = 0, splits = 1, max_rows = 0;
+  bool tc5 = false;
+};
+AttnPlan make_plan(const kvr_model *m, const Rows &r, const int32_t *pos, const int32_t *rowdoc,
+                   int force_splits = 0) {
   const Dims &dm = m->dims;
+  AttnPlan p;
   const int grp = dm.H / dm.G;
   // the tcgen05 kernels (query blocks of up to 128 query vectors) when every
   // document has a TMA view of its pages, else the mma.sync kernel
-  r.tc5 = m->use_tc5 && (rowdoc ? r.tmaps != nullptr : r.tm_kv != nullptr) &&
+  p.tc5 = m->use_tc5 && (rowdoc ? r.tmaps != nullptr : r.tm_kv != nullptr) &&
           attn_tc5_rows_per_block(grp) > 0;
-  const int qb = r.tc5 ? attn_tc5_rows_per_block(grp) : attn_tc_rows_per_block(grp);
-  std::vector<int32_t> b;
-  std::vector<std::array<int32_t, 4>> pairs;  // (first tile, tiles, kmax, doc)
-  int max_chunks = 0, max_rows = 0;
+  const int qb = p.tc5 ? attn_tc5_rows_per_block(grp) : attn_tc_rows_per_block(grp);
+  std::vector<int32_t> &b = p.b;
+  auto &pairs = p.pairs;
+  int max_chunks = 0, &max_rows = p.max_rows;
   // a document's rows in equal blocks of at most qb rows (`pair`: in whole pairs)
   auto cut = [&](bool pair) {
     b.clear();
@@ -265,8 +270,8 @@ kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32
     return (int)b.size() / 4;
   };
   auto one_wave = [&](int nb) {
-    const int target = m->num_sms * (r.tc5 ? attn_tc5_ctas_per_sm(dm.dh) : 1), ctas = nb * dm.G;
-    const int s = r.tc5 ? std::max(1, target / ctas)  // one wave: no straggler CTAs
+    const int target = m->num_sms * (p.tc5 ? attn_tc5_ctas_per_sm(dm.dh) : 1), ctas = nb * dm.G;
+    const int s = p.tc5 ? std::max(1, target / ctas)  // one wave: no straggler CTAs
                         : std::max(1, (target + ctas - 1) / ctas);
     return std::min(std::min(s, max_chunks), 64);  // the combine merges <= 64 splits
   };
@@ -274,8 +279,10 @@ kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32
   // half as many and twice as long: it is taken where the model says that its
   // launch ends first (never with one or two tiles, whose CTAs it would
   // leave alone on their SMs).
-  int nb = cut(false), splits = one_wave(nb);
-  if (r.tc5 && r.M > 2 * qb) {
+  int &nb = p.nb, &splits = p.splits;
+  nb = cut(false);
+  splits = force_splits ? force_splits : one_wave(nb);
+  if (p.tc5 && r.M > 2 * qb && !force_splits) {
     std::vector<int> pages;
     for (int t = 0; t < nb; ++t) pages.push_back(b[4 * t + 2] / KVR_PAGE + 1);
     const int tile_cost = attn_cost(COST_TILE, pages, dm.G, splits, m->num_sms);
@@ -292,22 +299,33 @@ kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32
       nb = cut(false);
     }
   }
-  if (nb > m->max_blocks) return fail(KVR_E_UNSUPPORTED, "too many attention blocks (%d)", nb);
   while (splits > 1 && attn_tc_ws_floats(splits, nb, dm.G, dm.dh) > m->attn_ws_floats) --splits;
-  if (!pairs.empty()) {
-    // split ranges come from the pair's last key: the combine takes it from the tiles
-    if (splits > 1)
-      for (const auto &x : pairs)
-        for (int t = 0; t < x[1]; ++t) b[4 * (x[0] + t) + 2] = x[2];
-    for (const auto &x : pairs) b.insert(b.end(), x.begin(), x.end());
-    r.pairs = m->blocks_d + nb;
-    r.n_pairs = (int)pairs.size();
+  // split ranges come from the pair's last key: the combine takes it from the tiles
+  if (splits > 1)
+    for (const auto &x : pairs)
+      for (int t = 0; t < x[1]; ++t) b[4 * (x[0] + t) + 2] = x[2];
+  return p;
+}
+
+kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32_t *rowdoc,
+                          int force_splits = 0) {
+  r.tc5 = false;
+  r.pairs = nullptr;
+  r.n_pairs = 0;
+  if (!use_tc_attention(m) || r.M <= 0) return KVR_OK;
+  AttnPlan p = make_plan(m, r, pos, rowdoc, force_splits);
+  if (p.nb > m->max_blocks) return fail(KVR_E_UNSUPPORTED, "too many attention blocks (%d)", p.nb);
+  if (!p.pairs.empty()) {
+    for (const auto &x : p.pairs) p.b.insert(p.b.end(), x.begin(), x.end());
+    r.pairs = m->blocks_d + p.nb;
+    r.n_pairs = (int)p.pairs.size();
   }
-  KVR_TRY(stage_h2d(m, (int32_t *)m->blocks_d, b.data(), b.size()));
+  KVR_TRY(stage_h2d(m, (int32_t *)m->blocks_d, p.b.data(), p.b.size()));
+  r.tc5 = p.tc5;
   r.blocks = m->blocks_d;
-  r.n_blocks = nb;
-  r.n_splits = splits;
-  r.max_block_rows = max_rows;
+  r.n_blocks = p.nb;
+  r.n_splits = p.splits;
+  r.max_block_rows = p.max_rows;
   return KVR_OK;
 }
 
@@ -1152,10 +1170,13 @@ static kvr_status check_context(const kvr_model *m, const int32_t *tokens, int32
   return KVR_OK;
 }
 
-// A new cache of n positions holding `tokens`: zeroed pages (slots never
-// written hold finite values, so a masked key meets probability 0 and never
-// 0 * NaN), the identity block table, the device copy of the tokens and, for
-// bf16, the TMA view of the page pool.  Enqueued on the model's stream.
+// A new cache of n positions holding `tokens`: pages whose slots are zero
+// unless they are written before they are first read (slots never written
+// hold finite values, so a masked key meets probability 0 and never 0 * NaN),
+// the identity block table, the device copy of the tokens and, for bf16, the
+// TMA view of the page pool.  Behind the table's pages the pool holds
+// KVR_SPARE_PAGES more, for a second continuation past n (kvr_margin).
+// Enqueued on the model's stream.
 static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_cache **out) {
   const Dims &dm = m->dims;
   kvr_cache *c = new kvr_cache();
@@ -1165,7 +1186,8 @@ static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_
   c->cap = (n + KVR_QUERY_RESERVE + KVR_PAGE - 1) / KVR_PAGE * KVR_PAGE;
   c->n_pages = c->cap / KVR_PAGE;
   size_t page_bytes = dm.page_elems() * dm.es();
-  c->pages = dev_alloc((size_t)c->n_pages * page_bytes);
+  const int pool_pages = c->n_pages + KVR_SPARE_PAGES;
+  c->pages = dev_alloc((size_t)pool_pages * page_bytes);
   c->table = (int32_t *)dev_alloc((size_t)c->n_pages * 4);
   c->tokens_d = (int32_t *)dev_alloc((size_t)c->cap * 4);
   if (!c->pages || !c->table || !c->tokens_d) {
@@ -1173,12 +1195,17 @@ static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_
     return fail(KVR_E_NOMEM, "cache of %d pages", c->n_pages);
   }
   c->tokens_h.assign(tokens, tokens + n);
-  if (cudaMemsetAsync(c->pages, 0, (size_t)c->n_pages * page_bytes, m->stream)) {
+  // The caller writes every position below n, a prefill in chunks of max_rows,
+  // each chunk before its attention: with whole pages per chunk only the pages
+  // from n on hold slots that are read unwritten.
+  const int clean = dm.max_rows % KVR_PAGE == 0 ? n / KVR_PAGE : 0;
+  if (cudaMemsetAsync((char *)c->pages + (size_t)clean * page_bytes, 0,
+                      (size_t)(pool_pages - clean) * page_bytes, m->stream)) {
     kvr_cache_free(c);
     return fail(KVR_E_CUDA, "cache clear");
   }
   if (dm.dtype == KVR_DTYPE_BF16) {
-    const long long rows = (long long)c->n_pages * dm.L * 2 * dm.G * KVR_PAGE;
+    const long long rows = (long long)pool_pages * dm.L * 2 * dm.G * KVR_PAGE;
     c->tm_kv_ok = rows < (1ll << 31) && make_tmap_bf16(&c->tm_kv, c->pages, (int)rows, dm.dh, KVR_PAGE);
   }
   std::vector<int32_t> tab(c->n_pages);
@@ -1736,22 +1763,69 @@ kvr_status kvr_transplant(kvr_cache *dst, const kvr_cache *src, const int32_t *p
   return st;
 }
 
-kvr_status kvr_answer_logprob(kvr_model *m, const kvr_cache *c, const int32_t *prompt,
-                              int32_t mp, const int32_t *answer, int32_t ma, double *out) {
-  if (!m || !c || !prompt || !answer || !out) return fail(KVR_E_INVAL, "NULL argument");
+// Arguments of one answer's log-probability; feed: prompt and answer, the
+// answer one token behind.
+static kvr_status check_answer(const kvr_model *m, const kvr_cache *c, const int32_t *prompt,
+                               int32_t mp, const int32_t *answer, int32_t ma,
+                               std::vector<int32_t> &feed) {
+  if (!m || !c || !prompt || !answer) return fail(KVR_E_INVAL, "NULL argument");
   if (c->model != m) return fail(KVR_E_INVAL, "cache of another model");
   if (c->poisoned) return fail(KVR_E_POISONED, "cache poisoned");
   const Dims &dm = m->dims;
-  int rows = mp + ma - 1;
+  const int rows = mp + ma - 1;
   if (mp < 1 || ma < 1 || rows > KVR_QUERY_RESERVE || c->n + rows > c->cap)
     return fail(KVR_E_RANGE, "prompt + answer - 1 must be in [1, %d]", KVR_QUERY_RESERVE);
-  std::vector<int32_t> feed(prompt, prompt + mp);
+  feed.assign(prompt, prompt + mp);
   feed.insert(feed.end(), answer, answer + ma - 1);
   for (int t : feed)
     if (t < 0 || t >= dm.V) return fail(KVR_E_RANGE, "token out of range");
   for (int i = 0; i < ma; ++i)
     if (answer[i] < 0 || answer[i] >= dm.V) return fail(KVR_E_RANGE, "answer token out of range");
+  return KVR_OK;
+}
+
+// The length-averaged log-probabilities of n_ans answers after a pass that
+// left answer k's rows in h from row first[k] on: final norm, lm_head, one
+// log-softmax per row.  Synchronises the stream.
+static kvr_status answers_logprob(kvr_model *m, int n_ans, const int *first,
+                                  const int32_t *const *answer, const int32_t *ma, double *out) {
+  const Dims &dm = m->dims;
+  std::vector<int32_t> target;
+  for (int k = 0; k < n_ans; ++k) {
+    Prof pr(m, P_NORM, (int64_t)ma[k] * dm.d * 4);
+    launch_rmsnorm(m->h, m->final_norm, first[k], ma[k], dm.d, dm.eps,
+                   (char *)m->a + target.size() * dm.d * dm.es(), dm.dtype, m->stream,
+                   &m->pending);
+    KVR_TRY(launch_check(m, 1));
+    target.insert(target.end(), answer[k], answer[k] + ma[k]);
+  }
+  m->pending = SplitView{};
+  const int rows = (int)target.size();
+  KVR_TRY(gemm(m, P_LMHEAD, m->a, m->lm_head, m->tc_lm ? &m->tm_lm : nullptr, nullptr, m->logits,
+               rows, dm.V, dm.d, GEMM_EPI_STORE));
+  // answer ids go to the row-document slot
+  KVR_TRY(stage_h2d(m, m->rowdoc_d, target.data(), rows));
+  float *lp = m->scores;  // [rows] scratch
+  launch_row_logprob(m->logits, rows, dm.V, m->rowdoc_d, lp, m->stream);
+  KVR_TRY(launch_check(m, 1));
+  std::vector<float> h(rows);
+  CUDA_TRY(cudaMemcpyAsync(h.data(), lp, (size_t)rows * 4, cudaMemcpyDeviceToHost, m->stream));
+  KVR_TRY(sync_model(m));
+  for (int k = 0, i = 0; k < n_ans; ++k) {
+    double acc = 0.0;
+    for (int j = 0; j < ma[k]; ++j) acc += h[i++];
+    out[k] = acc / ma[k];
+  }
+  return KVR_OK;
+}
+
+kvr_status kvr_answer_logprob(kvr_model *m, const kvr_cache *c, const int32_t *prompt,
+                              int32_t mp, const int32_t *answer, int32_t ma, double *out) {
+  if (!out) return fail(KVR_E_INVAL, "NULL argument");
+  std::vector<int32_t> feed;
+  KVR_TRY(check_answer(m, c, prompt, mp, answer, ma, feed));
   KVR_TRY(use_device(m));
+  const int rows = (int)feed.size();
   std::vector<int32_t> P(rows);
   for (int i = 0; i < rows; ++i) P[i] = c->n + i;
   KVR_TRY(stage_h2d(m, c->tokens_d + c->n, feed.data(), rows));
@@ -1765,38 +1839,122 @@ kvr_status kvr_answer_logprob(kvr_model *m, const kvr_cache *c, const int32_t *p
   r.max_pos = c->n + rows - 1;
   KVR_TRY(plan_attention(m, r, P.data(), nullptr));
   KVR_TRY(run_pass(m, r, false));
-  // rows mp-1 .. mp+ma-2 predict answer[0..ma-1]
-  {
-    Prof pr(m, P_NORM, (int64_t)ma * dm.d * 4);
-    launch_rmsnorm(m->h, m->final_norm, mp - 1, ma, dm.d, dm.eps, m->a, dm.dtype, m->stream,
-                   &m->pending);
-    m->pending = SplitView{};
-    KVR_TRY(launch_check(m, 1));
+  const int first = mp - 1;  // rows mp-1 .. mp+ma-2 predict answer[0..ma-1]
+  return answers_logprob(m, 1, &first, &answer, &ma, out);
+}
+
+// Whether the two answers of a margin give the same bits in one pass as in one
+// each, and in how many key splits (0: no): every projection on the
+// tensor-core GEMM, whose split of K does not depend on the row count (gate/up
+// too where the passes differ in cluster split-K), and the same attention plan
+// for either answer's rows alone.
+static int margin_splits(const kvr_model *m, const kvr_cache *c, size_t rows0, size_t rows1) {
+  const Dims &dm = m->dims;
+  if (!use_tc_attention(m) || !m->use_tc || !m->tc_lm || !c->tm_kv_ok) return 0;
+  for (const LayerW &w : m->layers)
+    if (!w.tc_qkv || !w.tc_o || !w.tc_gu || !w.tc_d) return 0;
+  if (rows0 + rows1 > 64 && 2 * (2 * dm.F / 128) <= m->num_sms) return 0;
+  int splits[2];
+  const size_t rows[2] = {rows0, rows1};
+  for (int k = 0; k < 2; ++k) {
+    std::vector<int32_t> P(rows[k]);
+    for (size_t i = 0; i < rows[k]; ++i) P[i] = c->n + (int)i;
+    Rows r;
+    r.M = (int)rows[k];
+    r.tm_kv = &c->tm_kv;
+    const AttnPlan p = make_plan(m, r, P.data(), nullptr);
+    if (!p.tc5 || !p.pairs.empty() ||
+        attn_tc_ws_floats(p.splits, 2 * p.nb, dm.G, dm.dh) > m->attn_ws_floats)
+      return 0;
+    splits[k] = p.splits;
   }
-  KVR_TRY(gemm(m, P_LMHEAD, m->a, m->lm_head, m->tc_lm ? &m->tm_lm : nullptr, nullptr, m->logits,
-               ma, dm.V, dm.d, GEMM_EPI_STORE));
-  // answer ids staged behind the positions in the row-document slot
-  KVR_TRY(stage_h2d(m, m->rowdoc_d, answer, ma));
-  float *lp = m->scores;  // [ma] scratch
-  launch_row_logprob(m->logits, ma, dm.V, m->rowdoc_d, lp, m->stream);
-  KVR_TRY(launch_check(m, 1));
-  std::vector<float> h(ma);
-  CUDA_TRY(cudaMemcpyAsync(h.data(), lp, (size_t)ma * 4, cudaMemcpyDeviceToHost, m->stream));
-  KVR_TRY(sync_model(m));
-  double acc = 0.0;
-  for (int i = 0; i < ma; ++i) acc += h[i];
-  *out = acc / ma;
-  return KVR_OK;
+  return splits[0] == splits[1] ? splits[0] : 0;
+}
+
+// Both answers in one pass, as two documents that share every page below n: the
+// second one's table ends in the cache's spare pages (the first of them a
+// copy of the page that n falls into), so that its rows' K/V past n have a
+// place of their own.  The pass streams the weights and lm_head once for both
+// (two 29-row answers on four 8B-shape layers: 1.25 -> 0.71 ms).
+static kvr_status margin_one_pass(kvr_model *m, const kvr_cache *c,
+                                  const std::vector<int32_t> (&feed)[2], int32_t mp,
+                                  const int32_t *const *answer, const int32_t *ma, int splits,
+                                  double *lp) {
+  const Dims &dm = m->dims;
+  auto al = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t tab_b = al((size_t)c->n_pages * 4), tok_b = al((size_t)c->cap * 4);
+  const size_t mb = al(2 * sizeof(CUtensorMap));
+  const size_t vb = al(2 * sizeof(KVView)), pb = al(2 * sizeof(void *));
+  // scratch: tensor maps, views, token pointers, the second document's table,
+  // its tokens (those from n on are read)
+  const size_t head = mb + vb + pb + tab_b;
+  KVR_TRY(grow_scratch(m, m->batch_scratch, m->batch_scratch_bytes, head + tok_b, "margin tables"));
+  char *dev = (char *)m->batch_scratch;
+  int32_t *table1 = (int32_t *)(dev + mb + vb + pb), *tokens1 = (int32_t *)(dev + head);
+  std::vector<int32_t> host(head / 4);
+  char *hb = (char *)host.data();
+  KVView views[2] = {c->view(), c->view()};
+  views[1].table = table1;
+  const int32_t *tokens[2] = {c->tokens_d, tokens1};
+  for (int k = 0; k < 2; ++k) memcpy(hb + k * sizeof(CUtensorMap), &c->tm_kv, sizeof c->tm_kv);
+  memcpy(hb + mb, views, sizeof views);
+  memcpy(hb + mb + vb, tokens, sizeof tokens);
+  const int tail = c->n / KVR_PAGE;  // the page that position n falls into
+  for (int i = 0; i < c->n_pages; ++i)
+    ((int32_t *)(hb + mb + vb + pb))[i] = i < tail ? i : c->n_pages + i - tail;
+  KVR_TRY(stage_h2d(m, (int32_t *)dev, host.data(), host.size()));
+  const size_t page_b = dm.page_elems() * dm.es();
+  if (c->n % KVR_PAGE)
+    CUDA_TRY(cudaMemcpyAsync((char *)c->pages + c->n_pages * page_b,
+                             (char *)c->pages + tail * page_b, page_b, cudaMemcpyDeviceToDevice,
+                             m->stream));
+  std::vector<int32_t> P, doc;
+  for (int k = 0; k < 2; ++k) {
+    KVR_TRY(stage_h2d(m, (int32_t *)tokens[k] + c->n, feed[k].data(), feed[k].size()));
+    for (size_t i = 0; i < feed[k].size(); ++i) {
+      P.push_back(c->n + (int)i);
+      doc.push_back(k);
+    }
+  }
+  KVR_TRY(stage_h2d(m, m->pos_d, P.data(), P.size()));
+  KVR_TRY(stage_h2d(m, m->rowdoc_d, doc.data(), doc.size()));
+  Rows r;
+  r.M = (int)P.size();
+  r.pos = m->pos_d;
+  r.rowdoc = m->rowdoc_d;
+  r.views = (const KVView *)(dev + mb);
+  r.doc_tokens = (const int32_t *const *)(dev + mb + vb);
+  r.tmaps = (const CUtensorMap *)dev;
+  r.max_pos = c->n + (int)std::max(feed[0].size(), feed[1].size()) - 1;
+  KVR_TRY(plan_attention(m, r, P.data(), doc.data(), splits));
+  KVR_TRY(run_pass(m, r, false));
+  const int first[2] = {mp - 1, (int)feed[0].size() + mp - 1};
+  return answers_logprob(m, 2, first, answer, ma, lp);
 }
 
 kvr_status kvr_margin(kvr_model *m, const kvr_cache *c, const int32_t *prompt, int32_t mp,
                       const int32_t *a_new, int32_t m_new, const int32_t *a_old, int32_t m_old,
                       double *margin_out) {
   if (!margin_out) return fail(KVR_E_INVAL, "NULL argument");
-  double lp_new = 0.0, lp_old = 0.0;
-  KVR_TRY(kvr_answer_logprob(m, c, prompt, mp, a_new, m_new, &lp_new));
-  KVR_TRY(kvr_answer_logprob(m, c, prompt, mp, a_old, m_old, &lp_old));
-  *margin_out = lp_new - lp_old;
+  std::vector<int32_t> feed[2];
+  KVR_TRY(check_answer(m, c, prompt, mp, a_new, m_new, feed[0]));
+  KVR_TRY(check_answer(m, c, prompt, mp, a_old, m_old, feed[1]));
+  KVR_TRY(use_device(m));
+  double lp[2] = {0.0, 0.0};
+  // one pass where its rows fit the pass and the answers' rows the logits
+  const int splits = (int)(feed[0].size() + feed[1].size()) <= m->dims.max_rows &&
+                             m_new + m_old <= KVR_QUERY_RESERVE
+                         ? margin_splits(m, c, feed[0].size(), feed[1].size())
+                         : 0;
+  if (splits) {
+    const int32_t *answer[2] = {a_new, a_old};
+    const int32_t ma[2] = {m_new, m_old};
+    KVR_TRY(margin_one_pass(m, c, feed, mp, answer, ma, splits, lp));
+  } else {
+    KVR_TRY(kvr_answer_logprob(m, c, prompt, mp, a_new, m_new, &lp[0]));
+    KVR_TRY(kvr_answer_logprob(m, c, prompt, mp, a_old, m_old, &lp[1]));
+  }
+  *margin_out = lp[0] - lp[1];
   return KVR_OK;
 }
 

@@ -34,6 +34,7 @@ namespace kvr {
 constexpr int KVR_PAGE = 64;          // positions per KV page
 constexpr int KVR_RD_GROUPS = 8;      // layer groups of kvr_repair_read's overlapped copies
 constexpr int KVR_QUERY_RESERVE = 64; // positions past n reserved for fresh queries
+constexpr int KVR_SPARE_PAGES = 2;    // pages for a second continuation past n (reserve and n's page)
 constexpr int GU_BLOCK = 16;          // gate/up interleave block (rows)
 
 struct Dims {
