@@ -1003,14 +1003,14 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
     size_t sz[] = {R * 4,          R * 4,          R * d * 4,        R * d * es,  R * Nq * 4,
                    R * HD * 4,     R * HD * es,    R * F * es,
                    (size_t)KVR_QUERY_RESERVE * V * 4,
-                   P * 4,          P * 8,          P * 4,            256,         R * HD * 2};
+                   P * 4,          P * 8,          256,         R * HD * 2};
     size_t tot = 0;
     for (size_t x : sz) tot += al(x);
     m->ws_block = dev_alloc(tot);
     if (!m->ws_block) return bail(fail(KVR_E_NOMEM, "workspace: %zu bytes", tot));
     char *p = (char *)m->ws_block;
-    void *ptrs[14];
-    for (int i = 0; i < 14; ++i) {
+    void *ptrs[13];
+    for (int i = 0; i < 13; ++i) {
       ptrs[i] = p;
       p += al(sz[i]);
     }
@@ -1025,9 +1025,8 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
     m->logits = (float *)ptrs[8];
     m->scores = (float *)ptrs[9];
     m->keys = (unsigned long long *)ptrs[10];
-    m->sel_out = (int32_t *)ptrs[11];
-    m->sel_count = (int32_t *)ptrs[12];
-    m->qb = ptrs[13];
+    m->sel_count = (int32_t *)ptrs[11];
+    m->qb = ptrs[12];
     m->dev_flag = (int *)dev_alloc(256);
     if (!m->dev_flag) return bail(fail(KVR_E_NOMEM, "flag"));
     cudaMemset(m->dev_flag, 0, 256);
@@ -1557,10 +1556,12 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
   int n = c->n, s_end = edit_start + edit_len;
   *count_out = 0;
   if (n - s_end <= 0 || K == 0) return KVR_OK;
-  // scratch: the edited context, then (Attention, CacheBlend) the stale rows
-  // the read-only passes overwrite and the span queries' probabilities
+  // scratch (Attention, CacheBlend): the edited context, the stale rows the
+  // read-only passes overwrite, the span queries and their probabilities.  The
+  // other policies read at most the pool's tokens, which the edit leaves alone.
+  const bool runs_model = policy == KVR_POLICY_ATTENTION || policy == KVR_POLICY_CACHEBLEND;
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-  const size_t tok_b = al((size_t)c->cap * 4);
+  const size_t tok_b = runs_model ? al((size_t)c->cap * 4) : 0;
   size_t save_b = 0, prob_b = 0;
   if (policy == KVR_POLICY_ATTENTION) {
     save_b = al((size_t)edit_len * dm.L * 2 * dm.G * dm.dh * dm.es());
@@ -1572,11 +1573,13 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
   KVR_TRY(grow_scratch(m, m->sel_scratch, m->sel_scratch_bytes, tok_b + save_b + prob_b,
                        "selector scratch"));
   char *scr = (char *)m->sel_scratch;
-  int32_t *toks = (int32_t *)scr;
+  int32_t *toks = runs_model ? (int32_t *)scr : c->tokens_d;
   kvr_status st = KVR_OK;
-  if (cudaMemcpyAsync(toks, c->tokens_d, (size_t)n * 4, cudaMemcpyDeviceToDevice, m->stream))
-    st = fail(KVR_E_CUDA, "token copy");
-  if (!st && edit_len) st = stage_h2d(m, toks + edit_start, new_tokens, edit_len);
+  if (runs_model) {
+    if (cudaMemcpyAsync(toks, c->tokens_d, (size_t)n * 4, cudaMemcpyDeviceToDevice, m->stream))
+      st = fail(KVR_E_CUDA, "token copy");
+    if (!st && edit_len) st = stage_h2d(m, toks + edit_start, new_tokens, edit_len);
+  }
   int topk_k = K;
   SimpleKeys gen;  // simple policies: keys made inside the top-K kernel
   void *save = nullptr;
@@ -1710,29 +1713,25 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
   }
   if (!st) {
     Prof pr(m, P_SELECT, 0);
-    // sel_out: [count][device flag][positions ...], read back in one copy
-    const char *e = launch_topk(m->keys, n, s_end, topk_k, m->sel_out + 2, m->sel_out,
-                                m->stream, gen, m->dev_flag, m->sel_out + 1);
+    // The kernel writes the count, the device flag and the positions straight
+    // into page-locked host memory: a copy behind it took 3 us of a selection.
+    const char *e = launch_topk(m->keys, n, s_end, topk_k, m->rb_h + 2, m->rb_h, m->stream, gen,
+                                m->dev_flag, m->rb_h + 1);
     st = e ? fail(KVR_E_CUDA, "top-K over %d candidates: %s", n - s_end, e) : launch_check(m, 1);
   }
-  // one readback: the count, the device error flag and up to K positions
   int32_t cnt = 0;
+  const cudaError_t e = cudaStreamSynchronize(m->stream);
   if (!st) {
-    const int kmax = std::min(K, n - s_end);
-    int32_t *rb = m->rb_h;
-    cudaError_t e = cudaMemcpyAsync(rb, m->sel_out, (size_t)(kmax + 2) * 4,
-                                    cudaMemcpyDeviceToHost, m->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+    const int32_t *rb = m->rb_h;
     if (e != cudaSuccess) {
-      st = fail(KVR_E_CUDA, "select readback: %s", cudaGetErrorString(e));
+      st = fail(KVR_E_CUDA, "select: %s", cudaGetErrorString(e));
     } else if (rb[1]) {
       st = sync_model(m);  // reports the bounded wait that ran out and clears the flag
     } else {
-      cnt = std::min(rb[0], kmax);
+      cnt = std::min(rb[0], std::min(K, n - s_end));
       std::copy(rb + 2, rb + 2 + cnt, positions_out);
     }
   }
-  cudaStreamSynchronize(m->stream);
   if (!st) *count_out = cnt;
   return st;
 }
@@ -2003,8 +2002,10 @@ kvr_status cache_read(const kvr_cache *c, const int32_t *positions, int32_t n_po
   if (!st && (cudaMemcpyAsync(k_out, kd, elems * eb, cudaMemcpyDeviceToHost, m->stream) ||
               cudaMemcpyAsync(v_out, vd, elems * eb, cudaMemcpyDeviceToHost, m->stream)))
     st = fail(KVR_E_CUDA, "readback");
-  if (!st) st = sync_model(m);
-  cudaStreamSynchronize(m->stream);
+  if (!st)
+    st = sync_model(m);
+  else
+    cudaStreamSynchronize(m->stream);
   return st;
 }
 

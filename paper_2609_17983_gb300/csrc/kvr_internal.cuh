@@ -243,8 +243,7 @@ struct kvr_model {
   void *a = nullptr, *attn = nullptr, *act = nullptr;
   float *scores = nullptr;     // [max_ctx + reserve] selector scores
   unsigned long long *keys = nullptr;  // [max_ctx + reserve] top-K keys
-  int32_t *sel_out = nullptr;  // [max_ctx] selected positions
-  int32_t *sel_count = nullptr;
+  int32_t *sel_count = nullptr;  // EditLocal@boundary's bound at [1]
   void *read_scratch = nullptr;  // cache readback: positions, then the gathered K and V
   size_t read_scratch_bytes = 0;
   // kvr_repair_read: the pass's K/V rows as RoPE writes them, copied to the
@@ -272,7 +271,7 @@ struct kvr_model {
   size_t stage_cap = 0;
   size_t stage_off = 0;           // next free slot (copies take consecutive slots)
   cudaEvent_t stage_ev = nullptr;  // recorded after the last staged copy
-  int32_t *rb_h = nullptr;         // pinned readback: selector count, flag, positions
+  int32_t *rb_h = nullptr;         // pinned: selector count, flag, positions (written by the top-K)
   int32_t *flag_h = nullptr;       // pinned readback of the device error flag
   // profiling
   bool prof = false;
