@@ -131,21 +131,23 @@ kvr_status stage_h2d(kvr_model *m, int32_t *dst_dev, const int32_t *src, size_t 
 // descriptor, else the FFMA kernel.  epi selects the epilogue (SwiGLU goes to
 // m->act).
 // defer: split tiles of the tensor-core GEMM are left to the kernel that
-// next reads Y, which must take *defer (ws null when Y is complete).
+// next reads Y, which must take *defer (ws null when Y is complete).  ldy: row
+// stride of Y (0: N).
 kvr_status gemm(kvr_model *m, int cls, const void *X, const void *W, const CUtensorMap *tm,
                 const float *bias, float *Y, int M, int N, int K, int epi,
-                SplitView *defer = nullptr) {
+                SplitView *defer = nullptr, int ldy = 0) {
   const Dims &dm = m->dims;
   Prof pr(m, cls, (int64_t)N * K * (int64_t)dm.es());
   if (defer) *defer = SplitView{};
+  if (!ldy) ldy = N;
   if (tm && m->use_tc) {
-    GemmArgs g{X, W, bias, Y, M, N, K, K, N, dm.dtype, epi == GEMM_EPI_ACCUM};
+    GemmArgs g{X, W, bias, Y, M, N, K, K, ldy, dm.dtype, epi == GEMM_EPI_ACCUM};
     const char *e = launch_gemm_tc(g, *tm, epi, epi == GEMM_EPI_SWIGLU ? m->act : nullptr,
                                    N / 2, m->tcw, m->stream, m->defer_splits ? defer : nullptr);
     if (e) return fail(KVR_E_CUDA, "tensor-core GEMM (M=%d N=%d K=%d): %s", M, N, K, e);
     return launch_check(m, 1);
   }
-  GemmArgs g{X, W, bias, Y, M, N, K, K, N, dm.dtype, epi == GEMM_EPI_ACCUM};
+  GemmArgs g{X, W, bias, Y, M, N, K, K, ldy, dm.dtype, epi == GEMM_EPI_ACCUM};
   launch_gemm_simt(g, epi == GEMM_EPI_SWIGLU ? m->act : nullptr, m->num_sms, m->stream);
   return launch_check(m, 1);
 }
@@ -172,6 +174,9 @@ struct Rows {
   // [M][L][G][dh]); after every rd_every layers an event marks them ready
   void *rows_out = nullptr;
   int rd_every = 0;
+  // the Attention selector: where RoPE leaves the layer's fp32 queries (else
+  // m->q, and only where the attention reads them)
+  float *q = nullptr;
 };
 
 bool use_tc_attention(const kvr_model *m) {
@@ -347,34 +352,48 @@ kvr_status norm(kvr_model *m, const float *g, int M, int row0 = 0) {
   return launch_check(m, 1);
 }
 
-// QKV projection, RoPE, and (write_kv) the K/V scatter of layer l.  keep_qkv:
-// m->qkv must hold the complete projection afterwards (else split tiles of
-// the GEMM are completed by the RoPE kernel alone).  need_q: the fp32 q
-// (m->q) is read afterwards (attention selector); the tensor-core attention
-// reads only the bf16 q, and the fp32 one is then not written.
 // RoPE of layer l's projection in m->qkv (completed from sv, the QKV GEMM's
-// deferred split tiles), q to m->qb (and m->q when need_q or no tensor-core
-// attention), and (write_kv) the K/V rows into the cache.
-kvr_status rope(kvr_model *m, const Rows &r, int l, bool write_kv, bool need_q,
-                const SplitView &sv) {
+// deferred split tiles), q to m->qb (and in fp32 to r.q, or m->q without
+// tensor-core attention), and (write_kv) the K/V rows into the cache.
+kvr_status rope(kvr_model *m, const Rows &r, int l, bool write_kv, const SplitView &sv) {
   const Dims &dm = m->dims;
   Prof pr(m, P_ROPE, (int64_t)r.M * dm.Nqkv() * 4);
   const bool tc = use_tc_attention(m);
   launch_rope_scatter(m->qkv, m->rope, r.pos, r.M, dm, l, r.views, r.rowdoc, r.single,
-                      tc && !need_q ? nullptr : m->q, tc ? m->qb : nullptr, 1.0f, write_kv,
+                      r.q ? r.q : (tc ? nullptr : m->q), tc ? m->qb : nullptr, 1.0f, write_kv,
                       m->stream, &sv, write_kv ? r.rows_out : nullptr);
   return launch_check(m, 1);
 }
 
-kvr_status layer_qkv(kvr_model *m, const Rows &r, int l, bool write_kv, bool keep_qkv = false,
-                     bool need_q = false) {
+// QKV projection, RoPE, and (write_kv) the K/V scatter of layer l; split tiles of
+// the GEMM are completed by the RoPE kernel alone.
+kvr_status layer_qkv(kvr_model *m, const Rows &r, int l, bool write_kv) {
   const Dims &dm = m->dims;
   const LayerW &w = m->layers[l];
   KVR_TRY(norm(m, w.attn_norm, r.M));
   SplitView sv;
   KVR_TRY(gemm(m, P_GEMM_QKV, m->a, w.wqkv, w.tc_qkv ? &w.tm_qkv : nullptr, w.bqkv, m->qkv, r.M,
-               dm.Nqkv(), dm.d, GEMM_EPI_STORE, keep_qkv ? nullptr : &sv));
-  return rope(m, r, l, write_kv, need_q, sv);
+               dm.Nqkv(), dm.d, GEMM_EPI_STORE, &sv));
+  return rope(m, r, l, write_kv, sv);
+}
+
+// The columns of heads [h0, h1) (q heads, then k, then v) of layer l's QKV
+// projection of the normalised rows into m->qkv.  A tensor-core weight is cut
+// at a 128-feature tile; where the heads do not end on one the whole
+// projection is computed.
+kvr_status project_heads(kvr_model *m, const Rows &r, int l, int h0, int h1, SplitView *defer) {
+  const Dims &dm = m->dims;
+  const LayerW &w = m->layers[l];
+  const int n0 = h0 * dm.dh, n1 = h1 * dm.dh;
+  const char *W = (const char *)w.wqkv + (size_t)n0 * dm.d * dm.es();
+  CUtensorMap tm;
+  const bool cut = !(m->use_tc && w.tc_qkv) ||
+                   (n0 % 128 == 0 && n1 % 128 == 0 && make_tmap_weight(&tm, W, n1 - n0, dm.d));
+  if (!cut)
+    return gemm(m, P_GEMM_QKV, m->a, w.wqkv, &w.tm_qkv, w.bqkv, m->qkv, r.M, dm.Nqkv(), dm.d,
+                GEMM_EPI_STORE, defer);
+  return gemm(m, P_GEMM_QKV, m->a, W, w.tc_qkv ? &tm : nullptr, w.bqkv ? w.bqkv + n0 : nullptr,
+              m->qkv + n0, r.M, n1 - n0, dm.d, GEMM_EPI_STORE, defer, dm.Nqkv());
 }
 
 // Attention of layer l (after its RoPE and K/V write) into m->attn.
@@ -411,7 +430,7 @@ kvr_status attention(kvr_model *m, const Rows &r, int l) {
       if (e) return fail(KVR_E_CUDA, "attention: %s", e);
       KVR_TRY(launch_check(m, r.n_splits > 1 ? 2 : 1));
     } else {
-      launch_attention_simt(m->q, r.pos, r.M, dm, l, r.views, r.rowdoc, r.single,
+      launch_attention_simt(r.q ? r.q : m->q, r.pos, r.M, dm, l, r.views, r.rowdoc, r.single,
                             (float *)m->attn, m->stream);
       KVR_TRY(launch_check(m, 1));
     }
@@ -509,7 +528,7 @@ kvr_status run_pass_chain(kvr_model *m, const Rows &r, bool kv_only) {
   KVR_TRY(run({norm_step(m->layers[0].attn_norm), qkv_step(0)}, &sv));
   for (int l = 0; l < dm.L; ++l) {
     const LayerW &w = m->layers[l];
-    KVR_TRY(rope(m, r, l, true, false, sv));
+    KVR_TRY(rope(m, r, l, true, sv));
     if (kv_only && l + 1 == dm.L) break;
     KVR_TRY(attention(m, r, l));
     std::vector<ChainStep> st = {
@@ -1625,26 +1644,22 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
         r.max_pos = s_end - 1;
         st = plan_attention(m, r, P.data(), nullptr);
         launch_rows_copy(r.single, dm.dtype, r.pos, edit_len, 0, dm.L, save, true, m->stream);
-        launch_fill_f32(m->scores, 0.f, (size_t)n, m->stream);
-        if (!st) st = launch_check(m, 2);
+        if (!st) st = launch_check(m, 1);
         if (!st) st = embed(m, r);
         for (int l = 0; l < dm.L && !st; ++l) {
-          st = layer_qkv(m, r, l, true, false, true);
+          r.q = attn_select_queries(probs, edit_len, dm, n - s_end, l);
+          st = layer_qkv(m, r, l, true);
           if (!st) {
             Prof pr(m, P_SELECT, 0);
-            launch_attn_select_scores(m->q, edit_len, dm, l, r.single, s_end, n, probs, l == 0,
-                                      m->scores, m->stream);
-            st = launch_check(m, 2);
+            const int k = launch_attn_select_scores(edit_len, dm, l, r.single, s_end, n, probs,
+                                                    m->keys, m->stream);
+            st = launch_check(m, k);
           }
           // the scores need the queries of every layer; no K/V follow the last
           if (!st && l + 1 < dm.L) st = layer_rest(m, r, l);
         }
         launch_rows_copy(r.single, dm.dtype, r.pos, edit_len, 0, dm.L, save, false, m->stream);
         if (!st) st = launch_check(m, 1);
-        if (!st) {
-          launch_float_keys(m->scores, n, s_end, m->keys, m->stream);
-          st = launch_check(m, 1);
-        }
       }
     }
   } else if (!st && policy == KVR_POLICY_CACHEBLEND) {
@@ -1688,9 +1703,15 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
         r.max_pos = c0 + M - 1;
         st = plan_attention(m, r, D.data(), nullptr);
         if (!st) st = embed(m, r);
-        if (!st) st = layer_qkv(m, r, 0, false);
+        // the pool rows need layer 0's queries (their K/V stay as cached) and
+        // layer 1's K and V before RoPE (the deviation rotates them)
+        if (!st) st = norm(m, m->layers[0].attn_norm, M);
+        SplitView sv;
+        if (!st) st = project_heads(m, r, 0, 0, dm.H, &sv);
+        if (!st) st = rope(m, r, 0, false, sv);
         if (!st) st = layer_rest(m, r, 0);
-        if (!st) st = layer_qkv(m, r, 1, false, true);
+        if (!st) st = norm(m, m->layers[1].attn_norm, M);
+        if (!st) st = project_heads(m, r, 1, dm.H, dm.H + 2 * dm.G, nullptr);
         if (!st) {
           Prof pr(m, P_SELECT, 0);
           launch_kv_deviation(m->qkv, m->rope, r.pos, M, dm, r.single, m->scores, m->stream);

@@ -187,6 +187,7 @@ struct RopeArgs {
   const float2 *rope;
   const int32_t *pos;
   int M, H, G, dh, layer, L;
+  int heads;  // heads to take: all, or (no K/V written) the query heads alone
   const KVView *views;
   const int32_t *rowdoc;
   KVView single;
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(ROPE_HEADS * 64) k_rope_scatter(const RopeArgs
   pdl_trigger();
   const int half = a.dh >> 1, i = blockIdx.x;
   const int hh = blockIdx.y * ROPE_HEADS + threadIdx.x / half, t = threadIdx.x % half;
-  if (hh >= a.H + 2 * a.G) return;
+  if (hh >= a.heads) return;
   const int n1 = hh * a.dh + t, n2 = n1 + half;
   const int p = a.pos[i];
   float2 cs = make_float2(1.f, 0.f);
@@ -291,9 +292,9 @@ __global__ void __launch_bounds__(ROPE_THREADS) k_rope_rows(const RopeArgs a) {
   TraceScope ts(TK_ROPE);
   pdl_trigger();
   const int half = a.dh >> 1, tph = half >> 2;  // threads per head
-  const int hh = blockIdx.y * (ROPE_THREADS / tph) + threadIdx.x / tph;
+  const int hh = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph;
   const int t = threadIdx.x % tph * 4;
-  if (hh >= a.H + 2 * a.G) return;
+  if (hh >= a.heads) return;
   const int Nqkv = (a.H + 2 * a.G) * a.dh, n1 = hh * a.dh + t, n2 = n1 + half;
   const int r0 = blockIdx.x * RPB, nr = min(RPB, a.M - r0);
   const SplitView &sv = a.sv;
@@ -608,20 +609,21 @@ void launch_rope_scatter(const float *qkv, const float2 *rope, const int32_t *po
                          KVView single, float *q_out, void *qb_out, float qscale, bool write_kv,
                          cudaStream_t s, const SplitView *sv, void *rows_out) {
   if (M <= 0) return;
-  RopeArgs a{qkv,    rope,   pos,   M,      dm.H,
-             dm.G,   dm.dh,  layer, dm.L,   views,
-             rowdoc, single, q_out, (__nv_bfloat16 *)qb_out,
+  const int heads = write_kv ? dm.H + 2 * dm.G : dm.H;
+  RopeArgs a{qkv,   rope,   pos,    M,     dm.H,
+             dm.G,  dm.dh,  layer,  dm.L,  heads,
+             views, rowdoc, single, q_out, (__nv_bfloat16 *)qb_out,
              qscale, write_kv ? 1 : 0, sv ? *sv : SplitView{}, rows_out};
-  const int heads = dm.H + 2 * dm.G;
   auto go = [&](auto *tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
     if (M < ROPE_MANY) {
       launch_pdl(k_rope_scatter<T>, dim3(M, (heads + ROPE_HEADS - 1) / ROPE_HEADS),
                  ROPE_HEADS * dm.dh / 2, 0, s, a);
     } else {
-      const int hpc = ROPE_THREADS / (dm.dh / 8), rpb = a.sv.ws ? 1 : ROPE_RPB;
+      const int tph = dm.dh / 8, threads = std::min(ROPE_THREADS, (heads * tph + 31) / 32 * 32);
+      const int hpc = threads / tph, rpb = a.sv.ws ? 1 : ROPE_RPB;
       launch_pdl(rpb > 1 ? k_rope_rows<T, ROPE_RPB> : k_rope_rows<T, 1>,
-                 dim3((M + rpb - 1) / rpb, (heads + hpc - 1) / hpc), ROPE_THREADS, 0, s, a);
+                 dim3((M + rpb - 1) / rpb, (heads + hpc - 1) / hpc), threads, 0, s, a);
     }
   };
   if (dm.dtype == KVR_DTYPE_BF16)

@@ -242,10 +242,14 @@ __global__ void __launch_bounds__(TOPK_THREADS)
   }
 }
 
-// Attention selector, one layer, in two kernels over a workspace.  The
-// queries of kv group g are the span rows' heads hh with hh / (H/G) == g;
-// within the group a query is ql = r * (H/G) + (hh mod H/G), globally
-// qg = g * S * (H/G) + ql.  A CTA of k_attn_select_logits takes SEL_KC pool
+// Attention selector, a group of layers, in two kernels over a workspace.  The
+// stale pool keys are written by no kernel of the pass and the span's queries
+// of every layer are kept, so the scores of many layers run in one launch,
+// where one layer's fill the chip for a few us and wait out their latencies
+// for twenty.  The queries of kv group g are the span rows' heads hh with
+// hh / (H/G) == g; within the group a query is ql = r * (H/G) + (hh mod H/G),
+// globally qg = g * S * (H/G) + ql.  blockIdx.z is layer-major: query tile
+// z % n_qtiles of layer layer0 + z / n_qtiles, whose arrays lie NQ apart.  A CTA of k_attn_select_logits takes SEL_KC pool
 // keys and SEL_QT queries of one group: the keys are read once into shared
 // memory and serve every query of the tile (so a group's key rows leave L2
 // once per query tile, not once per query).  It stores the scaled logits,
@@ -262,10 +266,10 @@ constexpr int SEL_FOLD = 16;         // chunk statistics in flight per thread in
 static_assert(SEL_KG * (SEL_QT / 4) == SEL_THREADS, "one 4x4 micro-tile per thread");
 
 struct SelWs {
-  float *logit;  // [S*H][c]
-  float2 *ml;    // [S*H][n_chunks] chunk (max, sum of exp)
-  float2 *mz;    // [S*H] pool (max, 1 / sum of exp)
-  int *cnt;      // [G][n_qtiles] arrivals
+  float *logit;  // [layers][S*H][c]
+  float2 *ml;    // [layers][S*H][n_chunks] chunk (max, sum of exp)
+  float2 *mz;    // [layers][S*H] pool (max, 1 / sum of exp)
+  int *cnt;      // [layers][G][n_qtiles] arrivals
 };
 
 __host__ __device__ inline int sel_chunks(int c) { return (c + SEL_KC - 1) / SEL_KC; }
@@ -297,12 +301,21 @@ __device__ __forceinline__ void sel_mma_bf16(float *d, uint32_t a0, uint32_t a1,
 
 template <typename T>
 __global__ void __launch_bounds__(SEL_THREADS)
-    k_attn_select_logits(const float *q, int S, int H, int G, int dh, int layer, KVView v,
-                         int s_end, int c, float scale, SelWs ws) {
+    k_attn_select_logits(const float *q, int S, int H, int G, int dh, int layer0, int n_qt,
+                         KVView v, int s_end, int c, float scale, SelWs ws) {
   TraceScope ts(TK_SELECT);
   pdl_trigger();
-  const int chunk = blockIdx.x, g = blockIdx.y, qt = blockIdx.z, nch = gridDim.x;
+  const int chunk = blockIdx.x, g = blockIdx.y, nch = gridDim.x;
+  const int li = blockIdx.z / n_qt, qt = blockIdx.z - li * n_qt, layer = layer0 + li;
   const int hpg = H / G, Nq = S * hpg;
+  {  // this layer's queries and arrays
+    const size_t NQ = (size_t)S * H;
+    q += li * NQ * dh;
+    ws.logit += li * NQ * c;
+    ws.ml += li * NQ * nch;
+    ws.mz += li * NQ;
+    ws.cnt += (size_t)li * G * n_qt;
+  }
   const int t0 = chunk * SEL_KC, q0 = qt * SEL_QT;
   const int nk = min(SEL_KC, c - t0), nq = min(SEL_QT, Nq - q0);
   const int tid = threadIdx.x;
@@ -523,12 +536,12 @@ __global__ void __launch_bounds__(SEL_THREADS)
   __threadfence();
   __syncthreads();
   if (tid == 0) trace_mark(2);  // chunk statistics stored
-  int *cnt = ws.cnt + (size_t)g * gridDim.z + qt;
+  int *cnt = ws.cnt + (size_t)g * n_qt + qt;
   if (tid == 0) *last = atomicAdd(cnt, 1) == nch - 1;
   __syncthreads();
   if (tid == 0) trace_mark(3);  // arrival counted
   if (!*last) return;
-  if (tid == 0) *cnt = 0;  // ready for the next layer's launch
+  if (tid == 0) *cnt = 0;  // ready for the next launch
   __threadfence();
   // fold: 4 threads per query, each over chunks o, o + 4, ... (SEL_FOLD
   // loads in flight), then the quad
@@ -556,19 +569,20 @@ __global__ void __launch_bounds__(SEL_THREADS)
   if (tid == 0) trace_mark(4);  // fold done (last CTA of the group)
 }
 
-// score[j] += sum over the S*H queries of exp(logit - max) / sum, in a fixed
-// order: a CTA takes ACC_KEYS keys; its ACC_SLICES thread slices sum
+// tot[layer][t] = sum over the S*H queries of exp(logit - max) / sum, in a fixed
+// order: a CTA takes ACC_KEYS keys of a layer; its ACC_SLICES thread slices sum
 // interleaved sets of the queries (coalesced along the keys), then one
 // thread per key adds the slice sums in slice order.
 constexpr int ACC_KEYS = 16, ACC_SLICES = 32;
 __global__ void __launch_bounds__(ACC_KEYS * ACC_SLICES)
-    k_attn_select_accum(const float *logit, const float2 *mz, int NQ, int c, int s_end,
-                        float *score) {
+    k_attn_select_accum(const float *logit, const float2 *mz, int NQ, int c, float *tot) {
   TraceScope ts(TK_SELECT_ACC);
   pdl_trigger();
   __shared__ float part[ACC_SLICES][ACC_KEYS];
   const int kk = threadIdx.x % ACC_KEYS, sl = threadIdx.x / ACC_KEYS;
   const int t = blockIdx.x * ACC_KEYS + kk;
+  logit += (size_t)blockIdx.y * NQ * c;
+  mz += (size_t)blockIdx.y * NQ;
   pdl_wait();  // logits and softmax statistics of the kernel before
   float s = 0.f;
   if (t < c) {
@@ -581,10 +595,22 @@ __global__ void __launch_bounds__(ACC_KEYS * ACC_SLICES)
   part[sl][kk] = s;
   __syncthreads();
   if (sl == 0 && t < c) {
-    float tot = 0.f;
+    float sum = 0.f;
 #pragma unroll
-    for (int i = 0; i < ACC_SLICES; ++i) tot += part[i][kk];
-    score[s_end + t] += tot;
+    for (int i = 0; i < ACC_SLICES; ++i) sum += part[i][kk];
+    tot[(size_t)blockIdx.y * c + t] = sum;
+  }
+}
+
+// Keys of the layers' sums, added in layer order.
+__global__ void k_layer_sum_keys(const float *tot, int layers, int c, unsigned long long *keys) {
+  pdl_trigger();
+  pdl_wait();
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < c; t += gridDim.x * blockDim.x) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int l = 0; l < layers; ++l) s += tot[(size_t)l * c + t];
+    keys[t] = (unsigned long long)ord_f32(s) + 1ull;
   }
 }
 
@@ -692,17 +718,26 @@ const char *launch_topk(const unsigned long long *keys, int n, int s_end, int K,
 
 namespace {
 struct SelLayout {
-  size_t logit, ml, mz, cnt, total;  // byte offsets into the workspace
+  size_t q, tot, logit, ml, mz, cnt, total;  // byte offsets into the workspace
+  int group;                                 // layers scored per launch
 };
+// The logits of a group of layers stay within SEL_GROUP_BYTES (about half of
+// L2, from which the next kernel reads them), at least one layer.
+constexpr size_t SEL_GROUP_BYTES = (size_t)64 << 20;
 SelLayout sel_layout(int S, const Dims &dm, int c) {
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t NQ = (size_t)S * dm.H, nqt = ((size_t)S * (dm.H / dm.G) + SEL_QT - 1) / SEL_QT;
+  const size_t fit = SEL_GROUP_BYTES / (NQ * c * sizeof(float));
   SelLayout o;
-  o.logit = 0;
-  o.ml = o.logit + al(NQ * c * sizeof(float));
-  o.mz = o.ml + al(NQ * sel_chunks(c) * sizeof(float2));
-  o.cnt = o.mz + al(NQ * sizeof(float2));
-  o.total = o.cnt + al((size_t)dm.G * nqt * sizeof(int));
+  o.group = fit < 1 ? 1 : fit < (size_t)dm.L ? (int)fit : dm.L;
+  while (o.group > 1 && (size_t)o.group * nqt > 65535) --o.group;  // grid z
+  o.q = 0;
+  o.tot = o.q + al((size_t)dm.L * NQ * dm.dh * sizeof(float));
+  o.logit = o.tot + al((size_t)dm.L * c * sizeof(float));
+  o.ml = o.logit + al(o.group * NQ * c * sizeof(float));
+  o.mz = o.ml + al(o.group * NQ * sel_chunks(c) * sizeof(float2));
+  o.cnt = o.mz + al(o.group * NQ * sizeof(float2));
+  o.total = o.cnt + al((size_t)o.group * dm.G * nqt * sizeof(int));
   return o;
 }
 }  // namespace
@@ -711,19 +746,26 @@ size_t attn_select_ws_bytes(int S, const Dims &dm, int n_pool) {
   return n_pool > 0 && S > 0 ? sel_layout(S, dm, n_pool).total : 0;
 }
 
-void launch_attn_select_scores(const float *q, int S, const Dims &dm, int layer, KVView v,
-                               int s_end, int n, void *ws_base, bool first_layer,
-                               float *scores, cudaStream_t s) {
+float *attn_select_queries(void *ws_base, int S, const Dims &dm, int n_pool, int layer) {
+  const SelLayout o = sel_layout(S, dm, n_pool);
+  return (float *)((char *)ws_base + o.q) + (size_t)layer * S * dm.H * dm.dh;
+}
+
+int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_end, int n,
+                              void *ws_base, unsigned long long *keys, cudaStream_t s) {
   const int c = n - s_end;
-  if (c <= 0 || S <= 0) return;
+  if (c <= 0 || S <= 0) return 0;
   const float scale = (float)(1.0 / sqrt((double)dm.dh));
   const SelLayout o = sel_layout(S, dm, c);
+  if (layer + 1 < dm.L && (layer + 1) % o.group) return 0;  // the group's last layer scores it
   char *b = (char *)ws_base;
   SelWs ws{(float *)(b + o.logit), (float2 *)(b + o.ml), (float2 *)(b + o.mz), (int *)(b + o.cnt)};
+  float *tot = (float *)(b + o.tot);
   const int nqt = (S * (dm.H / dm.G) + SEL_QT - 1) / SEL_QT;
+  const int layer0 = layer / o.group * o.group, layers = layer - layer0 + 1;
   // arrival counts start at zero; each launch's last CTAs leave them at zero
-  if (first_layer) cudaMemsetAsync(ws.cnt, 0, (size_t)dm.G * nqt * sizeof(int), s);
-  const dim3 grid(sel_chunks(c), dm.G, nqt);
+  if (layer0 == 0) cudaMemsetAsync(ws.cnt, 0, (size_t)o.group * dm.G * nqt * sizeof(int), s);
+  const dim3 grid(sel_chunks(c), dm.G, nqt * layers);
   // bf16: q_hi, q_lo and keys as bf16 rows of dh + 8; fp32: q and keys as
   // fp32 columns of dh.  The logits tile reuses the keys' space.
   const bool bf16 = dm.dtype == KVR_DTYPE_BF16;
@@ -734,10 +776,15 @@ void launch_attn_select_scores(const float *q, int S, const Dims &dm, int layer,
   auto kern = bf16 ? k_attn_select_logits<__nv_bfloat16> : k_attn_select_logits<float>;
   // fp32 at dh 128, plus the trace build's static shared memory, passes 48 KB
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  launch_pdl(kern, grid, SEL_THREADS, smem, s, q, S, dm.H, dm.G, dm.dh, layer, v, s_end, c, scale,
-             ws);
-  launch_pdl(k_attn_select_accum, (c + ACC_KEYS - 1) / ACC_KEYS, ACC_KEYS * ACC_SLICES, 0, s,
-             (const float *)ws.logit, (const float2 *)ws.mz, S * dm.H, c, s_end, scores);
+  launch_pdl(kern, grid, SEL_THREADS, smem, s,
+             (const float *)attn_select_queries(ws_base, S, dm, c, layer0), S, dm.H, dm.G, dm.dh,
+             layer0, nqt, v, s_end, c, scale, ws);
+  launch_pdl(k_attn_select_accum, dim3((c + ACC_KEYS - 1) / ACC_KEYS, layers),
+             ACC_KEYS * ACC_SLICES, 0, s, (const float *)ws.logit, (const float2 *)ws.mz, S * dm.H,
+             c, tot + (size_t)layer0 * c);
+  if (layer + 1 < dm.L) return 2;
+  launch_pdl(k_layer_sum_keys, grid_for(c, 256), 256, 0, s, (const float *)tot, dm.L, c, keys);
+  return 3;
 }
 
 void launch_kv_deviation(const float *qkv, const float2 *rope, const int32_t *pos, int M,

@@ -623,14 +623,17 @@ struct SimpleKeys {
 // *bound, which must hold n - 1 on entry.
 void launch_first_delim(const int32_t *tokens, int n, int s_end, int delim, int *bound,
                         cudaStream_t s);
-// Attention selector, one layer: adds to scores[j], j in [s_end, n), the
-// pool-softmax probabilities of the S span rows' queries (fp32 q, [S][H*dh]).
-// ws_base: attn_select_ws_bytes(S, dm, n - s_end) bytes; first_layer zeroes
-// its arrival counts.
+// Attention selector over the workspace ws_base (attn_select_ws_bytes(S, dm,
+// n - s_end) bytes).  The pass leaves layer l's span queries (fp32 [S][H*dh])
+// in attn_select_queries(.., l) and calls launch_attn_select_scores after each
+// layer's: a group of layers is scored at its last one, and after the last
+// layer keys[j - s_end] are the top-K keys of the sums over the layers, in
+// layer order, of the pool-softmax probabilities of key j.  Returns the
+// kernels launched.
 size_t attn_select_ws_bytes(int S, const Dims &dm, int n_pool);
-void launch_attn_select_scores(const float *q, int S, const Dims &dm, int layer, KVView v,
-                               int s_end, int n, void *ws_base, bool first_layer,
-                               float *scores, cudaStream_t s);
+float *attn_select_queries(void *ws_base, int S, const Dims &dm, int n_pool, int layer);
+int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_end, int n,
+                              void *ws_base, unsigned long long *keys, cudaStream_t s);
 void launch_kv_deviation(const float *qkv, const float2 *rope, const int32_t *pos, int M,
                          const Dims &dm, KVView v, float *scores, cudaStream_t s);
 void launch_float_keys(const float *scores, int n, int s_end, unsigned long long *keys,

@@ -116,3 +116,30 @@ def test_answer_logprob_row_widths(vocab):
     want = oracle.answer_logprob(cfg, W, oracle.prefill(cfg, W, doc), prompt, answer)
     assert abs(got - want) <= 1e-4 * abs(want)  # the fp32 path's tolerance
     model.close()
+
+
+@pytest.mark.parametrize("policy,edit,n", [("attention", 3, 1500), ("attention", 220, 1500),
+                                           ("cacheblend", 3, 1500), ("cacheblend", 3, 700)])
+def test_model_selectors_over_layer_groups(policy, edit, n):
+    # Attention: 220 span rows' logits of 14 layers are more than one launch takes
+    # (groups of 6, 6 and 2 layers), 3 rows' are one launch; CacheBlend:
+    # head-wise projections of many and of fewer rows
+    cfg = small_cfg(n_heads=14, n_kv_heads=2, head_dim=128, n_layers=14)
+    W = synth.weights(cfg, 0)
+    model = kv.Model(cfg, None, seed=0, max_context=2048, max_rows=2048)
+    doc = synth.document(6, n, cfg["vocab"])
+    cache = model.prefill(doc)
+    k, v = cache.read(np.arange(n))
+    ref = oracle.Cache(*(np.ascontiguousarray(x.transpose(1, 0, 2, 3)) for x in (k, v)), doc.copy())
+    s = n // 3
+    new = synth.edit_tokens(8, doc[s:s + edit], cfg["vocab"])
+    got = model.select(cache, policy, 32, s, new)
+    sc, D = oracle.scores(cfg, W, ref, policy, s, new)
+    sc, at = np.asarray(sc)[s + edit:n], got - s - edit
+    # the 32 highest, but for scores within the rounding of the 32nd
+    kth, band = np.sort(sc)[-32], TOL * np.abs(sc).max()
+    assert len(got) == 32 and np.all(np.diff(got) > 0) and np.all(sc[at] >= kth - band)
+    assert set(np.flatnonzero(sc > kth + band)) <= set(at.tolist())
+    k1, v1 = cache.read(np.arange(n))
+    assert np.array_equal(k, k1) and np.array_equal(v, v1)
+    model.close()
