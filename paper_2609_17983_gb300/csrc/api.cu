@@ -623,10 +623,12 @@ kvr_status run_pass_graph(kvr_model *m, kvr_cache *c, const Rows &r) {
   return KVR_OK;
 }
 
-kvr_status sync_model(kvr_model *m) {
+// flag_queued: the stream's work already writes the device flag to m->flag_h.
+kvr_status sync_model(kvr_model *m, bool flag_queued = false) {
   // the flag's copy joins the stream's work: one round trip to the host
-  cudaError_t e = cudaMemcpyAsync(m->flag_h, m->dev_flag, sizeof(int), cudaMemcpyDeviceToHost,
-                                  m->stream);
+  cudaError_t e = flag_queued ? cudaSuccess
+                              : cudaMemcpyAsync(m->flag_h, m->dev_flag, sizeof(int),
+                                                cudaMemcpyDeviceToHost, m->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
   if (e != cudaSuccess) return fail(KVR_E_CUDA, "device error: %s", cudaGetErrorString(e));
   const int flag = *m->flag_h;
@@ -650,6 +652,27 @@ kvr_status grow_scratch(kvr_model *m, void *&buf, size_t &have, size_t need, con
   have = buf ? need : 0;
   if (!buf) return fail(KVR_E_NOMEM, "%s: %zu bytes", what, need);
   return KVR_OK;
+}
+
+// Whether rows (bytes of K, as many of V) go to the host by the kernel's own stores
+// (launch_cache_read_host): into page-locked memory that the device writes
+// directly.  Measured against positions up, gather, two copies and the flag's:
+// 27 -> 19 us for 0.3 MB, 39 -> 31 for 1.3 MB, 70 -> 60 for 4.2 MB; larger reads
+// are bound by the link either way.
+constexpr size_t HOST_READ_MAX_BYTES = (size_t)8 << 20;
+bool host_read_direct(int n_pos, size_t bytes, const void *k_out, const void *v_out) {
+  if (n_pos > HOST_READ_MAX_POS || bytes > HOST_READ_MAX_BYTES ||
+      (((uintptr_t)k_out | (uintptr_t)v_out) & 15))
+    return false;
+  for (const void *p : {k_out, v_out}) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeHost || a.devicePointer != p) return false;
+  }
+  return true;
 }
 
 kvr_status use_device(const kvr_model *m) {
@@ -1364,7 +1387,14 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
     r.max_pos = P[M - 1];
     st = plan_attention(m, r, P.data(), nullptr);
     const size_t row_b = (size_t)dm.L * dm.G * dm.dh * dm.es();  // one row, all layers
-    if (!st && k_out) {
+    // Few rows of few layers are read from the cache when the pass is over: below
+    // this the copies behind the layer groups cost more than they overlap (36
+    // fp32 rows of two layers 89 -> 84 us, 134 rows of four 8B-shape layers 454 ->
+    // 449; 40 rows of 32 layers, 2.6 MB, 3140 against 3153).
+    constexpr size_t DIRECT_BYTES = (size_t)1 << 20;
+    const bool direct =
+        k_out && M * row_b <= DIRECT_BYTES && host_read_direct(M, M * row_b, k_out, v_out);
+    if (!st && k_out && !direct) {
       st = grow_scratch(m, m->rows_scratch, m->rows_scratch_bytes, 2 * M * row_b, "row buffer");
       r.rows_out = m->rows_scratch;
       r.rd_every = (dm.L + KVR_RD_GROUPS - 1) / KVR_RD_GROUPS;
@@ -1373,7 +1403,15 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
       launched = true;
       st = run_pass_graph(m, c, r);
     }
-    if (!st && k_out) {
+    if (!st && direct) {
+      launch_cache_read_host(r.single, dm.dtype, P.data(), M, 0, dm.L, dm.G, dm.dh, k_out, v_out,
+                             m->dev_flag, m->flag_h, m->stream);
+      st = launch_check(m, 1);
+      if (!st)
+        st = sync_model(m, true);
+      else
+        cudaStreamSynchronize(m->stream);
+    } else if (!st && k_out) {
       // group g's rows leave as soon as the pass has written them
       const char *kd = (const char *)r.rows_out, *vd = kd + M * row_b;
       const size_t lb = row_b / dm.L;
@@ -2000,6 +2038,14 @@ kvr_status cache_read(const kvr_cache *c, const int32_t *positions, int32_t n_po
   KVR_TRY(use_device(m));
   const size_t elems = (size_t)n_pos * (l1 - l0) * dm.G * dm.dh;
   const size_t eb = raw ? dm.es() : 4;
+  if (raw && host_read_direct(n_pos, elems * eb, k_out, v_out)) {
+    launch_cache_read_host(c->view(), dm.dtype, positions, n_pos, l0, l1, dm.G, dm.dh, k_out,
+                           v_out, m->dev_flag, m->flag_h, m->stream);
+    const kvr_status st = launch_check(m, 1);
+    if (!st) return sync_model(m, true);
+    cudaStreamSynchronize(m->stream);
+    return st;
+  }
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t pos_b = al((size_t)n_pos * 4), row_b = al(elems * eb);
   const size_t need = pos_b + 2 * row_b;

@@ -1,6 +1,8 @@
 // k_rows.cu -- per-row kernels of the repair pass: seeded weight init,
 // embedding gather, RMSNorm, RoPE + K/V scatter into the paged cache,
 // and cache row readback / save / restore.
+#include <algorithm>
+
 #include "kvr_internal.cuh"
 
 namespace kvr {
@@ -400,6 +402,35 @@ __global__ void k_cache_gather_raw(KVView v, const int32_t *pos, int n_pos, int 
   }
 }
 
+// k_cache_gather_raw into page-locked host memory, for a read that is over
+// sooner than its copies would be set up: the positions come with the launch,
+// the rows leave by the stores themselves, and the device error flag goes
+// with them (everything queued before has run).
+struct HostReadPos {
+  int32_t p[HOST_READ_MAX_POS];
+};
+__global__ void k_cache_read_host(KVView v, const __grid_constant__ HostReadPos pos, int n_pos,
+                                  int l0, int nl, int G, int vr, int es, uint4 *k_out,
+                                  uint4 *v_out, const int *flag_in, int *flag_out) {
+  pdl_trigger();
+  pdl_wait();
+  const unsigned total = (unsigned)n_pos * nl * G * vr;
+  const uint4 *c = (const uint4 *)v.pages;
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += gridDim.x * blockDim.x) {
+    const unsigned i = e % vr;
+    unsigned r = e / vr;
+    const int g = (int)(r % G);
+    r /= G;
+    const int l = (int)(r % nl), p = pos.p[r / nl];
+    const uint4 k = c[v.offset(l0 + l, 0, g, p) * es / 16 + i];
+    const uint4 w = c[v.offset(l0 + l, 1, g, p) * es / 16 + i];
+    k_out[e] = k;
+    v_out[e] = w;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *flag_out = *flag_in;
+}
+
 // The inverse of k_cache_gather_raw for consecutive positions p0 .. p0+n_pos-1
 // and every layer: rows [n_pos][L][G][dh] of k_in / v_in written into the pages.
 template <typename T>
@@ -657,6 +688,16 @@ void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, int n_pos,
         v, pos + p0, np, l0, l1 - l0, G, vr, es, (uint4 *)k_out + p0 * per_pos,
         (uint4 *)v_out + p0 * per_pos);
   }
+}
+
+void launch_cache_read_host(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
+                            int G, int dh, void *k_out, void *v_out, const int *flag_in,
+                            int *flag_out, cudaStream_t s) {
+  const int es = dtype == KVR_DTYPE_BF16 ? 2 : 4, vr = dh * es / 16;
+  HostReadPos p;
+  std::copy(pos, pos + n_pos, p.p);
+  launch_pdl(k_cache_read_host, grid_for((size_t)n_pos * (l1 - l0) * G * vr, 256), 256, 0, s, v, p,
+             n_pos, l0, l1 - l0, G, vr, es, (uint4 *)k_out, (uint4 *)v_out, flag_in, flag_out);
 }
 
 void launch_cache_scatter_raw(KVView v, int dtype, int p0, int n_pos, const void *k_in,

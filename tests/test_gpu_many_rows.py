@@ -143,3 +143,24 @@ def test_model_selectors_over_layer_groups(policy, edit, n):
     k1, v1 = cache.read(np.arange(n))
     assert np.array_equal(k, k1) and np.array_equal(v, v1)
     model.close()
+
+
+@pytest.mark.parametrize("rows", [1, 512, 513])
+def test_read_into_page_locked_memory(rows):
+    # by the kernel's stores (up to 512 positions, 16-byte aligned), and by copies
+    # (more, or off the alignment): the same rows as into pageable memory
+    import torch
+    cfg = small_cfg(n_heads=8, n_kv_heads=2, head_dim=64)
+    model = kv.Model(cfg, None, seed=0, max_context=1024, max_rows=1024)
+    cache, _ = loaded(model, cfg, 700, 3)
+    P = np.sort(np.random.default_rng(rows).permutation(700)[:rows])
+    want = cache.read_raw(P)
+    shape, count = want[0].shape, want[0].size
+    for off in (0, 4):
+        buf = [torch.zeros(count + 8, dtype=torch.int16, pin_memory=True).numpy().view(np.uint16)
+               for _ in range(2)]
+        out = [b[off:off + count].reshape(shape) for b in buf]
+        cache.read_raw(P, k_out=out[0], v_out=out[1])
+        assert all(np.array_equal(o, w) for o, w in zip(out, want))
+        assert all(not b[:off].any() and not b[off + count:].any() for b in buf)
+    model.close()
