@@ -447,17 +447,18 @@ size_t configure(PairGemm &p, int M, int N, int K, int clusters, int smem_limit)
 // one token tile the few-row kernel splits K over all SMs and leaves the sums to
 // the next kernel, and only gate/up, which sums its own tiles, gains by pairs
 // (192 rows and below equal, 256 rows 63 -> 57).  Above 256 rows its CTAs walk
-// several token tiles (gate/up of 300 rows 107 -> 67), and what is left is the
-// pairs' launch cost, about 8 us: projections below 32.5 GFLOP stay (4096 x
-// 4096, 600 rows 27 against 33, 904 rows 34 against 37; 4096 x 14336, 300 rows
-// 52 against 49; 6144 x 4096, 904 rows 88 against 79).
+// several token tiles (gate/up of 300 rows 107 -> 67), and the sums it leaves
+// cost the next kernel more (with its RoPE, 6144 x 4096: 300 rows 81 -> 73, 600
+// rows 116 -> 87); against that stand the pairs' launch and tail, about 8 us:
+// 4096 x 4096 with its RMSNorm, 300 rows 46 against 52, 600 rows 57 against 59.
 bool gemm_pair_takes(int M, int N, int K, int epi) {
   static const bool off = [] {
     const char *e = getenv("KVR_DISABLE_PAIR_GEMM");
     return e && e[0] == '1';
   }();
-  if (off || 2.0 * M * N * K < 32.5e9) return false;
-  return M > 256 || (M > 192 && epi == GEMM_EPI_SWIGLU);
+  const double flops = 2.0 * M * N * K;
+  if (off) return false;
+  return M > 256 ? flops >= 12e9 : M > 192 && epi == GEMM_EPI_SWIGLU && flops >= 32.5e9;
 }
 
 const char *launch_gemm_pair(const GemmArgs &g, const CUtensorMap &tmW, int epi, void *out2,

@@ -283,67 +283,57 @@ __global__ void __launch_bounds__(ROPE_HEADS * 64) k_rope_scatter(const RopeArgs
   }
 }
 
-// Many rows: four rotated pairs per thread (16-byte loads, 8- or
-// 16-byte stores), and without a split view ROPE_RPB rows at a time, all their
-// loads in flight together.  One pair per thread, 2-byte stores: 75 us for 4096
-// rows of a 6144-wide projection (100 MB read, 50 MB written, 2.0 TB/s).
-constexpr int ROPE_RPB = 4, ROPE_THREADS = 256;
+// Many rows: a CTA per row, four rotated pairs per thread (16-byte loads, 8- or
+// 16-byte stores) of HPT heads, which share the position, its table entries and
+// page; the projection's loads do not wait for any of them.  One pair per thread
+// with 2-byte stores took 75 us for 4096 rows of a 6144-wide projection (100 MB
+// read, 50 MB written); four rows of one head per thread 44 (107 registers, two
+// CTAs an SM).
+constexpr int ROPE_THREADS = 256;
 constexpr int ROPE_MANY = 64;  // rows from which it is taken (40 rows: equal; 64 rows: 9.9 -> 8.2 us)
-template <typename T, int RPB>
-__global__ void __launch_bounds__(ROPE_THREADS) k_rope_rows(const RopeArgs a) {
+template <typename T, int HPT>
+__global__ void __launch_bounds__(ROPE_THREADS, HPT > 1 ? 4 : 1) k_rope_rows(const RopeArgs a) {
   TraceScope ts(TK_ROPE);
   pdl_trigger();
   const int half = a.dh >> 1, tph = half >> 2;  // threads per head
-  const int hh = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph;
+  const int slots = blockDim.x / tph, h0 = blockIdx.y * slots * HPT + threadIdx.x / tph;
   const int t = threadIdx.x % tph * 4;
-  if (hh >= a.heads) return;
-  const int Nqkv = (a.H + 2 * a.G) * a.dh, n1 = hh * a.dh + t, n2 = n1 + half;
-  const int r0 = blockIdx.x * RPB, nr = min(RPB, a.M - r0);
+  if (h0 >= a.heads) return;
+  const int i = blockIdx.x, Nqkv = (a.H + 2 * a.G) * a.dh;
   const SplitView &sv = a.sv;
-  int p[RPB];
-  T *c[RPB];
-  size_t o[RPB], ro[RPB];
-#pragma unroll
-  for (int k = 0; k < RPB; ++k) {
-    p[k] = k < nr ? a.pos[r0 + k] : 0;
-    c[k] = nullptr;
-    if (k < nr) rope_dst(a, hh, r0 + k, p[k], c[k], o[k], ro[k]);
-  }
+  const int p = a.pos[i];
   pdl_wait();
   ts.waited();
-  float4 x1[RPB], x2[RPB], ca[RPB], cb[RPB];
+  float4 x1[HPT], x2[HPT];
 #pragma unroll
-  for (int k = 0; k < RPB; ++k) {
-    if (k >= nr) continue;
-    const float *x = a.qkv + (size_t)(r0 + k) * Nqkv;
+  for (int k = 0; k < HPT; ++k) {
+    const int hh = h0 + k * slots, n1 = hh * a.dh + t;
+    if (hh >= a.heads) break;
+    const float *x = a.qkv + (size_t)i * Nqkv;
     x1[k] = ld4(x, n1);
-    x2[k] = ld4(x, n2);
-    ca[k] = cb[k] = make_float4(1.f, 0.f, 1.f, 0.f);
-    if (hh < a.H + a.G) {
-      const float4 *cs = (const float4 *)(a.rope + (size_t)p[k] * half + t);
-      ca[k] = cs[0];
-      cb[k] = cs[1];
-    }
-    if (RPB == 1 && sv.ws) {
-      const int i = r0;
+    x2[k] = ld4(x, n1 + half);
+    if (HPT == 1 && sv.ws) {
       const SplitTile stl = split_tile(sv, (long long)((hh * a.dh) >> 7) * sv.m_tiles + i / sv.BN);
       x1[k] = split_value4(sv, stl, x1[k], i, n1);
-      x2[k] = split_value4(sv, stl, x2[k], i, n2);
+      x2[k] = split_value4(sv, stl, x2[k], i, n1 + half);
     }
   }
+  const float4 *cs = (const float4 *)(a.rope + (size_t)p * half + t);
+  const float4 ca = cs[0], cb = cs[1];
 #pragma unroll
-  for (int k = 0; k < RPB; ++k) {
-    if (k >= nr) continue;
-    float4 y1 = x1[k], y2 = x2[k];
+  for (int k = 0; k < HPT; ++k) {
+    const int hh = h0 + k * slots;
+    if (hh >= a.heads) break;
+    const float4 u = x1[k], w = x2[k];
+    float4 y1 = u, y2 = w;
     if (hh < a.H + a.G) {
-      const float4 u = x1[k], w = x2[k];
-      y1 = make_float4(u.x * ca[k].x - w.x * ca[k].y, u.y * ca[k].z - w.y * ca[k].w,
-                       u.z * cb[k].x - w.z * cb[k].y, u.w * cb[k].z - w.w * cb[k].w);
-      y2 = make_float4(w.x * ca[k].x + u.x * ca[k].y, w.y * ca[k].z + u.y * ca[k].w,
-                       w.z * cb[k].x + u.z * cb[k].y, w.w * cb[k].z + u.w * cb[k].w);
+      y1 = make_float4(u.x * ca.x - w.x * ca.y, u.y * ca.z - w.y * ca.w, u.z * cb.x - w.z * cb.y,
+                       u.w * cb.z - w.w * cb.w);
+      y2 = make_float4(w.x * ca.x + u.x * ca.y, w.y * ca.z + u.y * ca.w, w.z * cb.x + u.z * cb.y,
+                       w.w * cb.z + u.w * cb.w);
     }
     if (hh < a.H) {
-      const size_t q = (size_t)(r0 + k) * a.H * a.dh + n1;
+      const size_t q = (size_t)i * a.H * a.dh + hh * a.dh + t;
       if (a.q_out) {
         st4(a.q_out, q, y1);
         st4(a.q_out, q + half, y2);
@@ -353,13 +343,17 @@ __global__ void __launch_bounds__(ROPE_THREADS) k_rope_rows(const RopeArgs a) {
         st4(a.qb_out, q, make_float4(y1.x * s, y1.y * s, y1.z * s, y1.w * s));
         st4(a.qb_out, q + half, make_float4(y2.x * s, y2.y * s, y2.z * s, y2.w * s));
       }
-    } else if (c[k]) {
-      st4(c[k], o[k] + t, y1);
-      st4(c[k], o[k] + t + half, y2);
-      if (a.rows_out) {
-        st4((T *)a.rows_out, ro[k] + t, y1);
-        st4((T *)a.rows_out, ro[k] + t + half, y2);
-      }
+      continue;
+    }
+    T *c;
+    size_t o = 0, ro = 0;
+    rope_dst(a, hh, i, p, c, o, ro);
+    if (!c) continue;
+    st4(c, o + t, y1);
+    st4(c, o + t + half, y2);
+    if (a.rows_out) {
+      st4((T *)a.rows_out, ro + t, y1);
+      st4((T *)a.rows_out, ro + t + half, y2);
     }
   }
 }
@@ -651,10 +645,12 @@ void launch_rope_scatter(const float *qkv, const float2 *rope, const int32_t *po
       launch_pdl(k_rope_scatter<T>, dim3(M, (heads + ROPE_HEADS - 1) / ROPE_HEADS),
                  ROPE_HEADS * dm.dh / 2, 0, s, a);
     } else {
+      // heads per thread: three where a CTA's thread groups are that many times
+      // fewer; one to add split tiles (each has up to eight parts in flight)
       const int tph = dm.dh / 8, threads = std::min(ROPE_THREADS, (heads * tph + 31) / 32 * 32);
-      const int hpc = threads / tph, rpb = a.sv.ws ? 1 : ROPE_RPB;
-      launch_pdl(rpb > 1 ? k_rope_rows<T, ROPE_RPB> : k_rope_rows<T, 1>,
-                 dim3((M + rpb - 1) / rpb, (heads + hpc - 1) / hpc), threads, 0, s, a);
+      const int slots = threads / tph, hpt = a.sv.ws || heads <= slots ? 1 : 3;
+      launch_pdl(hpt > 1 ? k_rope_rows<T, 3> : k_rope_rows<T, 1>,
+                 dim3(M, (heads + slots * hpt - 1) / (slots * hpt)), threads, 0, s, a);
     }
   };
   if (dm.dtype == KVR_DTYPE_BF16)
