@@ -217,6 +217,13 @@ __device__ __forceinline__ void rope_dst(const RopeArgs &a, int hh, int i, int p
   }
 }
 
+// A pair rotated, with the rounding written out: a row's bits do not depend on how
+// many rows share its pass (kvr_margin runs two answers in one).
+__device__ __forceinline__ void rotate(float x1, float x2, float c, float s, float &y1, float &y2) {
+  y1 = __fmaf_rn(x1, c, -__fmul_rn(x2, s));  // x1, x2: copies, y may name the same pair
+  y2 = __fmaf_rn(x2, c, __fmul_rn(x1, s));
+}
+
 // A few rows: grid (M, ceil((H + 2G) / ROPE_HEADS)), block ROPE_HEADS * dh/2, a
 // rotated pair per thread -- latency counts, and every load is in flight at once.
 constexpr int ROPE_HEADS = 8;  // heads per CTA
@@ -257,11 +264,7 @@ __global__ void __launch_bounds__(ROPE_HEADS * 64) k_rope_scatter(const RopeArgs
     x1 = x[n1];
     x2 = x[n2];
   }
-  if (hh < a.H + a.G) {
-    const float r1 = x1 * cs.x - x2 * cs.y, r2 = x2 * cs.x + x1 * cs.y;
-    x1 = r1;
-    x2 = r2;
-  }
+  if (hh < a.H + a.G) rotate(x1, x2, cs.x, cs.y, x1, x2);
   if (hh < a.H) {
     const size_t q = (size_t)i * a.H * a.dh + n1;
     if (a.q_out) {
@@ -327,10 +330,10 @@ __global__ void __launch_bounds__(ROPE_THREADS, HPT > 1 ? 4 : 1) k_rope_rows(con
     const float4 u = x1[k], w = x2[k];
     float4 y1 = u, y2 = w;
     if (hh < a.H + a.G) {
-      y1 = make_float4(u.x * ca.x - w.x * ca.y, u.y * ca.z - w.y * ca.w, u.z * cb.x - w.z * cb.y,
-                       u.w * cb.z - w.w * cb.w);
-      y2 = make_float4(w.x * ca.x + u.x * ca.y, w.y * ca.z + u.y * ca.w, w.z * cb.x + u.z * cb.y,
-                       w.w * cb.z + u.w * cb.w);
+      rotate(u.x, w.x, ca.x, ca.y, y1.x, y2.x);
+      rotate(u.y, w.y, ca.z, ca.w, y1.y, y2.y);
+      rotate(u.z, w.z, cb.x, cb.y, y1.z, y2.z);
+      rotate(u.w, w.w, cb.z, cb.w, y1.w, y2.w);
     }
     if (hh < a.H) {
       const size_t q = (size_t)i * a.H * a.dh + hh * a.dh + t;
