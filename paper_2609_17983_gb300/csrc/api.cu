@@ -105,25 +105,50 @@ void prof_collect(kvr_model *m) {
 
 // ------------------------------------------------------------ staging
 
-// Copy host int32 data to device through the model's pinned staging buffer.
-// Copies take consecutive 128-byte-aligned slots, so a call does not wait for
-// the copies queued before it; when the next slot would not fit, the buffer
-// starts over after every queued copy has completed.
-kvr_status stage_h2d(kvr_model *m, int32_t *dst_dev, const int32_t *src, size_t count) {
+// Host int32 data to the device through the model's pinned staging buffer:
+// stage_add fills a slot, stage_flush sends every slot filled since in one
+// launch, ahead of all work queued after it.  A pass flushes by itself (embed);
+// what reads staged data before that calls stage_flush.  Slots are consecutive
+// and 128-byte aligned, so a call does not wait for the uploads queued before
+// it; when the next slot would not fit, the buffer starts over after every queued
+// upload has completed.
+kvr_status stage_flush(kvr_model *m) {
+  if (m->staged.empty()) return KVR_OK;
+  launch_upload(m->staged.data(), (int)m->staged.size(), m->stream);
+  m->staged.clear();
+  KVR_TRY(launch_check(m, 0));  // an upload, not a kernel of the pass
+  CUDA_TRY(cudaEventRecord(m->stage_ev, m->stream));
+  return KVR_OK;
+}
+
+kvr_status stage_add(kvr_model *m, int32_t *dst, const int32_t *src, size_t count) {
   if (count == 0) return KVR_OK;
   if (count > m->stage_cap) return fail(KVR_E_UNSUPPORTED, "staging overflow (%zu)", count);
+  // the segments of a launch run in no order: one that overwrites another goes behind it
+  bool flush = m->staged.size() == UPLOAD_MAX || m->stage_off + count > m->stage_cap;
+  for (const Upload &u : m->staged) flush = flush || (dst < u.dst + u.words && u.dst < dst + count);
+  if (flush) KVR_TRY(stage_flush(m));
   if (m->stage_off + count > m->stage_cap) {
     CUDA_TRY(cudaEventSynchronize(m->stage_ev));
     m->stage_off = 0;
   }
   int32_t *h = m->stage_h + m->stage_off;
   memcpy(h, src, count * sizeof(int32_t));
-  CUDA_TRY(cudaMemcpyAsync(dst_dev, h, count * sizeof(int32_t), cudaMemcpyHostToDevice,
-                           m->stream));
-  CUDA_TRY(cudaEventRecord(m->stage_ev, m->stream));
+  m->staged.push_back({dst, h, count});
   m->stage_off += (count + 31) / 32 * 32;
   return KVR_OK;
 }
+
+kvr_status stage_h2d(kvr_model *m, int32_t *dst, const int32_t *src, size_t count) {
+  KVR_TRY(stage_add(m, dst, src, count));
+  return stage_flush(m);
+}
+
+// Nothing stays staged when a call returns, whichever way it does.
+struct StageScope {
+  kvr_model *m;
+  ~StageScope() { stage_flush(m); }
+};
 
 // ------------------------------------------------------------ GEMM dispatch
 
@@ -325,7 +350,7 @@ kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32
     r.pairs = m->blocks_d + p.nb;
     r.n_pairs = (int)p.pairs.size();
   }
-  KVR_TRY(stage_h2d(m, (int32_t *)m->blocks_d, p.b.data(), p.b.size()));
+  KVR_TRY(stage_add(m, (int32_t *)m->blocks_d, p.b.data(), p.b.size()));
   r.tc5 = p.tc5;
   r.blocks = m->blocks_d;
   r.n_blocks = p.nb;
@@ -335,6 +360,7 @@ kvr_status plan_attention(kvr_model *m, Rows &r, const int32_t *pos, const int32
 }
 
 kvr_status embed(kvr_model *m, const Rows &r) {
+  KVR_TRY(stage_flush(m));
   Prof pr(m, P_EMBED, (int64_t)r.M * m->dims.d * (int64_t)m->dims.es());
   m->pending = SplitView{};
   launch_embed_rows(m->embed, m->dims.dtype, r.tokens, r.doc_tokens, r.rowdoc, r.pos, r.M,
@@ -593,6 +619,7 @@ kvr_status run_pass(kvr_model *m, const Rows &r, bool kv_only) {
 // can be captured (not the legacy default stream) and with profiling off.
 kvr_status run_pass_graph(kvr_model *m, kvr_cache *c, const Rows &r) {
   if (!m->use_graphs || m->prof || m->stream == nullptr) return run_pass(m, r, true);
+  KVR_TRY(stage_flush(m));  // not part of the graph
   for (auto &g : c->graphs)
     if (g.M == r.M && g.nb == r.n_blocks && g.np == r.n_pairs && g.ns == r.n_splits &&
         g.rows_out == r.rows_out) {
@@ -1185,6 +1212,7 @@ int64_t kvr_launch_count(const kvr_model *m) { return m ? m->launches : 0; }
 void kvr_cache_free(kvr_cache *c) {
   if (!c) return;
   cudaSetDevice(c->model->device);
+  stage_flush(c->model);
   cudaStreamSynchronize(c->model->stream);
   for (auto &g : c->graphs) cudaGraphExecDestroy(g.exec);
   auto &live = c->model->caches;
@@ -1251,8 +1279,8 @@ static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_
   }
   std::vector<int32_t> tab(c->n_pages);
   for (int i = 0; i < c->n_pages; ++i) tab[i] = i;
-  kvr_status st = stage_h2d(m, c->table, tab.data(), tab.size());
-  if (!st) st = stage_h2d(m, c->tokens_d, tokens, n);
+  kvr_status st = stage_add(m, c->table, tab.data(), tab.size());
+  if (!st) st = stage_add(m, c->tokens_d, tokens, n);
   if (st) {
     cudaStreamSynchronize(m->stream);
     kvr_cache_free(c);
@@ -1278,6 +1306,7 @@ kvr_status kvr_cache_load(kvr_model *m, const int32_t *tokens, int32_t n, const 
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   kvr_status st = grow_scratch(m, m->read_scratch, m->read_scratch_bytes,
                                2 * al((size_t)chunk * row_b), "cache load scratch");
+  if (!st) st = stage_flush(m);
   char *kd = (char *)m->read_scratch, *vd = kd + al((size_t)chunk * row_b);
   for (int p0 = 0; !st && p0 < n; p0 += chunk) {
     const int cnt = std::min(chunk, n - p0);
@@ -1318,7 +1347,7 @@ kvr_status kvr_prefill(kvr_model *m, const int32_t *tokens, int32_t n, kvr_cache
     int M = std::min(dm.max_rows, n - c0);
     pos.resize(M);
     for (int i = 0; i < M; ++i) pos[i] = c0 + i;
-    st = stage_h2d(m, m->pos_d, pos.data(), M);
+    st = stage_add(m, m->pos_d, pos.data(), M);
     if (st) break;
     r.M = M;
     r.pos = m->pos_d;
@@ -1375,8 +1404,9 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
   for (int i = 0; i < n_positions; ++i) P[edit_len + i] = positions[i];
   kvr_status st = KVR_OK;
   bool launched = false;
-  if (edit_len) st = stage_h2d(m, c->tokens_d + edit_start, new_tokens, edit_len);
-  if (!st) st = stage_h2d(m, m->pos_d, P.data(), M);
+  const StageScope scope{m};
+  if (edit_len) st = stage_add(m, c->tokens_d + edit_start, new_tokens, edit_len);
+  if (!st) st = stage_add(m, m->pos_d, P.data(), M);
   if (!st) {
     Rows r;
     r.M = M;
@@ -1489,25 +1519,29 @@ kvr_status kvr_repair_batch(kvr_model *m, const kvr_repair_req *reqs, int32_t n_
       if (inP[p]) return fail(KVR_E_RANGE, "request %d: position %d inside an edit", r, p);
       inP[p] = 2;
     }
-    for (int p = 0; p < q.cache->n; ++p)
-      if (inP[p]) {
+    for (int p = 0; p < q.cache->n; ++p) {
+      uint64_t eight;  // most of a document is untouched
+      while (p + 8 <= q.cache->n && (memcpy(&eight, &inP[p], 8), eight == 0)) p += 8;
+      if (p < q.cache->n && inP[p]) {
         P.push_back(p);
         rowdoc.push_back(r);
         max_pos = std::max(max_pos, p);
       }
+    }
   }
   int M = (int)P.size();
   if (M > dm.max_rows) return fail(KVR_E_UNSUPPORTED, "sum |P|=%d above max_rows", M);
   KVR_TRY(use_device(m));
   if (M == 0) return KVR_OK;
   // apply the edits
+  const StageScope scope{m};
   for (int r = 0; r < n_reqs; ++r) {
     const kvr_repair_req &q = reqs[r];
     int tk = 0;
     for (int e = 0; e < q.n_edits; ++e) {
       int s0 = q.edit_start[e], L = q.edit_len[e];
       for (int i = 0; i < L; ++i) q.cache->tokens_h[s0 + i] = q.new_tokens[tk + i];
-      if (L) KVR_TRY(stage_h2d(m, q.cache->tokens_d + s0, q.new_tokens + tk, L));
+      if (L) KVR_TRY(stage_add(m, q.cache->tokens_d + s0, q.new_tokens + tk, L));
       tk += L;
     }
   }
@@ -1530,12 +1564,9 @@ kvr_status kvr_repair_batch(kvr_model *m, const kvr_repair_req *reqs, int32_t n_
   KVR_TRY(grow_scratch(m, m->batch_scratch, m->batch_scratch_bytes, host.size() * 4,
                        "batch tables"));
   char *tab = (char *)m->batch_scratch;
-  kvr_status st = stage_h2d(m, (int32_t *)tab, host.data(), host.size());
-  if (!st) st = stage_h2d(m, m->pos_d, P.data(), M);
-  if (!st) {
-    // rowdoc goes through a second staging round
-    st = stage_h2d(m, m->rowdoc_d, rowdoc.data(), M);
-  }
+  kvr_status st = stage_add(m, (int32_t *)tab, host.data(), host.size());
+  if (!st) st = stage_add(m, m->pos_d, P.data(), M);
+  if (!st) st = stage_add(m, m->rowdoc_d, rowdoc.data(), M);
   if (!st) {
     Rows r;
     r.M = M;
@@ -1566,8 +1597,9 @@ kvr_status kvr_logits(kvr_model *m, const kvr_cache *c, const int32_t *query, in
   KVR_TRY(use_device(m));
   std::vector<int32_t> P(qm);
   for (int i = 0; i < qm; ++i) P[i] = c->n + i;
-  KVR_TRY(stage_h2d(m, c->tokens_d + c->n, query, qm));
-  KVR_TRY(stage_h2d(m, m->pos_d, P.data(), qm));
+  const StageScope scope{m};
+  KVR_TRY(stage_add(m, c->tokens_d + c->n, query, qm));
+  KVR_TRY(stage_add(m, m->pos_d, P.data(), qm));
   Rows r;
   r.M = qm;
   r.pos = m->pos_d;
@@ -1630,12 +1662,13 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
   KVR_TRY(grow_scratch(m, m->sel_scratch, m->sel_scratch_bytes, tok_b + save_b + prob_b,
                        "selector scratch"));
   char *scr = (char *)m->sel_scratch;
+  const StageScope scope{m};
   int32_t *toks = runs_model ? (int32_t *)scr : c->tokens_d;
   kvr_status st = KVR_OK;
   if (runs_model) {
     if (cudaMemcpyAsync(toks, c->tokens_d, (size_t)n * 4, cudaMemcpyDeviceToDevice, m->stream))
       st = fail(KVR_E_CUDA, "token copy");
-    if (!st && edit_len) st = stage_h2d(m, toks + edit_start, new_tokens, edit_len);
+    if (!st && edit_len) st = stage_add(m, toks + edit_start, new_tokens, edit_len);
   }
   int topk_k = K;
   SimpleKeys gen;  // simple policies: keys made inside the top-K kernel
@@ -1671,7 +1704,7 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
       for (int i = 0; i < edit_len; ++i) P[i] = edit_start + i;
       save = scr + tok_b;
       probs = scr + tok_b + save_b;
-      st = stage_h2d(m, m->pos_d, P.data(), edit_len);
+      st = stage_add(m, m->pos_d, P.data(), edit_len);
       if (!st) {
         Rows r;
         r.M = edit_len;
@@ -1681,6 +1714,8 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
         r.tm_kv = c->tm_kv_ok ? &c->tm_kv : nullptr;
         r.max_pos = s_end - 1;
         st = plan_attention(m, r, P.data(), nullptr);
+        const kvr_status sf = stage_flush(m);  // the copies below read r.pos whatever st is
+        if (!st) st = sf;
         launch_rows_copy(r.single, dm.dtype, r.pos, edit_len, 0, dm.L, save, true, m->stream);
         if (!st) st = launch_check(m, 1);
         if (!st) st = embed(m, r);
@@ -1715,7 +1750,8 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
       r.tokens = toks;
       r.single = c->view();
       r.tm_kv = c->tm_kv_ok ? &c->tm_kv : nullptr;
-      if (!st) st = stage_h2d(m, m->pos_d, P.data(), edit_len);
+      if (!st) st = stage_add(m, m->pos_d, P.data(), edit_len);
+      if (!st) st = stage_flush(m);
       if (!st) {
         // refresh the span's layer-0 K/V (saved and restored afterwards)
         r.M = edit_len;
@@ -1734,7 +1770,7 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
         int M = std::min(dm.max_rows, n - c0);
         D.resize(M);
         for (int i = 0; i < M; ++i) D[i] = c0 + i;
-        st = stage_h2d(m, m->pos_d, D.data(), M);
+        st = stage_add(m, m->pos_d, D.data(), M);
         if (st) break;
         r.M = M;
         r.pos = m->pos_d;
@@ -1861,14 +1897,10 @@ static kvr_status answers_logprob(kvr_model *m, int n_ans, const int *first,
   const int rows = (int)target.size();
   KVR_TRY(gemm(m, P_LMHEAD, m->a, m->lm_head, m->tc_lm ? &m->tm_lm : nullptr, nullptr, m->logits,
                rows, dm.V, dm.d, GEMM_EPI_STORE));
-  // answer ids go to the row-document slot
-  KVR_TRY(stage_h2d(m, m->rowdoc_d, target.data(), rows));
-  float *lp = m->scores;  // [rows] scratch
-  launch_row_logprob(m->logits, rows, dm.V, m->rowdoc_d, lp, m->stream);
+  float *h = (float *)m->rb_h;  // page-locked
+  launch_row_logprob(m->logits, rows, dm.V, target.data(), h, m->dev_flag, m->flag_h, m->stream);
   KVR_TRY(launch_check(m, 1));
-  std::vector<float> h(rows);
-  CUDA_TRY(cudaMemcpyAsync(h.data(), lp, (size_t)rows * 4, cudaMemcpyDeviceToHost, m->stream));
-  KVR_TRY(sync_model(m));
+  KVR_TRY(sync_model(m, true));
   for (int k = 0, i = 0; k < n_ans; ++k) {
     double acc = 0.0;
     for (int j = 0; j < ma[k]; ++j) acc += h[i++];
@@ -1886,8 +1918,9 @@ kvr_status kvr_answer_logprob(kvr_model *m, const kvr_cache *c, const int32_t *p
   const int rows = (int)feed.size();
   std::vector<int32_t> P(rows);
   for (int i = 0; i < rows; ++i) P[i] = c->n + i;
-  KVR_TRY(stage_h2d(m, c->tokens_d + c->n, feed.data(), rows));
-  KVR_TRY(stage_h2d(m, m->pos_d, P.data(), rows));
+  const StageScope scope{m};
+  KVR_TRY(stage_add(m, c->tokens_d + c->n, feed.data(), rows));
+  KVR_TRY(stage_add(m, m->pos_d, P.data(), rows));
   Rows r;
   r.M = rows;
   r.pos = m->pos_d;
@@ -1960,7 +1993,8 @@ static kvr_status margin_one_pass(kvr_model *m, const kvr_cache *c,
   const int tail = c->n / KVR_PAGE;  // the page that position n falls into
   for (int i = 0; i < c->n_pages; ++i)
     ((int32_t *)(hb + mb + vb + pb))[i] = i < tail ? i : c->n_pages + i - tail;
-  KVR_TRY(stage_h2d(m, (int32_t *)dev, host.data(), host.size()));
+  const StageScope scope{m};
+  KVR_TRY(stage_add(m, (int32_t *)dev, host.data(), host.size()));
   const size_t page_b = dm.page_elems() * dm.es();
   if (c->n % KVR_PAGE)
     CUDA_TRY(cudaMemcpyAsync((char *)c->pages + c->n_pages * page_b,
@@ -1968,14 +2002,14 @@ static kvr_status margin_one_pass(kvr_model *m, const kvr_cache *c,
                              m->stream));
   std::vector<int32_t> P, doc;
   for (int k = 0; k < 2; ++k) {
-    KVR_TRY(stage_h2d(m, (int32_t *)tokens[k] + c->n, feed[k].data(), feed[k].size()));
+    KVR_TRY(stage_add(m, (int32_t *)tokens[k] + c->n, feed[k].data(), feed[k].size()));
     for (size_t i = 0; i < feed[k].size(); ++i) {
       P.push_back(c->n + (int)i);
       doc.push_back(k);
     }
   }
-  KVR_TRY(stage_h2d(m, m->pos_d, P.data(), P.size()));
-  KVR_TRY(stage_h2d(m, m->rowdoc_d, doc.data(), doc.size()));
+  KVR_TRY(stage_add(m, m->pos_d, P.data(), P.size()));
+  KVR_TRY(stage_add(m, m->rowdoc_d, doc.data(), doc.size()));
   Rows r;
   r.M = (int)P.size();
   r.pos = m->pos_d;

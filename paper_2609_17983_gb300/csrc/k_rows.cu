@@ -91,6 +91,9 @@ __global__ void k_fill_f32(float *dst, float v, size_t n) {
 
 // A CTA per row (d % 4 == 0), four elements per access: with 2-byte loads and
 // 4-byte stores 4096 rows of d = 4096 took 36.6 us (100 MB, 2.7 TB/s).
+// Launched without programmatic dependence: kernels behind it read positions
+// and attention blocks ahead of their own waits, so the pass begins when the
+// kernel that uploads those (k_upload) is over.
 constexpr int EMBED_THREADS = 256;
 template <typename T>
 __global__ void k_embed_rows(const T *embed, const int32_t *tokens,
@@ -98,7 +101,6 @@ __global__ void k_embed_rows(const T *embed, const int32_t *tokens,
                              const int32_t *pos, int d, float *h) {
   TraceScope ts(TK_EMBED);
   pdl_trigger();
-  pdl_wait();
   ts.waited();
   int i = blockIdx.x;
   const int32_t *tk = doc_tokens ? doc_tokens[rowdoc[i]] : tokens;
@@ -106,6 +108,29 @@ __global__ void k_embed_rows(const T *embed, const int32_t *tokens,
 #pragma unroll 4
   for (int c = 4 * threadIdx.x; c < d; c += 4 * EMBED_THREADS)
     st4(h, (size_t)i * d + c, ld4(embed, base + c));
+}
+
+// A call's small arrays (edited tokens, positions, attention blocks, a batch's
+// tables) from page-locked host memory to their places, all in one launch:
+// blockIdx.y is the segment.  Bound by a round trip to the host.  A copy engine takes
+// 3.2 us a segment, one after another, and more to hand over to the kernels:
+// the 68 segments of 64 edits in 16 documents took 230 us, k_upload 2.7.
+constexpr int UP_THREADS = 256, UP_WORDS = 4;
+template <int N>
+struct UploadList {
+  Upload u[N];
+};
+template <int N>
+__global__ void __launch_bounds__(UP_THREADS) k_upload(const __grid_constant__ UploadList<N> l) {
+  const Upload u = l.u[blockIdx.y];
+  const size_t i0 = (size_t)blockIdx.x * (UP_THREADS * UP_WORDS) + threadIdx.x;
+  int32_t v[UP_WORDS];
+#pragma unroll
+  for (int k = 0; k < UP_WORDS; ++k)
+    if (i0 + k * UP_THREADS < u.words) v[k] = u.src[i0 + k * UP_THREADS];
+#pragma unroll
+  for (int k = 0; k < UP_WORDS; ++k)
+    if (i0 + k * UP_THREADS < u.words) u.dst[i0 + k * UP_THREADS] = v[k];
 }
 
 // One block per row (d <= 8192, d % 4 == 0), each load issued before its
@@ -497,11 +522,15 @@ __global__ void k_transplant(KVView dst, KVView src, const int32_t *pos, int n_p
 }
 
 // out[i] = logits[i][target[i]] - logsumexp(logits[i]) for each row, one CTA a
-// row.  One pass: a thread keeps its maximum and the sum of exponentials
+// row; out is page-locked host memory, and the device error flag goes with it
+// (copies of targets, results and flag took 30 us of a pass).  One pass: a thread keeps its maximum and the sum of exponentials
 // against it, LP_VEC float4 loads in flight (V % 4 == 0 keeps every row on a
 // 16-byte boundary; other widths load one at a time).  Two passes of scalar
 // loads by 256 threads took 49 us for 128256 logits.
 constexpr int LP_THREADS = 1024, LP_VEC = 4;
+struct AnswerIds {
+  int32_t id[KVR_QUERY_RESERVE];
+};
 __device__ __forceinline__ void lse_add(float &m, float &s, float m2, float s2) {
   const float mm = fmaxf(m, m2);
   if (mm == -INFINITY) return;  // both empty
@@ -509,7 +538,9 @@ __device__ __forceinline__ void lse_add(float &m, float &s, float m2, float s2) 
   m = mm;
 }
 __global__ void __launch_bounds__(LP_THREADS)
-    k_row_logprob(const float *logits, int V, const int32_t *target, float *out) {
+    k_row_logprob(const float *logits, int V, const __grid_constant__ AnswerIds target, float *out,
+                  const int *flag_in, int *flag_out) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *flag_out = *flag_in;
   const float *x = logits + (size_t)blockIdx.x * V;
   __shared__ float2 red[LP_THREADS / 32];
   float m = -INFINITY, s = 0.f;
@@ -562,7 +593,7 @@ __global__ void __launch_bounds__(LP_THREADS)
     m = red[threadIdx.x].x;
     s = red[threadIdx.x].y;
     fold();
-    if (threadIdx.x == 0) out[blockIdx.x] = x[target[blockIdx.x]] - (m + logf(s));
+    if (threadIdx.x == 0) out[blockIdx.x] = x[target.id[blockIdx.x]] - (m + logf(s));
   }
 }
 
@@ -585,16 +616,30 @@ void launch_fill_f32(float *dst, float v, size_t n, cudaStream_t s) {
   k_fill_f32<<<grid_for(n, 256), 256, 0, s>>>(dst, v, n);
 }
 
+void launch_upload(const Upload *u, int n, cudaStream_t s) {
+  size_t most = 1;
+  for (int i = 0; i < n; ++i) most = std::max(most, u[i].words);
+  const dim3 grid((unsigned)((most + UP_THREADS * UP_WORDS - 1) / (UP_THREADS * UP_WORDS)), n);
+  auto go = [&](auto list) {  // a call's few segments leave the larger list's bytes out of the launch
+    std::copy(u, u + n, list.u);
+    k_upload<<<grid, UP_THREADS, 0, s>>>(list);
+  };
+  if (n <= 8)
+    go(UploadList<8>{});
+  else
+    go(UploadList<UPLOAD_MAX>{});
+}
+
 void launch_embed_rows(const void *embed, int dtype, const int32_t *tokens,
                        const int32_t *const *doc_tokens, const int32_t *rowdoc,
                        const int32_t *pos, int M, int d, float *h, cudaStream_t s) {
   if (M <= 0) return;
   if (dtype == KVR_DTYPE_BF16)
-    launch_pdl(k_embed_rows<__nv_bfloat16>, M, EMBED_THREADS, 0, s, (const __nv_bfloat16 *)embed, tokens,
-               doc_tokens, rowdoc, pos, d, h);
+    k_embed_rows<<<M, EMBED_THREADS, 0, s>>>((const __nv_bfloat16 *)embed, tokens, doc_tokens,
+                                             rowdoc, pos, d, h);
   else
-    launch_pdl(k_embed_rows<float>, M, EMBED_THREADS, 0, s, (const float *)embed, tokens, doc_tokens,
-               rowdoc, pos, d, h);
+    k_embed_rows<<<M, EMBED_THREADS, 0, s>>>((const float *)embed, tokens, doc_tokens, rowdoc, pos,
+                                             d, h);
 }
 
 void launch_rmsnorm(float *h, const float *g, int row0, int M, int d, double eps, void *out,
@@ -720,8 +765,10 @@ void launch_transplant(KVView dst, KVView src, int dtype, const int32_t *pos, in
 }
 
 void launch_row_logprob(const float *logits, int rows, int V, const int32_t *target, float *out,
-                        cudaStream_t s) {
-  if (rows > 0) k_row_logprob<<<rows, LP_THREADS, 0, s>>>(logits, V, target, out);
+                        const int *flag_in, int *flag_out, cudaStream_t s) {
+  AnswerIds t;
+  std::copy(target, target + rows, t.id);
+  k_row_logprob<<<rows, LP_THREADS, 0, s>>>(logits, V, t, out, flag_in, flag_out);
 }
 
 void launch_rows_copy(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,

@@ -200,6 +200,14 @@ struct TcWorkspace {
   long long max_tiles;
 };
 
+// A segment of an upload: words 32-bit words from page-locked host memory to the device.
+struct Upload {
+  int32_t *dst;
+  const int32_t *src;
+  size_t words;
+};
+constexpr int UPLOAD_MAX = 128;  // segments of one launch (3 KB of arguments)
+
 // Accumulated device time of one kernel class.
 struct ProfClass {
   std::string name;
@@ -269,7 +277,8 @@ struct kvr_model {
   int32_t *stage_h = nullptr;
   int32_t *stage_d = nullptr;
   size_t stage_cap = 0;
-  size_t stage_off = 0;           // next free slot (copies take consecutive slots)
+  size_t stage_off = 0;           // next free slot (uploads take consecutive slots)
+  std::vector<kvr::Upload> staged;     // slots filled but not yet uploaded
   cudaEvent_t stage_ev = nullptr;  // recorded after the last staged copy
   int32_t *rb_h = nullptr;         // pinned: selector count, flag, positions (written by the top-K)
   int32_t *flag_h = nullptr;       // pinned readback of the device error flag
@@ -457,6 +466,7 @@ void launch_init_tensor(void *dst, int dtype, bool out_f32, uint64_t tensor_seed
 void launch_fill_f32(float *dst, float v, size_t n, cudaStream_t s);
 
 // ---- kernels: row ops ----
+void launch_upload(const Upload *u, int n, cudaStream_t s);
 void launch_embed_rows(const void *embed, int dtype, const int32_t *tokens,
                        const int32_t *const *doc_tokens, const int32_t *rowdoc,
                        const int32_t *pos, int M, int d, float *h, cudaStream_t s);
@@ -489,8 +499,10 @@ void launch_rows_copy(KVView v, int dtype, const int32_t *pos, int n_pos, int l0
                       void *buf, bool to_buf, cudaStream_t s);
 void launch_transplant(KVView dst, KVView src, int dtype, const int32_t *pos, int n_pos,
                        int32_t *tok_dst, const int32_t *tok_src, cudaStream_t s);
+// 1 to KVR_QUERY_RESERVE rows; target: host memory; out and flag_out: page-locked
+// host memory.
 void launch_row_logprob(const float *logits, int rows, int V, const int32_t *target, float *out,
-                        cudaStream_t s);
+                        const int *flag_in, int *flag_out, cudaStream_t s);
 
 // ---- kernels: GEMM  Y[M][N] (+)= X[M][K] W[N][K]^T (+ bias) ----
 struct GemmArgs {
