@@ -372,8 +372,8 @@ kvr_status embed(kvr_model *m, const Rows &r) {
 // tiles a deferred GEMM left pending in h.
 kvr_status norm(kvr_model *m, const float *g, int M, int row0 = 0) {
   Prof pr(m, P_NORM, (int64_t)M * m->dims.d * 4);
-  launch_rmsnorm(m->h, g, row0, M, m->dims.d, m->dims.eps, m->a, m->dims.dtype, m->stream,
-                 &m->pending);
+  launch_rmsnorm(m->h, g, row0, M, m->dims.d, m->dims.eps, m->a, m->dims.dtype, m->num_sms,
+                 m->stream, &m->pending);
   m->pending = SplitView{};
   return launch_check(m, 1);
 }
@@ -1612,8 +1612,8 @@ kvr_status kvr_logits(kvr_model *m, const kvr_cache *c, const int32_t *query, in
   // final RMSNorm of the last row, lm_head
   {
     Prof pr(m, P_NORM, (int64_t)dm.d * 4);
-    launch_rmsnorm(m->h, m->final_norm, qm - 1, 1, dm.d, dm.eps, m->a, dm.dtype, m->stream,
-                   &m->pending);
+    launch_rmsnorm(m->h, m->final_norm, qm - 1, 1, dm.d, dm.eps, m->a, dm.dtype, m->num_sms,
+                   m->stream, &m->pending);
     m->pending = SplitView{};
     KVR_TRY(launch_check(m, 1));
   }
@@ -1888,8 +1888,8 @@ static kvr_status answers_logprob(kvr_model *m, int n_ans, const int *first,
   for (int k = 0; k < n_ans; ++k) {
     Prof pr(m, P_NORM, (int64_t)ma[k] * dm.d * 4);
     launch_rmsnorm(m->h, m->final_norm, first[k], ma[k], dm.d, dm.eps,
-                   (char *)m->a + target.size() * dm.d * dm.es(), dm.dtype, m->stream,
-                   &m->pending);
+                   (char *)m->a + target.size() * dm.d * dm.es(), dm.dtype, m->num_sms,
+                   m->stream, &m->pending);
     KVR_TRY(launch_check(m, 1));
     target.insert(target.end(), answer[k], answer[k] + ma[k]);
   }

@@ -203,6 +203,59 @@ __global__ void __launch_bounds__(TPB, TPB == NORM_THREADS_WIDE && NV <= 4 ? 4 :
   }
 }
 
+// Many complete rows: the CTAs that fit (four an SM, NV <= 4) stay and take rows
+// in turn, the next row's loads in flight while this one is reduced and written.
+// Bound by HBM: 4096 rows of d = 4096 move 100 MB.  A CTA per row waited for
+// its loads, then for the sum, and left: 21 us, this 14.
+template <typename T, int NV>
+__global__ void __launch_bounds__(NORM_THREADS_WIDE, 4)
+    k_rmsnorm_rows(const float *h, const float *g, int row0, int M, int d, float eps, T *out) {
+  constexpr int TPB = NORM_THREADS_WIDE;
+  __shared__ float red[2][TPB / 32];
+  TraceScope ts(TK_NORM);
+  pdl_trigger();
+  const int nq = d >> 2;
+  pdl_wait();
+  ts.waited();
+  float4 nx[NV];
+  auto fetch = [&](int i) {
+    const float4 *x = (const float4 *)(h + (size_t)(row0 + i) * d);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int q = k * TPB + threadIdx.x;
+      nx[k] = i < M && q < nq ? x[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  fetch(blockIdx.x);
+  for (int i = blockIdx.x, b = 0; i < M; i += gridDim.x, b ^= 1) {
+    float4 v[NV];
+    float ss = 0.f;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      v[k] = nx[k];
+      ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
+    }
+    fetch(i + gridDim.x);
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    // two sets of sums: a warp writes a set again only when all have read it
+    if ((threadIdx.x & 31) == 0) red[b][threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < TPB / 32; ++w) tot += red[b][w];
+    const float r = 1.0f / sqrtf(tot / (float)d + eps);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int q = k * TPB + threadIdx.x;
+      if (q < nq) {
+        const float4 w = __ldg((const float4 *)g + q);
+        st4(out, (size_t)i * d + 4 * q,
+            make_float4(v[k].x * r * w.x, v[k].y * r * w.y, v[k].z * r * w.z, v[k].w * r * w.w));
+      }
+    }
+  }
+}
+
 // RoPE of the q and k heads of the projection at each row's position: q ->
 // q_out fp32 (if given) and qb_out, k and v -> cache (if write_kv) and rows_out
 // (if given).  With a split view the projection is completed from the GEMM's
@@ -643,15 +696,31 @@ void launch_embed_rows(const void *embed, int dtype, const int32_t *tokens,
 }
 
 void launch_rmsnorm(float *h, const float *g, int row0, int M, int d, double eps, void *out,
-                    int out_dtype, cudaStream_t s, const SplitView *sv) {
+                    int out_dtype, int num_sms, cudaStream_t s, const SplitView *sv) {
   if (M <= 0) return;
   const SplitView v = sv ? *sv : SplitView{};
   // A pass of a few rows is latency-bound: 1024 threads, each with one
-  // float4 in flight.  Hundreds of rows (prefill) run in waves: 256 threads a
-  // row, several rows per SM at once.
+  // float4 in flight.  Hundreds of rows (prefill): 256 threads a row, several
+  // rows per SM at once, staying on the SM unless split tiles are to be added or
+  // a row does not fit 64 registers a thread twice.
   if (M > 256 && d <= 4 * 8 * NORM_THREADS_WIDE) {
     constexpr int W = NORM_THREADS_WIDE;
     const int nv = (d + 4 * W - 1) / (4 * W);
+    if (!v.ws && nv <= 4) {
+      const int grid = std::min(M, 4 * num_sms);
+      if (out_dtype == KVR_DTYPE_BF16) {
+        auto k = nv <= 1 ? k_rmsnorm_rows<__nv_bfloat16, 1>
+                 : nv <= 2 ? k_rmsnorm_rows<__nv_bfloat16, 2>
+                           : k_rmsnorm_rows<__nv_bfloat16, 4>;
+        launch_pdl(k, grid, W, 0, s, (const float *)h, g, row0, M, d, (float)eps, (__nv_bfloat16 *)out);
+      } else {
+        auto k = nv <= 1 ? k_rmsnorm_rows<float, 1>
+                 : nv <= 2 ? k_rmsnorm_rows<float, 2>
+                           : k_rmsnorm_rows<float, 4>;
+        launch_pdl(k, grid, W, 0, s, (const float *)h, g, row0, M, d, (float)eps, (float *)out);
+      }
+      return;
+    }
     if (out_dtype == KVR_DTYPE_BF16) {
       auto k = nv <= 1 ? k_rmsnorm<__nv_bfloat16, 1, W>
                : nv <= 2 ? k_rmsnorm<__nv_bfloat16, 2, W>

@@ -473,7 +473,7 @@ void launch_embed_rows(const void *embed, int dtype, const int32_t *tokens,
 // Rows row0 .. row0+M-1 of h; out row i is h row row0 + i.  With a split
 // view (rows indexed from h's base), the completed rows are written back to h.
 void launch_rmsnorm(float *h, const float *g, int row0, int M, int d, double eps, void *out,
-                    int out_dtype, cudaStream_t s, const SplitView *sv = nullptr);
+                    int out_dtype, int num_sms, cudaStream_t s, const SplitView *sv = nullptr);
 // q_out: fp32 rotated q; qb_out (optional): bf16 rotated q times qscale;
 // rows_out (optional, with write_kv): the K/V rows as written into the cache,
 // K then V, each [M][L][G][dh] in the cache dtype.

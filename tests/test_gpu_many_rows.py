@@ -164,3 +164,23 @@ def test_read_into_page_locked_memory(rows):
         assert all(np.array_equal(o, w) for o, w in zip(out, want))
         assert all(not b[:off].any() and not b[off + count:].any() for b in buf)
     model.close()
+
+
+# rows 1, 2 and 3 to a CTA, and a last CTA with one fewer; a float4, two and
+# four a thread, the last ones ragged.  Layer 0's V is W_v times the norm of the
+# embedding rows, here in float64; the bound is that of two fp32 sums of d terms
+# relative to the largest entry (absolute sums stay below four of them).
+@pytest.mark.parametrize("d", [256, 1280, 3584])
+def test_norm_of_many_rows(d):
+    cfg = synth.preset("tiny", n_layers=2, d_model=d, ffn=256)
+    W = synth.weights(cfg, 0)
+    model = kv.Model(cfg, None, seed=0, max_context=2048, max_rows=2048)
+    for n in (257, 609, 1217, 1823):
+        doc = synth.document(n, n, cfg["vocab"])
+        x = W["embed"][doc].astype(np.float64)
+        x /= np.sqrt((x * x).mean(axis=1, keepdims=True) + cfg["rms_eps"])
+        want = (x * W["layers"][0]["attn_norm"]) @ W["layers"][0]["wv"].astype(np.float64).T
+        _, v = model.prefill(doc).read(np.arange(n))
+        err = np.abs(v[:, 0].reshape(n, -1) - want).max()
+        assert err <= 8 * d * 2.0 ** -24 * np.abs(want).max(), n
+    model.close()
