@@ -121,13 +121,27 @@ kvr_status stage_flush(kvr_model *m) {
   return KVR_OK;
 }
 
+// Room for one more segment.  Those of a launch run in no order: one that
+// overwrites another goes behind it.
+kvr_status stage_room(kvr_model *m, const int32_t *dst, size_t count) {
+  bool flush = m->staged.size() == UPLOAD_MAX;
+  for (const Upload &u : m->staged) flush = flush || (dst < u.dst + u.words && u.dst < dst + count);
+  return flush ? stage_flush(m) : KVR_OK;
+}
+
+// Device memory that no staged segment writes, copied by the same launch.
+kvr_status stage_copy(kvr_model *m, int32_t *dst, const int32_t *src, size_t count) {
+  if (count == 0) return KVR_OK;
+  KVR_TRY(stage_room(m, dst, count));
+  m->staged.push_back({dst, src, count});
+  return KVR_OK;
+}
+
 kvr_status stage_add(kvr_model *m, int32_t *dst, const int32_t *src, size_t count) {
   if (count == 0) return KVR_OK;
   if (count > m->stage_cap) return fail(KVR_E_UNSUPPORTED, "staging overflow (%zu)", count);
-  // the segments of a launch run in no order: one that overwrites another goes behind it
-  bool flush = m->staged.size() == UPLOAD_MAX || m->stage_off + count > m->stage_cap;
-  for (const Upload &u : m->staged) flush = flush || (dst < u.dst + u.words && u.dst < dst + count);
-  if (flush) KVR_TRY(stage_flush(m));
+  KVR_TRY(stage_room(m, dst, count));
+  if (m->stage_off + count > m->stage_cap) KVR_TRY(stage_flush(m));
   if (m->stage_off + count > m->stage_cap) {
     CUDA_TRY(cudaEventSynchronize(m->stage_ev));
     m->stage_off = 0;
@@ -1665,9 +1679,9 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
   const StageScope scope{m};
   int32_t *toks = runs_model ? (int32_t *)scr : c->tokens_d;
   kvr_status st = KVR_OK;
-  if (runs_model) {
-    if (cudaMemcpyAsync(toks, c->tokens_d, (size_t)n * 4, cudaMemcpyDeviceToDevice, m->stream))
-      st = fail(KVR_E_CUDA, "token copy");
+  if (runs_model) {  // the edited context: the document's tokens around the span's
+    st = stage_copy(m, toks, c->tokens_d, edit_start);
+    if (!st) st = stage_copy(m, toks + s_end, c->tokens_d + s_end, n - s_end);
     if (!st && edit_len) st = stage_add(m, toks + edit_start, new_tokens, edit_len);
   }
   int topk_k = K;
@@ -1997,9 +2011,8 @@ static kvr_status margin_one_pass(kvr_model *m, const kvr_cache *c,
   KVR_TRY(stage_add(m, (int32_t *)dev, host.data(), host.size()));
   const size_t page_b = dm.page_elems() * dm.es();
   if (c->n % KVR_PAGE)
-    CUDA_TRY(cudaMemcpyAsync((char *)c->pages + c->n_pages * page_b,
-                             (char *)c->pages + tail * page_b, page_b, cudaMemcpyDeviceToDevice,
-                             m->stream));
+    KVR_TRY(stage_copy(m, (int32_t *)((char *)c->pages + c->n_pages * page_b),
+                       (const int32_t *)((const char *)c->pages + tail * page_b), page_b / 4));
   std::vector<int32_t> P, doc;
   for (int k = 0; k < 2; ++k) {
     KVR_TRY(stage_add(m, (int32_t *)tokens[k] + c->n, feed[k].data(), feed[k].size()));

@@ -111,8 +111,9 @@ __global__ void k_embed_rows(const T *embed, const int32_t *tokens,
 }
 
 // A call's small arrays (edited tokens, positions, attention blocks, a batch's
-// tables) from page-locked host memory to their places, all in one launch:
-// blockIdx.y is the segment.  Bound by a round trip to the host.  A copy engine takes
+// tables) from page-locked host memory, and what goes with them from device
+// memory, to their places, all in one launch: blockIdx.y is the segment.
+// Bound by a round trip to the host.  A copy engine takes
 // 3.2 us a segment, one after another, and more to hand over to the kernels:
 // the 68 segments of 64 edits in 16 documents took 230 us, k_upload 2.7.
 constexpr int UP_THREADS = 256, UP_WORDS = 4;

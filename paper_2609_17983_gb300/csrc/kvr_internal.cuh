@@ -200,7 +200,7 @@ struct TcWorkspace {
   long long max_tiles;
 };
 
-// A segment of an upload: words 32-bit words from page-locked host memory to the device.
+// A segment of an upload: 32-bit words from page-locked host (or device) memory to the device.
 struct Upload {
   int32_t *dst;
   const int32_t *src;
@@ -278,7 +278,7 @@ struct kvr_model {
   int32_t *stage_d = nullptr;
   size_t stage_cap = 0;
   size_t stage_off = 0;           // next free slot (uploads take consecutive slots)
-  std::vector<kvr::Upload> staged;     // slots filled but not yet uploaded
+  std::vector<kvr::Upload> staged;     // slots filled (and copies asked for) but not yet uploaded
   cudaEvent_t stage_ev = nullptr;  // recorded after the last staged copy
   int32_t *rb_h = nullptr;         // pinned: selector count, flag, positions (written by the top-K)
   int32_t *flag_h = nullptr;       // pinned readback of the device error flag
