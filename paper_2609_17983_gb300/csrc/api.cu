@@ -1739,7 +1739,7 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
           if (!st) {
             Prof pr(m, P_SELECT, 0);
             const int k = launch_attn_select_scores(edit_len, dm, l, r.single, s_end, n, probs,
-                                                    m->keys, m->stream);
+                                                    m->keys, m->num_sms, m->stream);
             st = launch_check(m, k);
           }
           // the scores need the queries of every layer; no K/V follow the last

@@ -249,30 +249,34 @@ __global__ void __launch_bounds__(TOPK_THREADS)
 // for twenty.  The queries of kv group g are the span rows' heads hh with
 // hh / (H/G) == g; within the group a query is ql = r * (H/G) + (hh mod H/G),
 // globally qg = g * S * (H/G) + ql.  blockIdx.z is layer-major: query tile
-// z % n_qtiles of layer layer0 + z / n_qtiles, whose arrays lie NQ apart.  A CTA of k_attn_select_logits takes SEL_KC pool
-// keys and SEL_QT queries of one group: the keys are read once into shared
-// memory and serve every query of the tile (so a group's key rows leave L2
-// once per query tile, not once per query).  It stores the scaled logits,
-// logit[qg * c + (j - s_end)], and per query the chunk's max and sum of
-// exp(logit - max); the last CTA of (group, query tile) to finish folds the
+// z % n_qtiles of layer layer0 + z / n_qtiles, whose arrays lie NQ apart.  A CTA
+// of k_attn_select_logits takes SEL_QT queries of one group and some chunks of
+// SEL_KC pool keys, the next chunk's keys in flight while one is computed: a
+// chunk's keys are read once into shared memory and serve every query of the
+// tile (so a group's key rows leave L2 once per query tile, not once per query).
+// It stores the scaled logits, logit[qg * stride + (j - s_end)], and per query
+// the chunk's max and sum of exp(logit - max); the last CTA of (group, query tile) to finish folds the
 // chunk statistics into the pool softmax's max and 1 / sum.  Arrival is an
 // atomic count with no waiting: every other CTA just exits.  The contraction
 // runs on mma.sync for bf16 caches and on FFMA micro-tiles for fp32 caches.
+// Eight layers of 8 span rows and 2,492 keys: 69 us for both kernels with a CTA
+// per chunk, run-time head sizes and scalar fragment loads, 45 now; mma.sync
+// itself, twice for the split queries, takes 14 of it and the 41 MB of keys 6.
 constexpr int SEL_KC = 64, SEL_QT = 32, SEL_THREADS = 128;
 constexpr int SEL_KG = SEL_KC / 4;   // fp32 path: key groups of 4 (a thread: 4 queries x 4 keys)
 constexpr int SEL_LTS = SEL_KC + 4;  // logits tile row stride (floats)
-constexpr int SEL_DH_MAX = 128;      // head_dim is 64 or 128 (checked at model creation)
 constexpr int SEL_FOLD = 16;         // chunk statistics in flight per thread in the fold
 static_assert(SEL_KG * (SEL_QT / 4) == SEL_THREADS, "one 4x4 micro-tile per thread");
 
 struct SelWs {
-  float *logit;  // [layers][S*H][c]
+  float *logit;  // [layers][S*H][sel_stride(c)]
   float2 *ml;    // [layers][S*H][n_chunks] chunk (max, sum of exp)
   float2 *mz;    // [layers][S*H] pool (max, 1 / sum of exp)
   int *cnt;      // [layers][G][n_qtiles] arrivals
 };
 
 __host__ __device__ inline int sel_chunks(int c) { return (c + SEL_KC - 1) / SEL_KC; }
+inline int sel_stride(int c) { return (c + 3) / 4 * 4; }  // logit rows on 16-byte boundaries
 
 // (m, z) <- the (max, sum of exp) of the union of two sets, either possibly
 // empty (m = -inf, z = 0).  Symmetric in its operands, bit for bit.
@@ -299,79 +303,105 @@ __device__ __forceinline__ void sel_mma_bf16(float *d, uint32_t a0, uint32_t a1,
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <typename T>
-__global__ void __launch_bounds__(SEL_THREADS)
-    k_attn_select_logits(const float *q, int S, int H, int G, int dh, int layer0, int n_qt,
-                         KVView v, int s_end, int c, float scale, SelWs ws) {
+// Four 8 x 8 matrices of 16-bit elements, lane l's address the row l % 8 of matrix l / 8.
+__device__ __forceinline__ void sel_ldmatrix(uint32_t *r, const __nv_bfloat16 *row) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(row)));
+}
+
+template <typename T, int DH>
+__global__ void __launch_bounds__(SEL_THREADS, sizeof(T) == 2 ? 6 : 4)
+    k_attn_select_logits(const float *q, int S, int H, int G, int layer0, int n_qt, KVView v, int s_end, int c, int cs, float scale, SelWs ws) {
+  constexpr bool BF16 = sizeof(T) == 2;
   TraceScope ts(TK_SELECT);
   pdl_trigger();
-  const int chunk = blockIdx.x, g = blockIdx.y, nch = gridDim.x;
+  const int g = blockIdx.y, nch = sel_chunks(c);
   const int li = blockIdx.z / n_qt, qt = blockIdx.z - li * n_qt, layer = layer0 + li;
   const int hpg = H / G, Nq = S * hpg;
   {  // this layer's queries and arrays
     const size_t NQ = (size_t)S * H;
-    q += li * NQ * dh;
-    ws.logit += li * NQ * c;
+    q += li * NQ * DH;
+    ws.logit += li * NQ * cs;
     ws.ml += li * NQ * nch;
     ws.mz += li * NQ;
     ws.cnt += (size_t)li * G * n_qt;
   }
-  const int t0 = chunk * SEL_KC, q0 = qt * SEL_QT;
-  const int nk = min(SEL_KC, c - t0), nq = min(SEL_QT, Nq - q0);
+  const int q0 = qt * SEL_QT, nq = min(SEL_QT, Nq - q0);
   const int tid = threadIdx.x;
   const size_t qg0 = (size_t)g * Nq + q0;
   extern __shared__ float4 sel_smem[];
-  float *lt;  // [SEL_QT][SEL_LTS] logits, over the keys once they are consumed
-  int *last;  // arrival flag, over the queries once they are consumed
-  if constexpr (sizeof(T) == 2) {
-    // bf16 keys: tensor cores (mma.sync m16n8k16, fp32 accumulate).  Each
-    // query is split into two bf16 parts, q = q_hi + q_lo with q_lo the
-    // rounding remainder, and logit = q_hi . k + q_lo . k: about 16 bits of
-    // q's mantissa, the keys exact.  Rows are d-contiguous with a stride of
-    // dh + 8 elements (4 mod 32 words), so a fragment load's 8 rows x 4
-    // lanes fall on 32 banks.
-    const int RS = dh + 8;
-    __nv_bfloat16 *qh = (__nv_bfloat16 *)sel_smem;  // [SEL_QT][RS]
-    __nv_bfloat16 *qo = qh + SEL_QT * RS;           // [SEL_QT][RS] the remainders
-    __nv_bfloat16 *ks = qo + SEL_QT * RS;           // [SEL_KC][RS]
-    lt = (float *)ks;
-    last = (int *)qh;
-    // the pool's stale keys: no kernel of the pass writes them, so they are
-    // read before the wait on the predecessor; a thread issues all its loads
-    // (page lookups, then rows) before it uses the first
-    constexpr int KLD = SEL_KC * (SEL_DH_MAX / 8) / SEL_THREADS;
-    const __nv_bfloat16 *kc = (const __nv_bfloat16 *)v.pages;
-    const int L = dh / 8;  // 16-byte pieces per key row
-    uint4 kx[KLD];
+  // bf16 keys: tensor cores (mma.sync m16n8k16, fp32 accumulate).  Each query is
+  // split into two bf16 parts, q = q_hi + q_lo with q_lo the rounding
+  // remainder, and logit = q_hi . k + q_lo . k: about 16 bits of q's mantissa,
+  // the keys exact.  Rows are d-contiguous with a stride of dh + 8 elements (4
+  // mod 32 words), so a fragment load's 8 rows x 4 lanes fall on 32 banks.
+  // fp32 keys: FFMA micro-tiles.  Both operands transposed, d-major: the thread
+  // of micro-tile (queries 4qg.., keys 4kg..) reads one float4 of each per d.
+  constexpr int RS = DH + 8;
+  __nv_bfloat16 *qh = (__nv_bfloat16 *)sel_smem;  // bf16: [SEL_QT][RS]
+  __nv_bfloat16 *qo = qh + SEL_QT * RS;           // [SEL_QT][RS] the remainders
+  __nv_bfloat16 *ks = qo + SEL_QT * RS;           // [SEL_KC][RS]
+  float *qT = (float *)sel_smem;                  // fp32: [DH][SEL_QT]
+  float *kT = qT + DH * SEL_QT;                   // [DH][SEL_KC]
+  float *lt = BF16 ? (float *)ks : kT;  // [SEL_QT][SEL_LTS] logits, over the keys once consumed
+  int *last = (int *)sel_smem;          // arrival flag, over the queries at the end
+
+  // A chunk's stale keys (no kernel of the pass writes them, so the first
+  // chunk's are read before the wait on the predecessor): all loads (page
+  // lookups, then rows) are issued before the first is used.
+  constexpr int EPV = 16 / (int)sizeof(T);  // elements per 16-byte load
+  constexpr int L = DH / EPV;               // 16-byte pieces per key row
+  constexpr int KLD = SEL_KC * L / SEL_THREADS;
+  uint4 kx[KLD];
+  // lanes: along a row (bf16), or consecutive keys (fp32, stored transposed)
+  auto key = [&](int i) { return BF16 ? i / L : i % SEL_KC; };
+  auto piece = [&](int i) { return BF16 ? i % L : i / SEL_KC; };
+  auto load_keys = [&](int t0) {
+    const T *kc = (const T *)v.pages;
 #pragma unroll
     for (int u = 0; u < KLD; ++u) {
-      const int i = tid + u * SEL_THREADS, kk = i / L, sub = i % L;
+      const int i = tid + u * SEL_THREADS, kk = key(i), sub = piece(i);
       kx[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (kk < nk) kx[u] = *(const uint4 *)(kc + v.offset(layer, 0, g, s_end + t0 + kk) + sub * 8);
+      if (kk < min(SEL_KC, c - t0))
+        kx[u] = *(const uint4 *)(kc + v.offset(layer, 0, g, s_end + t0 + kk) + sub * EPV);
     }
+  };
+  auto store_keys = [&]() {
 #pragma unroll
     for (int u = 0; u < KLD; ++u) {
-      const int i = tid + u * SEL_THREADS, kk = i / L, sub = i % L;
-      if (kk < SEL_KC) *(uint4 *)(ks + kk * RS + sub * 8) = kx[u];  // rows of 16-byte multiples
+      const int i = tid + u * SEL_THREADS, kk = key(i), sub = piece(i);
+      if constexpr (BF16) {
+        *(uint4 *)(ks + kk * RS + sub * 8) = kx[u];  // rows of 16-byte multiples
+      } else {
+        const float *f = (const float *)&kx[u];
+#pragma unroll
+        for (int e = 0; e < EPV; ++e) kT[(sub * EPV + e) * SEL_KC + kk] = f[e];
+      }
     }
-    pdl_wait();  // the queries come from the RoPE kernel just before
-    ts.waited();
-    constexpr int QLD = SEL_QT * (SEL_DH_MAX / 4) / SEL_THREADS;
-    const int D4 = dh / 4;
+  };
+  load_keys(blockIdx.x * SEL_KC);
+  pdl_wait();  // the queries come from the RoPE kernels before
+  ts.waited();
+  {
+    constexpr int D4 = DH / 4, QLD = SEL_QT * D4 / SEL_THREADS;
+    // lanes: along a row (bf16), or consecutive queries (fp32)
+    auto query = [&](int i) { return BF16 ? i / D4 : i % SEL_QT; };
+    auto quad = [&](int i) { return BF16 ? i % D4 : i / SEL_QT; };
     float4 qx[QLD];
 #pragma unroll
     for (int u = 0; u < QLD; ++u) {
-      const int i = tid + u * SEL_THREADS, ql = i / D4, d4 = i % D4;
+      const int i = tid + u * SEL_THREADS, ql = query(i), d4 = quad(i);
       qx[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (ql < nq) {
         const int qq = q0 + ql, r = qq / hpg, hh = g * hpg + qq % hpg;
-        qx[u] = *(const float4 *)(q + ((size_t)r * H + hh) * dh + 4 * d4);
+        qx[u] = *(const float4 *)(q + ((size_t)r * H + hh) * DH + 4 * d4);
       }
     }
 #pragma unroll
     for (int u = 0; u < QLD; ++u) {
-      const int i = tid + u * SEL_THREADS, ql = i / D4, d4 = i % D4;
-      if (ql < SEL_QT) {
+      const int i = tid + u * SEL_THREADS, ql = query(i), d4 = quad(i);
+      if constexpr (BF16) {
         const float2 x01 = make_float2(qx[u].x, qx[u].y), x23 = make_float2(qx[u].z, qx[u].w);
         const __nv_bfloat162 h01 = __float22bfloat162_rn(x01), h23 = __float22bfloat162_rn(x23);
         const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
@@ -379,147 +409,100 @@ __global__ void __launch_bounds__(SEL_THREADS)
         const __nv_bfloat162 l23 = __floats2bfloat162_rn(x23.x - f23.x, x23.y - f23.y);
         *(uint2 *)(qh + ql * RS + 4 * d4) = make_uint2(bf2_bits(h01), bf2_bits(h23));
         *(uint2 *)(qo + ql * RS + 4 * d4) = make_uint2(bf2_bits(l01), bf2_bits(l23));
-      }
-    }
-    __syncthreads();
-    if (tid == 0) trace_mark(0);  // keys and queries staged
-    // warp w: keys 16w .. 16w + 15 (two n-tiles of 8), all SEL_QT queries
-    // (two m-tiles of 16); lane: group gr = lane / 4, pair column gc
-    const int warp = tid >> 5, lane = tid & 31, gr = lane >> 2, gc = (lane & 3) * 2;
-    static_assert(SEL_QT == 32 && SEL_KC == 16 * (SEL_THREADS / 32), "warp tiling");
-    float acc[2][2][4];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
-    for (int k0 = 0; k0 < dh; k0 += 16) {
-      uint32_t b[2][2];
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const __nv_bfloat16 *kr = ks + (16 * warp + 8 * nt + gr) * RS + k0 + gc;
-        b[nt][0] = *(const uint32_t *)kr;
-        b[nt][1] = *(const uint32_t *)(kr + 8);
-      }
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int part = 0; part < 2; ++part) {
-          const __nv_bfloat16 *qr = (part ? qo : qh) + (16 * mt + gr) * RS + k0 + gc;
-          const uint32_t a0 = *(const uint32_t *)qr, a1 = *(const uint32_t *)(qr + 8 * RS);
-          const uint32_t a2 = *(const uint32_t *)(qr + 8), a3 = *(const uint32_t *)(qr + 8 * RS + 8);
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt) sel_mma_bf16(acc[mt][nt], a0, a1, a2, a3, b[nt][0], b[nt][1]);
-        }
-    }
-    __syncthreads();  // keys consumed: lt reuses their space
-    if (tid == 0) trace_mark(1);  // logits computed
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int ql = 16 * mt + gr + (e >> 1) * 8, kk = 16 * warp + 8 * nt + gc + (e & 1);
-          const float l = acc[mt][nt][e] * scale;
-          lt[ql * SEL_LTS + kk] = kk < nk ? l : -INFINITY;
-          if (kk < nk && ql < nq) ws.logit[(qg0 + ql) * c + t0 + kk] = l;
-        }
-  } else {
-    // fp32 keys: FFMA micro-tiles.  Both operands transposed, d-major: the
-    // thread of micro-tile (queries 4qg.., keys 4kg..) reads one float4 of
-    // each per d
-    float *qT = (float *)sel_smem;   // [dh][SEL_QT]
-    float *kT = qT + dh * SEL_QT;    // [dh][SEL_KC]
-    lt = kT;
-    last = (int *)qT;
-    // the pool's stale keys: no kernel of the pass writes them, so they are
-    // read before the wait on the predecessor; a thread issues all its loads
-    // (page lookups, then rows) before it uses the first
-    constexpr int EPV = 16 / (int)sizeof(T);  // elements per 16-byte load
-    constexpr int KLD = SEL_KC * (SEL_DH_MAX / EPV) / SEL_THREADS;
-    const T *kc = (const T *)v.pages;
-    const int L = dh / EPV;
-    uint4 kx[KLD];
-#pragma unroll
-    for (int u = 0; u < KLD; ++u) {
-      const int i = tid + u * SEL_THREADS, kk = i % SEL_KC, sub = i / SEL_KC;
-      kx[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (kk < nk && sub < L)
-        kx[u] = *(const uint4 *)(kc + v.offset(layer, 0, g, s_end + t0 + kk) + sub * EPV);
-    }
-#pragma unroll
-    for (int u = 0; u < KLD; ++u) {
-      const int i = tid + u * SEL_THREADS, kk = i % SEL_KC, sub = i / SEL_KC;
-      if (sub < L) {
-        const float *f = (const float *)&kx[u];
-#pragma unroll
-        for (int e = 0; e < EPV; ++e) kT[(sub * EPV + e) * SEL_KC + kk] = f[e];  // lanes: consecutive keys
-      }
-    }
-    pdl_wait();  // the queries come from the RoPE kernel just before
-    ts.waited();
-    constexpr int QLD = SEL_QT * (SEL_DH_MAX / 4) / SEL_THREADS;
-    const int D4 = dh / 4;
-    float4 qx[QLD];
-#pragma unroll
-    for (int u = 0; u < QLD; ++u) {
-      const int i = tid + u * SEL_THREADS, ql = i % SEL_QT, d4 = i / SEL_QT;
-      qx[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (ql < nq && d4 < D4) {
-        const int qq = q0 + ql, r = qq / hpg, hh = g * hpg + qq % hpg;
-        qx[u] = *(const float4 *)(q + ((size_t)r * H + hh) * dh + 4 * d4);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < QLD; ++u) {
-      const int i = tid + u * SEL_THREADS, ql = i % SEL_QT, d4 = i / SEL_QT;
-      if (d4 < D4) {
-        float *dst = qT + 4 * d4 * SEL_QT + ql;  // lanes: consecutive queries
+      } else {
+        float *dst = qT + 4 * d4 * SEL_QT + ql;
         dst[0] = qx[u].x;
         dst[SEL_QT] = qx[u].y;
         dst[2 * SEL_QT] = qx[u].z;
         dst[3 * SEL_QT] = qx[u].w;
       }
     }
+  }
+  const int ql = tid >> 2, o = tid & 3;  // of the statistics: 4 threads per query
+  for (int chunk = blockIdx.x; chunk < nch; chunk += gridDim.x) {
+    const int t0 = chunk * SEL_KC, nk = min(SEL_KC, c - t0);
+    store_keys();
     __syncthreads();
     if (tid == 0) trace_mark(0);  // keys and queries staged
-    const int kg = tid % SEL_KG, qg = tid / SEL_KG;
-    float acc[4][4];
+    // the next chunk's keys travel while this one is computed
+    if (chunk + (int)gridDim.x < nch) load_keys((chunk + gridDim.x) * SEL_KC);
+    if constexpr (BF16) {
+      // warp w: keys 16w .. 16w + 15 (two n-tiles of 8), all SEL_QT queries
+      // (two m-tiles of 16); lane: group gr = lane / 4, pair column gc
+      const int warp = tid >> 5, lane = tid & 31, gr = lane >> 2, gc = (lane & 3) * 2;
+      static_assert(SEL_QT == 32 && SEL_KC == 16 * (SEL_THREADS / 32), "warp tiling");
+      float acc[2][2][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+      for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
-    for (int d = 0; d < dh; ++d) {
-      const float4 a = *(const float4 *)(qT + d * SEL_QT + 4 * qg);
-      const float4 b = *(const float4 *)(kT + d * SEL_KC + 4 * kg);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
+      const __nv_bfloat16 *ka = ks + (16 * warp + 8 * (lane >> 4) + (lane & 7)) * RS + (lane & 8);
+      const __nv_bfloat16 *qa = qh + (lane & 15) * RS + (lane >> 4) * 8;
+#pragma unroll
+      for (int k0 = 0; k0 < DH; k0 += 16) {
+        uint32_t b[4];
+        sel_ldmatrix(b, ka + k0);  // both n-tiles, d k0 .. +7 and +8 .. +15
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+          for (int part = 0; part < 2; ++part) {
+            uint32_t a[4];
+            sel_ldmatrix(a, qa + (part * SEL_QT + 16 * mt) * RS + k0);
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+              sel_mma_bf16(acc[mt][nt], a[0], a[1], a[2], a[3], b[2 * nt], b[2 * nt + 1]);
+          }
+      }
+      __syncthreads();  // keys consumed: lt reuses their space
+      if (tid == 0) trace_mark(1);  // logits computed
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {  // a pair of keys; a row's last one may be padding
+            const int qq = 16 * mt + gr + e * 4, kk = 16 * warp + 8 * nt + gc;
+            const float2 l = make_float2(acc[mt][nt][e] * scale, acc[mt][nt][e + 1] * scale);
+            *(float2 *)(lt + qq * SEL_LTS + kk) =
+                make_float2(kk < nk ? l.x : -INFINITY, kk + 1 < nk ? l.y : -INFINITY);
+            if (kk < nk && qq < nq) *(float2 *)(ws.logit + (qg0 + qq) * cs + t0 + kk) = l;
+          }
+    } else {
+      const int kg = tid % SEL_KG, qg = tid / SEL_KG;
+      float acc[4][4];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    __syncthreads();  // keys consumed: lt reuses their space
-    if (tid == 0) trace_mark(1);  // logits computed
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 4
+      for (int d = 0; d < DH; ++d) {
+        const float4 a = *(const float4 *)(qT + d * SEL_QT + 4 * qg);
+        const float4 b = *(const float4 *)(kT + d * SEL_KC + 4 * kg);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int ql = 4 * qg + i;
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int kk = 4 * kg + j;
-        const float l = acc[i][j] * scale;
-        lt[ql * SEL_LTS + kk] = kk < nk ? l : -INFINITY;
-        if (kk < nk && ql < nq) ws.logit[(qg0 + ql) * c + t0 + kk] = l;
+          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+      }
+      __syncthreads();  // keys consumed: lt reuses their space
+      if (tid == 0) trace_mark(1);  // logits computed
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int qq = 4 * qg + i;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int kk = 4 * kg + j;
+          const float l = acc[i][j] * scale;
+          lt[qq * SEL_LTS + kk] = kk < nk ? l : -INFINITY;
+          if (kk < nk && qq < nq) ws.logit[(qg0 + qq) * cs + t0 + kk] = l;
+        }
       }
     }
-  }
-  __syncthreads();
-  // chunk statistics: 4 threads per query, keys o, o + 4, ... (the row
-  // stride SEL_LTS = 4 mod 32 puts a warp's 8 queries x 4 lanes on 32 banks)
-  const int ql = tid >> 2, o = tid & 3;
-  {
+    __syncthreads();
+    // chunk statistics: keys o, o + 4, ... of a query (the row stride SEL_LTS = 4
+    // mod 32 puts a warp's 8 queries x 4 lanes on 32 banks)
     const float *row = lt + ql * SEL_LTS;
     float mx = -INFINITY;
 #pragma unroll
@@ -532,12 +515,13 @@ __global__ void __launch_bounds__(SEL_THREADS)
     z += __shfl_xor_sync(0xffffffffu, z, 2);
     z += __shfl_xor_sync(0xffffffffu, z, 1);
     if (o == 0 && ql < nq) ws.ml[(qg0 + ql) * nch + chunk] = make_float2(mx, z);
+    __syncthreads();  // lt consumed: the next chunk's keys take its place
   }
   __threadfence();
   __syncthreads();
   if (tid == 0) trace_mark(2);  // chunk statistics stored
   int *cnt = ws.cnt + (size_t)g * n_qt + qt;
-  if (tid == 0) *last = atomicAdd(cnt, 1) == nch - 1;
+  if (tid == 0) *last = atomicAdd(cnt, 1) == (int)gridDim.x - 1;
   __syncthreads();
   if (tid == 0) trace_mark(3);  // arrival counted
   if (!*last) return;
@@ -570,35 +554,40 @@ __global__ void __launch_bounds__(SEL_THREADS)
 }
 
 // tot[layer][t] = sum over the S*H queries of exp(logit - max) / sum, in a fixed
-// order: a CTA takes ACC_KEYS keys of a layer; its ACC_SLICES thread slices sum
-// interleaved sets of the queries (coalesced along the keys), then one
-// thread per key adds the slice sums in slice order.
-constexpr int ACC_KEYS = 16, ACC_SLICES = 32;
-__global__ void __launch_bounds__(ACC_KEYS * ACC_SLICES)
-    k_attn_select_accum(const float *logit, const float2 *mz, int NQ, int c, float *tot) {
+// order: a CTA takes ACC_KEYS keys of a layer, four a thread; its ACC_SLICES
+// thread slices sum interleaved sets of the queries, then one thread per key
+// adds the slice sums in slice order.
+constexpr int ACC_KEYS = 64, ACC_SLICES = 32;
+__global__ void __launch_bounds__(ACC_KEYS / 4 * ACC_SLICES)
+    k_attn_select_accum(const float *logit, const float2 *mz, int NQ, int c, int cs, float *tot) {
   TraceScope ts(TK_SELECT_ACC);
   pdl_trigger();
-  __shared__ float part[ACC_SLICES][ACC_KEYS];
-  const int kk = threadIdx.x % ACC_KEYS, sl = threadIdx.x / ACC_KEYS;
-  const int t = blockIdx.x * ACC_KEYS + kk;
-  logit += (size_t)blockIdx.y * NQ * c;
+  __shared__ float4 part[ACC_SLICES][ACC_KEYS / 4];
+  const int kq = threadIdx.x % (ACC_KEYS / 4), sl = threadIdx.x / (ACC_KEYS / 4);
+  const int t = blockIdx.x * ACC_KEYS + 4 * kq;
+  logit += (size_t)blockIdx.y * NQ * cs;
   mz += (size_t)blockIdx.y * NQ;
   pdl_wait();  // logits and softmax statistics of the kernel before
-  float s = 0.f;
-  if (t < c) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (t < c) {  // a row's last quad may end in its padding: sums that nobody takes
 #pragma unroll 8
     for (int qg = sl; qg < NQ; qg += ACC_SLICES) {
       const float2 st = mz[qg];
-      s += expf(logit[(size_t)qg * c + t] - st.x) * st.y;
+      const float4 l = *(const float4 *)(logit + (size_t)qg * cs + t);
+      s.x += expf(l.x - st.x) * st.y;
+      s.y += expf(l.y - st.x) * st.y;
+      s.z += expf(l.z - st.x) * st.y;
+      s.w += expf(l.w - st.x) * st.y;
     }
   }
-  part[sl][kk] = s;
+  part[sl][kq] = s;
   __syncthreads();
-  if (sl == 0 && t < c) {
+  const int k = threadIdx.x, tk = blockIdx.x * ACC_KEYS + k;
+  if (k < ACC_KEYS && tk < c) {
     float sum = 0.f;
 #pragma unroll
-    for (int i = 0; i < ACC_SLICES; ++i) sum += part[i][kk];
-    tot[(size_t)blockIdx.y * c + t] = sum;
+    for (int i = 0; i < ACC_SLICES; ++i) sum += ((const float *)part[i])[k];
+    tot[(size_t)blockIdx.y * c + tk] = sum;
   }
 }
 
@@ -727,14 +716,14 @@ constexpr size_t SEL_GROUP_BYTES = (size_t)64 << 20;
 SelLayout sel_layout(int S, const Dims &dm, int c) {
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t NQ = (size_t)S * dm.H, nqt = ((size_t)S * (dm.H / dm.G) + SEL_QT - 1) / SEL_QT;
-  const size_t fit = SEL_GROUP_BYTES / (NQ * c * sizeof(float));
+  const size_t cs = sel_stride(c), fit = SEL_GROUP_BYTES / (NQ * cs * sizeof(float));
   SelLayout o;
   o.group = fit < 1 ? 1 : fit < (size_t)dm.L ? (int)fit : dm.L;
   while (o.group > 1 && (size_t)o.group * nqt > 65535) --o.group;  // grid z
   o.q = 0;
   o.tot = o.q + al((size_t)dm.L * NQ * dm.dh * sizeof(float));
   o.logit = o.tot + al((size_t)dm.L * c * sizeof(float));
-  o.ml = o.logit + al(o.group * NQ * c * sizeof(float));
+  o.ml = o.logit + al(o.group * NQ * cs * sizeof(float));
   o.mz = o.ml + al(o.group * NQ * sel_chunks(c) * sizeof(float2));
   o.cnt = o.mz + al(o.group * NQ * sizeof(float2));
   o.total = o.cnt + al((size_t)o.group * dm.G * nqt * sizeof(int));
@@ -752,8 +741,9 @@ float *attn_select_queries(void *ws_base, int S, const Dims &dm, int n_pool, int
 }
 
 int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_end, int n,
-                              void *ws_base, unsigned long long *keys, cudaStream_t s) {
-  const int c = n - s_end;
+                              void *ws_base, unsigned long long *keys, int num_sms,
+                              cudaStream_t s) {
+  const int c = n - s_end, cs = sel_stride(c);
   if (c <= 0 || S <= 0) return 0;
   const float scale = (float)(1.0 / sqrt((double)dm.dh));
   const SelLayout o = sel_layout(S, dm, c);
@@ -765,7 +755,6 @@ int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_
   const int layer0 = layer / o.group * o.group, layers = layer - layer0 + 1;
   // arrival counts start at zero; each launch's last CTAs leave them at zero
   if (layer0 == 0) cudaMemsetAsync(ws.cnt, 0, (size_t)o.group * dm.G * nqt * sizeof(int), s);
-  const dim3 grid(sel_chunks(c), dm.G, nqt * layers);
   // bf16: q_hi, q_lo and keys as bf16 rows of dh + 8; fp32: q and keys as
   // fp32 columns of dh.  The logits tile reuses the keys' space.
   const bool bf16 = dm.dtype == KVR_DTYPE_BF16;
@@ -773,15 +762,22 @@ int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_
   const size_t k_b = bf16 ? (size_t)SEL_KC * (dm.dh + 8) * 2 : (size_t)SEL_KC * dm.dh * 4;
   const size_t lt_b = (size_t)SEL_QT * SEL_LTS * sizeof(float);
   const size_t smem = q_b + (k_b > lt_b ? k_b : lt_b);  // 34 KB (bf16), 48 KB (fp32) at dh 128
-  auto kern = bf16 ? k_attn_select_logits<__nv_bfloat16> : k_attn_select_logits<float>;
+  auto kern = dm.dh == 128 ? (bf16 ? k_attn_select_logits<__nv_bfloat16, 128>
+                                   : k_attn_select_logits<float, 128>)
+                           : (bf16 ? k_attn_select_logits<__nv_bfloat16, 64>
+                                   : k_attn_select_logits<float, 64>);
   // fp32 at dh 128, plus the trace build's static shared memory, passes 48 KB
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // one wave: the chunks spread evenly over the CTAs that fit at once
+  const int nch = sel_chunks(c), fit = (bf16 ? 6 : 4) * num_sms / (dm.G * nqt * layers);
+  const int per = fit < 1 ? nch : (nch + fit - 1) / fit;
+  const dim3 grid((nch + per - 1) / per, dm.G, nqt * layers);
   launch_pdl(kern, grid, SEL_THREADS, smem, s,
-             (const float *)attn_select_queries(ws_base, S, dm, c, layer0), S, dm.H, dm.G, dm.dh,
-             layer0, nqt, v, s_end, c, scale, ws);
+             (const float *)attn_select_queries(ws_base, S, dm, c, layer0), S, dm.H, dm.G,
+             layer0, nqt, v, s_end, c, cs, scale, ws);
   launch_pdl(k_attn_select_accum, dim3((c + ACC_KEYS - 1) / ACC_KEYS, layers),
-             ACC_KEYS * ACC_SLICES, 0, s, (const float *)ws.logit, (const float2 *)ws.mz, S * dm.H,
-             c, tot + (size_t)layer0 * c);
+             ACC_KEYS / 4 * ACC_SLICES, 0, s, (const float *)ws.logit, (const float2 *)ws.mz,
+             S * dm.H, c, cs, tot + (size_t)layer0 * c);
   if (layer + 1 < dm.L) return 2;
   launch_pdl(k_layer_sum_keys, grid_for(c, 256), 256, 0, s, (const float *)tot, dm.L, c, keys);
   return 3;

@@ -651,7 +651,7 @@ void launch_first_delim(const int32_t *tokens, int n, int s_end, int delim, int 
 size_t attn_select_ws_bytes(int S, const Dims &dm, int n_pool);
 float *attn_select_queries(void *ws_base, int S, const Dims &dm, int n_pool, int layer);
 int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_end, int n,
-                              void *ws_base, unsigned long long *keys, cudaStream_t s);
+                              void *ws_base, unsigned long long *keys, int num_sms, cudaStream_t s);
 void launch_kv_deviation(const float *qkv, const float2 *rope, const int32_t *pos, int M,
                          const Dims &dm, KVView v, float *scores, cudaStream_t s);
 void launch_float_keys(const float *scores, int n, int s_end, unsigned long long *keys,

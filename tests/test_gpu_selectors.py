@@ -1,0 +1,42 @@
+"""The Attention selector's scoring kernels over long pools: CTAs that take
+several key chunks each (two, three, and a last CTA with fewer), two query
+tiles per kv group with the second one ragged, pool lengths that leave a logit
+row's last quad and the last chunk ragged -- against the oracle's scores on the
+same stale cache, within the tie band that the other selector tests use."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2609_17983_gb300 import synth
+
+try:
+    from paper_2609_17983_gb300 import kvrepair as kv
+except ImportError as _e:  # pragma: no cover
+    kv, _IMPORT_ERROR = None, _e
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,dh,n", [("bf16", 128, 4299), ("bf16", 64, 3001), ("fp32", 128, 3002),
+                                        ("fp32", 64, 4301)])
+def test_attention_selector_of_long_pools(dtype, dh, n):
+    cfg = synth.preset("tiny", dtype=dtype, d_model=512, ffn=512, n_heads=32, n_kv_heads=8,
+                       head_dim=dh)
+    W = synth.weights(cfg, 0)
+    s, L, K = 100, 11, 32  # 44 queries a kv group
+    doc = synth.document(17, n, cfg["vocab"])
+    new = synth.edit_tokens(18, doc[s:s + L], cfg["vocab"], cfg["delim_id"])
+    bits = synth.kv_rows(19, n, cfg["n_layers"], 8, dh, "bf16", std=0.45)
+    k, v = (synth.bf16_bits_to_f32(x) for x in bits)
+    model = kv.Model(cfg, None, seed=0, max_context=4608, max_rows=256)
+    cache = model.load_cache(doc, *(bits if dtype == "bf16" else (k, v)))
+    got = model.select(cache, "attention", K, s, new)
+    to = lambda x: np.ascontiguousarray(x.transpose(1, 0, 2, 3))  # noqa: E731
+    sc, D = oracle.scores(cfg, W, oracle.Cache(to(k), to(v), doc.copy()), "attention", s, new)
+    ref = oracle.topk(sc, D, K)
+    band = (1e-4 if dtype == "fp32" else 2e-2) * np.abs(sc[D]).max()
+    kth = sc[ref].min()
+    assert len(got) == K
+    assert all(sc[j] >= kth - band for j in got)
+    assert all(j in got for j in ref if sc[j] > kth + band)
+    model.close()
