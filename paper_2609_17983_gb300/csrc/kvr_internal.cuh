@@ -307,7 +307,7 @@ struct kvr_cache {
     int64_t kernels;
     cudaGraphExec_t exec;
   };
-  std::vector<Graph> graphs;  // captured repair passes of this cache
+  std::vector<Graph> graphs;  // repair passes of this cache: run once (exec null), then captured
   kvr::KVView view() const {
     return kvr::KVView{pages, table, model->dims.L, model->dims.G, model->dims.dh};
   }
