@@ -708,15 +708,13 @@ kvr_status grow_scratch(kvr_model *m, void *&buf, size_t &have, size_t need, con
   return KVR_OK;
 }
 
-// Whether rows (bytes of K, as many of V) go to the host by the kernel's own stores
-// (launch_cache_read_host): into page-locked memory that the device writes
-// directly.  Measured against positions up, gather, two copies and the flag's:
-// 27 -> 19 us for 0.3 MB, 39 -> 31 for 1.3 MB, 70 -> 60 for 4.2 MB; larger reads
-// are bound by the link either way.
-constexpr size_t HOST_READ_MAX_BYTES = (size_t)8 << 20;
-bool host_read_direct(int n_pos, size_t bytes, const void *k_out, const void *v_out) {
-  if (n_pos > HOST_READ_MAX_POS || bytes > HOST_READ_MAX_BYTES ||
-      (((uintptr_t)k_out | (uintptr_t)v_out) & 15))
+// Whether n_pos rows (bytes of K, as many of V) go to the host by the kernel's own
+// stores (launch_cache_read_host): into page-locked memory that the device
+// writes directly.  Measured against gather, two copies and the flag's: 41 ->
+// 23 us for 1.3 MB, 48 -> 30 for 2.7, 142 -> 126 for 20, 488 -> 448 for 82; the
+// link (180 GB/s) bounds the large ones either way.
+bool host_read_direct(int n_pos, int max_pos, size_t bytes, const void *k_out, const void *v_out) {
+  if (n_pos > max_pos || bytes >= (size_t)1 << 35 || (((uintptr_t)k_out | (uintptr_t)v_out) & 15))
     return false;
   for (const void *p : {k_out, v_out}) {
     cudaPointerAttributes a{};
@@ -1451,7 +1449,7 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
     // 449; 40 rows of 32 layers, 2.6 MB, 3140 against 3153).
     constexpr size_t DIRECT_BYTES = (size_t)1 << 20;
     const bool direct =
-        k_out && M * row_b <= DIRECT_BYTES && host_read_direct(M, M * row_b, k_out, v_out);
+        k_out && M * row_b <= DIRECT_BYTES && host_read_direct(M, HOST_READ_MAX_POS, M * row_b, k_out, v_out);
     if (!st && k_out && !direct) {
       st = grow_scratch(m, m->rows_scratch, m->rows_scratch_bytes, 2 * M * row_b, "row buffer");
       r.rows_out = m->rows_scratch;
@@ -1462,7 +1460,7 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
       st = run_pass_graph(m, c, r);
     }
     if (!st && direct) {
-      launch_cache_read_host(r.single, dm.dtype, P.data(), M, 0, dm.L, dm.G, dm.dh, k_out, v_out,
+      launch_cache_read_host(r.single, dm.dtype, P.data(), nullptr, M, 0, dm.L, dm.G, dm.dh, k_out, v_out,
                              m->dev_flag, m->flag_h, m->stream);
       st = launch_check(m, 1);
       if (!st)
@@ -2099,8 +2097,15 @@ kvr_status cache_read(const kvr_cache *c, const int32_t *positions, int32_t n_po
   KVR_TRY(use_device(m));
   const size_t elems = (size_t)n_pos * (l1 - l0) * dm.G * dm.dh;
   const size_t eb = raw ? dm.es() : 4;
-  if (raw && host_read_direct(n_pos, elems * eb, k_out, v_out)) {
-    launch_cache_read_host(c->view(), dm.dtype, positions, n_pos, l0, l1, dm.G, dm.dh, k_out,
+  if (raw && host_read_direct(n_pos, (int)m->stage_cap, elems * eb, k_out, v_out)) {
+    int32_t *pd = nullptr;
+    if (n_pos > HOST_READ_MAX_POS) {  // more than a launch's arguments hold
+      KVR_TRY(grow_scratch(m, m->read_scratch, m->read_scratch_bytes, (size_t)n_pos * 4,
+                           "readback scratch"));
+      pd = (int32_t *)m->read_scratch;
+      KVR_TRY(stage_h2d(m, pd, positions, n_pos));
+    }
+    launch_cache_read_host(c->view(), dm.dtype, positions, pd, n_pos, l0, l1, dm.G, dm.dh, k_out,
                            v_out, m->dev_flag, m->flag_h, m->stream);
     const kvr_status st = launch_check(m, 1);
     if (!st) return sync_model(m, true);

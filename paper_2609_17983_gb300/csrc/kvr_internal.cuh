@@ -486,11 +486,12 @@ void launch_cache_gather(KVView v, int dtype, const int32_t *pos, int n_pos, int
 // The same gather in the cache's element type (no widening).
 void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
                              int G, int dh, void *k_out, void *v_out, cudaStream_t s);
-// The same into page-locked host memory (16-byte aligned), positions from host
-// memory (at most HOST_READ_MAX_POS), and the device error flag to *flag_out.
+// The same into page-locked host memory (16-byte aligned, fewer than 2^31 16-byte
+// pieces), positions from host memory (at most HOST_READ_MAX_POS) or, pos_d not
+// null, from the device, and the device error flag to *flag_out.
 constexpr int HOST_READ_MAX_POS = 512;
-void launch_cache_read_host(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
-                            int G, int dh, void *k_out, void *v_out, const int *flag_in,
+void launch_cache_read_host(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d,
+                            int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out, const int *flag_in,
                             int *flag_out, cudaStream_t s);
 // Rows [n_pos][L][G][dh] (cache dtype) of consecutive positions p0.. into the pages.
 void launch_cache_scatter_raw(KVView v, int dtype, int p0, int n_pos, const void *k_in,

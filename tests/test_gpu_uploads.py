@@ -60,3 +60,22 @@ def test_single_repairs_reach_the_device_in_order():
         doc[s:s + 4] = new
     check_layer0(model, [cache], [doc], cfg["d_model"])
     model.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_rows_read_into_page_locked_memory(dtype):
+    # the positions that a launch's arguments hold (512), one fewer and more, in
+    # any order and with repeats: exactly what pageable arrays get
+    import torch
+    cfg = synth.preset("tiny", n_layers=3, dtype=dtype)
+    model = kv.Model(cfg, None, seed=0, max_context=2048, max_rows=1024)
+    cache = model.prefill(synth.document(4, 1700, cfg["vocab"]))
+    for n in (511, 512, 513, 2300):
+        pos = np.random.default_rng(n).integers(0, 1700, n).astype(np.int32)
+        want = cache.read_raw(pos)
+        t = torch.int16 if dtype == "bf16" else torch.float32
+        got = [torch.zeros(want[0].shape, dtype=t, pin_memory=True).numpy().view(want[0].dtype)
+               for _ in range(2)]
+        cache.read_raw(pos, k_out=got[0], v_out=got[1])
+        assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1]), n
+    model.close()
