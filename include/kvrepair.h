@@ -151,10 +151,10 @@ kvr_status kvr_cache_load(kvr_model *model, const int32_t *tokens, int32_t n, co
  * cache and leave it bit-identical.  positions_out: host int32[K], receives
  * *count_out ascending positions in [edit_end, n).  *count_out == K except
  * for STRUCTURAL when the pool holds fewer delimiters, and when the pool is
- * smaller than K.  Ties go to the lowest position.  Device scratch (the
- * edited tokens; for ATTENTION and CACHEBLEND the saved span rows and the
- * ATTENTION logits) belongs to the model and only grows: a call that fits
- * allocates nothing.  Errors: KVR_E_RANGE (K < 0, span outside the
+ * smaller than K.  Ties go to the lowest position.  Device scratch (for
+ * ATTENTION and CACHEBLEND the edited tokens and the saved span rows, for
+ * ATTENTION its queries and logits) belongs to the model and only grows: a
+ * call that fits allocates nothing.  Errors: KVR_E_RANGE (K < 0, span outside the
  * context, token id outside the vocabulary, empty span for ATTENTION or
  * CACHEBLEND), KVR_E_INVAL (NULL argument, cache of another model, unknown
  * policy), KVR_E_POISONED, KVR_E_UNSUPPORTED (span above max_rows,

@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(TPB, TPB == NORM_THREADS_WIDE && NV <= 4 ? 4 :
 // Many complete rows: the CTAs that fit (four an SM, NV <= 4) stay and take rows
 // in turn, the next row's loads in flight while this one is reduced and written.
 // Bound by HBM: 4096 rows of d = 4096 move 100 MB.  A CTA per row waited for
-// its loads, then for the sum, and left: 21 us, this 14.
+// its loads, then for the sum, and left: 24 us between events, this 17.
 template <typename T, int NV>
 __global__ void __launch_bounds__(NORM_THREADS_WIDE, 4)
     k_rmsnorm_rows(const float *h, const float *g, int row0, int M, int d, float eps, T *out) {
@@ -367,12 +367,13 @@ __global__ void __launch_bounds__(ROPE_HEADS * 64) k_rope_scatter(const RopeArgs
 
 // Many rows: a CTA per row, four rotated pairs per thread (16-byte loads, 8- or
 // 16-byte stores) of HPT heads, which share the position, its table entries and
-// page; the projection's loads do not wait for any of them.  One pair per thread
-// with 2-byte stores took 75 us for 4096 rows of a 6144-wide projection (100 MB
-// read, 50 MB written); four rows of one head per thread 44 (107 registers, two
-// CTAs an SM).
+// page; the projection's loads do not wait for any of them.  Bound by HBM: 4096
+// rows of a 6144-wide projection, 100 MB read, 50 MB written, take 29 us between
+// events.  One pair per thread with 2-byte stores took 75; four rows of one head
+// per thread 44 (107 registers, two CTAs an SM).
 constexpr int ROPE_THREADS = 256;
-constexpr int ROPE_MANY = 64;  // rows from which it is taken (40 rows: equal; 64 rows: 9.9 -> 8.2 us)
+// rows from which it is taken (40 rows: equal; 64 rows: 9.9 -> 8.2 us)
+constexpr int ROPE_MANY = 64;
 template <typename T, int HPT>
 __global__ void __launch_bounds__(ROPE_THREADS, HPT > 1 ? 4 : 1) k_rope_rows(const RopeArgs a) {
   TraceScope ts(TK_ROPE);
@@ -578,8 +579,8 @@ __global__ void k_transplant(KVView dst, KVView src, const int32_t *pos, int n_p
 
 // out[i] = logits[i][target[i]] - logsumexp(logits[i]) for each row, one CTA a
 // row; out is page-locked host memory, and the device error flag goes with it
-// (copies of targets, results and flag took 30 us of a pass).  One pass: a thread keeps its maximum and the sum of exponentials
-// against it, LP_VEC float4 loads in flight (V % 4 == 0 keeps every row on a
+// (copies of targets, results and flag took 30 us of a pass).  One pass: a thread
+// keeps its maximum and the sum of exponentials against it, LP_VEC float4 loads in flight (V % 4 == 0 keeps every row on a
 // 16-byte boundary; other widths load one at a time).  Two passes of scalar
 // loads by 256 threads took 49 us for 128256 logits.
 constexpr int LP_THREADS = 1024, LP_VEC = 4;
@@ -675,7 +676,7 @@ void launch_upload(const Upload *u, int n, cudaStream_t s) {
   size_t most = 1;
   for (int i = 0; i < n; ++i) most = std::max(most, u[i].words);
   const dim3 grid((unsigned)((most + UP_THREADS * UP_WORDS - 1) / (UP_THREADS * UP_WORDS)), n);
-  auto go = [&](auto list) {  // a call's few segments leave the larger list's bytes out of the launch
+  auto go = [&](auto list) {  // few segments: a launch without the larger list's bytes
     std::copy(u, u + n, list.u);
     k_upload<<<grid, UP_THREADS, 0, s>>>(list);
   };
@@ -714,7 +715,8 @@ void launch_rmsnorm(float *h, const float *g, int row0, int M, int d, double eps
         auto k = nv <= 1 ? k_rmsnorm_rows<__nv_bfloat16, 1>
                  : nv <= 2 ? k_rmsnorm_rows<__nv_bfloat16, 2>
                            : k_rmsnorm_rows<__nv_bfloat16, 4>;
-        launch_pdl(k, grid, W, 0, s, (const float *)h, g, row0, M, d, (float)eps, (__nv_bfloat16 *)out);
+        launch_pdl(k, grid, W, 0, s, (const float *)h, g, row0, M, d, (float)eps,
+                   (__nv_bfloat16 *)out);
       } else {
         auto k = nv <= 1 ? k_rmsnorm_rows<float, 1>
                  : nv <= 2 ? k_rmsnorm_rows<float, 2>

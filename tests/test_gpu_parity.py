@@ -589,8 +589,8 @@ def test_select_long_context_exact(n):
 
 def test_graph_replay_matches_eager():
     # repair passes captured as a CUDA graph (model on a non-default stream)
-    # give bit-identical caches to eager launches, on the first (capturing)
-    # call and on replays with different positions of the same shape
+    # give bit-identical caches to eager launches: on the first call (eager),
+    # the second (capturing) and on replays with other positions of the same shape
     import torch
     cfg = synth.preset("llama8b", n_layers=2)
     n, s, L = 600, 300, 8
@@ -619,8 +619,8 @@ def test_graph_replay_matches_eager():
 @pytest.mark.parametrize("graphs", [True, False])
 def test_repair_read_returns_the_repaired_rows(shape, layers, graphs):
     # kvr_repair_read leaves the cache as kvr_repair does and returns exactly
-    # what kvr_cache_read_raw returns for P afterwards: on the capturing call
-    # and on replays (the copies wait on events the graph records on a side
+    # what kvr_cache_read_raw returns for P afterwards: on the first, the
+    # capturing call and on replays (the copies wait on events the graph records on a side
     # branch, layer groups with a ragged last one), and after eager launches
     # (no stream of its own: no graph); into page-locked and pageable buffers
     import torch
