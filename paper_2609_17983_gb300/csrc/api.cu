@@ -1097,14 +1097,14 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
     size_t sz[] = {R * 4,          R * 4,          R * d * 4,        R * d * es,  R * Nq * 4,
                    R * HD * 4,     R * HD * es,    R * F * es,
                    (size_t)KVR_QUERY_RESERVE * V * 4,
-                   P * 4,          P * 8,          256,         R * HD * 2};
+                   P * 4,          P * 8,          R * HD * 2};
     size_t tot = 0;
     for (size_t x : sz) tot += al(x);
     m->ws_block = dev_alloc(tot);
     if (!m->ws_block) return bail(fail(KVR_E_NOMEM, "workspace: %zu bytes", tot));
     char *p = (char *)m->ws_block;
-    void *ptrs[13];
-    for (int i = 0; i < 13; ++i) {
+    void *ptrs[12];
+    for (int i = 0; i < 12; ++i) {
       ptrs[i] = p;
       p += al(sz[i]);
     }
@@ -1119,8 +1119,7 @@ kvr_status kvr_model_create(const kvr_model_config *cfg, const kvr_weights *wts,
     m->logits = (float *)ptrs[8];
     m->scores = (float *)ptrs[9];
     m->keys = (unsigned long long *)ptrs[10];
-    m->sel_count = (int32_t *)ptrs[11];
-    m->qb = ptrs[12];
+    m->qb = ptrs[11];
     m->dev_flag = (int *)dev_alloc(256);
     if (!m->dev_flag) return bail(fail(KVR_E_NOMEM, "flag"));
     cudaMemset(m->dev_flag, 0, 256);
@@ -1702,21 +1701,10 @@ kvr_status kvr_select(kvr_model *m, const kvr_cache *c, kvr_policy policy, int32
   void *probs = nullptr;  // Attention: the selector workspace
   if (!st && (policy == KVR_POLICY_EDITLOCAL || policy == KVR_POLICY_STRUCTURAL ||
               policy == KVR_POLICY_RANDOM || policy == KVR_POLICY_EDITLOCAL_BOUNDARY)) {
-    int *bound = (int *)(m->sel_count + 1);
-    if (policy == KVR_POLICY_EDITLOCAL_BOUNDARY) {
-      Prof pr(m, P_SELECT, 0);
-      int init = n - 1;
-      st = stage_h2d(m, bound, &init, 1);
-      if (!st) {
-        launch_first_delim(toks, n, s_end, dm.delim, bound, m->stream);
-        st = launch_check(m, 1);
-      }
-    }
     gen.policy = (int)policy;
     gen.tokens = toks;
     gen.delim = dm.delim;
     gen.seed = seed;
-    gen.bound = bound;
     if (policy == KVR_POLICY_STRUCTURAL || policy == KVR_POLICY_EDITLOCAL_BOUNDARY) topk_k = -K;
   } else if (!st && policy == KVR_POLICY_ATTENTION) {
     if (edit_len == 0) {

@@ -27,27 +27,15 @@ __device__ __forceinline__ uint32_t ord_f32(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// First delimiter position at or after s_end (n - 1 if none): the document
-// boundary of EditLocal@boundary.  *bound must hold n - 1 on entry.
-__global__ void k_first_delim(const int32_t *tokens, int n, int s_end, int delim, int *bound) {
-  for (int j = s_end + blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-    if (tokens[j] == delim) atomicMin(bound, j);
-}
-
-// Key of pool entry t (position s_end + t) under a simple policy; bnd: the
-// EditLocal@boundary boundary.
-__device__ __forceinline__ unsigned long long simple_key(const SimpleKeys &g, int s_end, int t,
-                                                        int bnd) {
+// Key of pool entry t (position s_end + t) under Random or Structural.
+__device__ __forceinline__ unsigned long long simple_key(const SimpleKeys &g, int s_end, int t) {
   const int j = s_end + t;
   if (g.policy == KVR_POLICY_RANDOM) {
     // first SplitMix64 output of state seed ^ (j * gamma)
     return mix64((g.seed ^ ((uint64_t)j * GAMMA)) + GAMMA);
   }
-  // nearest to the span first
-  unsigned long long k = 0x100000000ull - (unsigned long long)t;
-  if (g.policy == KVR_POLICY_STRUCTURAL && g.tokens[j] != g.delim) k = 0;
-  if (g.policy == KVR_POLICY_EDITLOCAL_BOUNDARY && j > bnd) k = 0;
-  return k;
+  // Structural: delimiters, nearest to the span first
+  return g.tokens[j] == g.delim ? 0x100000000ull - (unsigned long long)t : 0;
 }
 
 __global__ void k_float_keys(const float *scores, int n, int s_end, unsigned long long *keys) {
@@ -58,17 +46,21 @@ __global__ void k_float_keys(const float *scores, int n, int s_end, unsigned lon
 
 // Top-K of c (key, index) pairs, one CTA of TOPK_THREADS: key descending, ties to
 // the lowest index, the chosen indices written ascending.  Instead of a sort,
-// the K-th key T is found by an MSB-first radix select (8 bits per pass, a
+// the K-th key T is found by an MSB-first radix select (11 bits per pass, a
 // shared-memory histogram of the keys that still match the prefix), starting
-// at the highest 8-bit digit in which the keys differ (the AND and OR of all
-// keys give the digits they share, which the passes would only confirm); then
+// at the highest bit in which the keys differ (the AND and OR of all keys give
+// the bits they share, which the passes would only confirm); then
 // every key above T is taken, and of the keys equal to T the lowest-indexed
 // ones until K are taken.  A pass that ends with every key of the chosen bin
 // taken ends the search: the digits below cannot change the set (Random's
-// 64-bit keys part after two or three of eight passes: 13.3 us with all of
-// them for 1544 keys, 8 without).  Thread i owns the contiguous keys [i*E, (i+1)*E),
-// so a block-wide scan of per-thread counts writes the output in index order.
+// 64-bit keys mostly part in the first).  8-bit digits counted bin by bin of a
+// warp (match.any) took 20.8 us a Random selection of 1544 keys through the
+// API and 25.5 of 4894, now 19.5 and 20.8.  Thread i owns the contiguous keys
+// [i*E, (i+1)*E), so a block-wide scan of per-thread counts writes the output in
+// index order.
 constexpr int TOPK_THREADS = 1024;
+constexpr int TOPK_BITS = 11;  // two bins a thread
+static_assert(1 << TOPK_BITS == 2 * TOPK_THREADS, "two bins a thread");
 
 __device__ __forceinline__ int block_excl_scan(int x, int *tmp) {
   // tmp: TOPK_THREADS / 32 ints
@@ -99,18 +91,28 @@ __global__ void __launch_bounds__(TOPK_THREADS)
            int32_t *out, int32_t *count, const SimpleKeys gen, const int *flag_in,
            int32_t *flag_out) {
   extern __shared__ unsigned long long sk[];  // c keys
-  __shared__ int hist[256];
+  __shared__ int hist[1 << TOPK_BITS];
   __shared__ int scan_tmp[TOPK_THREADS / 32];
   __shared__ int s_elig, s_bin, s_above, s_in;
   __shared__ unsigned long long s_and, s_or;
   const int tid = threadIdx.x;
-  if (gen.policy == KVR_POLICY_EDITLOCAL ||
-      (gen.policy == KVR_POLICY_EDITLOCAL_BOUNDARY && nonzero_only)) {
-    // EditLocal's keys fall strictly with t, all nonzero (@boundary: nonzero
-    // up to the boundary, zero after it, and only nonzero keys eligible): the
-    // K largest are the first K candidates, already in index order.
-    const int avail = gen.policy == KVR_POLICY_EDITLOCAL ? c : min(c, *gen.bound - s_end + 1);
-    const int cnt = min(K, max(avail, 0));
+  if (gen.policy == KVR_POLICY_EDITLOCAL || gen.policy == KVR_POLICY_EDITLOCAL_BOUNDARY) {
+    // EditLocal's keys fall strictly with t, and all are eligible (@boundary: up
+    // to the first delimiter, the whole pool without one): the K largest are the
+    // first K candidates, already in index order.
+    int avail = c;
+    if (gen.policy == KVR_POLICY_EDITLOCAL_BOUNDARY) {
+      if (tid == 0) s_in = c;
+      __syncthreads();
+      for (int t = tid; t < c; t += TOPK_THREADS)
+        if (gen.tokens[s_end + t] == gen.delim) {
+          atomicMin(&s_in, t + 1);
+          break;
+        }
+      __syncthreads();
+      avail = s_in;
+    }
+    const int cnt = min(K, avail);
     for (int t = tid; t < cnt; t += TOPK_THREADS) out[t] = s_end + t;
     if (tid == 0) {
       *count = cnt;
@@ -126,15 +128,17 @@ __global__ void __launch_bounds__(TOPK_THREADS)
     s_or = 0ull;
   }
   __syncthreads();
-  const int bnd = gen.policy == KVR_POLICY_EDITLOCAL_BOUNDARY ? *gen.bound : 0;
+  auto eligible = [&](unsigned long long k) { return !nonzero_only || k != 0ull; };
   int local = 0;
   unsigned long long kand = ~0ull, kor = 0ull;
   for (int t = tid; t < c; t += TOPK_THREADS) {
-    const unsigned long long k = gen.policy >= 0 ? simple_key(gen, s_end, t, bnd) : keys[t];
+    const unsigned long long k = gen.policy >= 0 ? simple_key(gen, s_end, t) : keys[t];
     sk[t] = k;
-    kand &= k;
-    kor |= k;
-    local += (!nonzero_only || k != 0ull) ? 1 : 0;
+    if (eligible(k)) {
+      kand &= k;
+      kor |= k;
+      ++local;
+    }
   }
   for (int o = 16; o > 0; o >>= 1) {
     local += __shfl_xor_sync(0xffffffffu, local, o);
@@ -149,69 +153,47 @@ __global__ void __launch_bounds__(TOPK_THREADS)
   __syncthreads();
   const int cnt = min(K, s_elig);
   // radix select: prefix/mask of T, need = how many keys equal to the prefix
-  // (so far) are still to be taken.  The digits above dtop are the same in
-  // every key: they start the prefix.
+  // (so far) are still to be taken.  The bits above hi are the same in every
+  // eligible key: they start the prefix.
   const unsigned long long differ = s_or ^ s_and;
-  const int dtop = differ ? (63 - __clzll((long long)differ)) / 8 * 8 : -8;
-  unsigned long long mask = dtop >= 56 ? 0ull : ~0ull << (dtop + 8);
+  int hi = 64 - (differ ? __clzll((long long)differ) : 64);  // bits not yet in the prefix
+  unsigned long long mask = hi == 64 ? 0ull : ~0ull << hi;
   unsigned long long pref = s_and & mask;
   int need = cnt;
-  for (int d = dtop; d >= 0 && need > 0; d -= 8) {
-    for (int i = tid; i < 256; i += TOPK_THREADS) hist[i] = 0;
+  while (hi > 0 && need > 0) {
+    const int d = max(0, hi - TOPK_BITS);  // this digit: bits d .. hi - 1
+    hist[tid] = hist[tid + TOPK_THREADS] = 0;
     __syncthreads();
-    // lanes whose keys fall in the same bin add their count once: keys near
-    // the span (EditLocal) share their upper digits, and one shared-memory
-    // address taking every key serialises the pass
+    // a warp whose keys all fall in one bin adds their count once (many equal keys
+    // on one shared-memory address would serialise the pass); matching lanes bin
+    // by bin instead took longer than their atomics
     for (int e = 0; e < E; ++e) {
       const int t = t0 + e;
       const unsigned long long k = t < t1 ? sk[t] : 0ull;
-      const int bin = t < t1 && (k & mask) == pref ? (int)(k >> d) & 255 : -1;
-      const unsigned peers = __match_any_sync(0xffffffffu, bin);
-      if (bin >= 0 && (tid & 31) == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
+      const bool in = t < t1 && (k & mask) == pref && eligible(k);
+      const int bin = in ? (int)(k >> d) & ((1 << (hi - d)) - 1) : -1;
+      int same;
+      __match_all_sync(0xffffffffu, bin, &same);
+      if (bin >= 0 && (!same || (tid & 31) == 0)) atomicAdd(&hist[bin], same ? 32 : 1);
     }
     __syncthreads();
-    if (tid < 32) {
-      // suffix sums over bins 255..0, 8 bins per lane (lane 0 holds 255..248)
-      int loc[8], sum = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        loc[j] = hist[255 - (tid * 8 + j)];
-        sum += loc[j];
-      }
-      int incl = sum;
-      for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (tid >= o) incl += y;
-      }
-      int acc = incl - sum;  // keys in bins above this lane's first bin
-      int found = -1, above = 0, in = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (found < 0 && acc + loc[j] >= need) {
-          found = 255 - (tid * 8 + j);
-          above = acc;
-          in = loc[j];
-        }
-        acc += loc[j];
-      }
-      const unsigned ball = __ballot_sync(0xffffffffu, found >= 0);
-      const int src = __ffs(ball) - 1;  // first lane (highest bins) that found it
-      const int bin = __shfl_sync(0xffffffffu, found, src);
-      const int ab = __shfl_sync(0xffffffffu, above, src);
-      const int ib = __shfl_sync(0xffffffffu, in, src);
-      if (tid == 0) {
-        s_bin = bin;
-        s_above = ab;
-        s_in = ib;
-      }
+    // the bin that holds the need-th key from the top: thread i's two bins,
+    // highest first, after the counts of the threads before it
+    const int b1 = 2 * (TOPK_THREADS - 1 - tid) + 1, h1 = hist[b1], h0 = hist[b1 - 1];
+    const int above = block_excl_scan(h1 + h0, scan_tmp);
+    if (above < need && above + h1 + h0 >= need) {
+      const bool first = above + h1 >= need;
+      s_bin = first ? b1 : b1 - 1;
+      s_above = first ? above : above + h1;
+      s_in = first ? h1 : h0;
     }
     __syncthreads();
     pref |= (unsigned long long)s_bin << d;
-    mask |= 0xFFull << d;
+    mask = d == 0 ? ~0ull : ~0ull << d;
     need -= s_above;
-    const bool all = s_in == need;
-    __syncthreads();
-    if (all) break;
+    hi = d;
+    if (s_in == need) break;  // the bin's keys are all taken
+    // the next pass writes s_bin, s_above and s_in behind three barriers
   }
   // T = pref in the digits of mask (when cnt > 0): take keys > T, and the first
   // `need` keys == T
@@ -219,8 +201,8 @@ __global__ void __launch_bounds__(TOPK_THREADS)
   if (cnt > 0)
     for (int t = t0; t < t1; ++t) {
       const unsigned long long k = sk[t];
-      gt += (k & mask) > pref ? 1 : 0;
-      eq += (k & mask) == pref ? 1 : 0;
+      gt += eligible(k) && (k & mask) > pref ? 1 : 0;
+      eq += eligible(k) && (k & mask) == pref ? 1 : 0;
     }
   const int eq_before = block_excl_scan(eq, scan_tmp);
   int take_eq = cnt > 0 ? min(eq, max(0, need - eq_before)) : 0;
@@ -228,6 +210,7 @@ __global__ void __launch_bounds__(TOPK_THREADS)
   int pos = block_excl_scan(sel, scan_tmp);
   if (cnt > 0)
     for (int t = t0; t < t1; ++t) {
+      if (!eligible(sk[t])) continue;
       const unsigned long long k = sk[t] & mask;
       bool take = k > pref;
       if (!take && k == pref && take_eq > 0) {
@@ -668,13 +651,6 @@ int grid_for(int n, int block) {
 }
 
 }  // namespace
-
-void launch_first_delim(const int32_t *tokens, int n, int s_end, int delim, int *bound,
-                        cudaStream_t s) {
-  int c = n - s_end;
-  if (c <= 0) return;
-  k_first_delim<<<grid_for(c, 256), 256, 0, s>>>(tokens, n, s_end, delim, bound);
-}
 
 void launch_float_keys(const float *scores, int n, int s_end, unsigned long long *keys,
                        cudaStream_t s) {

@@ -251,7 +251,6 @@ struct kvr_model {
   void *a = nullptr, *attn = nullptr, *act = nullptr;
   float *scores = nullptr;     // [max_ctx + reserve] selector scores
   unsigned long long *keys = nullptr;  // [max_ctx + reserve] top-K keys
-  int32_t *sel_count = nullptr;  // EditLocal@boundary's bound at [1]
   void *read_scratch = nullptr;  // cache readback: positions, then the gathered K and V
   size_t read_scratch_bytes = 0;
   // kvr_repair_read: the pass's K/V rows as RoPE writes them, copied to the
@@ -636,12 +635,7 @@ struct SimpleKeys {
   const int32_t *tokens = nullptr;  // the edited context (device)
   int delim = 0;
   uint64_t seed = 0;
-  const int *bound = nullptr;       // EditLocal@boundary: launch_first_delim's result
 };
-// EditLocal@boundary: the first delimiter position at or after s_end into
-// *bound, which must hold n - 1 on entry.
-void launch_first_delim(const int32_t *tokens, int n, int s_end, int delim, int *bound,
-                        cudaStream_t s);
 // Attention selector over the workspace ws_base (attn_select_ws_bytes(S, dm,
 // n - s_end) bytes).  The pass leaves layer l's span queries (fp32 [S][H*dh])
 // in attn_select_queries(.., l) and calls launch_attn_select_scores after each

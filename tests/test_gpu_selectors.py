@@ -40,3 +40,31 @@ def test_attention_selector_of_long_pools(dtype, dh, n):
     assert all(sc[j] >= kth - band for j in got)
     assert all(j in got for j in ref if sc[j] > kth + band)
     model.close()
+
+
+# The radix select of the K largest keys: pools around a thread's share (1024
+# keys) and of several keys a thread, up to the longest context; K from one to
+# the whole pool; delimiters that are many, few and absent.  The keys are whole numbers: exactly the oracle's set.
+@pytest.mark.parametrize("n", [40, 1055, 1056, 1057, 5000, 16384])
+def test_simple_policies_match_the_oracle(n):
+    cfg = synth.preset("tiny", n_layers=1)
+    model = kv.Model(cfg, None, seed=0, max_context=16384, max_rows=1024)
+    rng = np.random.default_rng(n)
+    s, L = 28, 4  # the pool: n - 32 positions
+    for every in (3, 700, None):
+        doc = synth.document(n, n, cfg["vocab"])
+        if every:
+            at = np.arange(s + L + every - 1, n, every)
+            doc[at[rng.random(len(at)) < 0.9]] = cfg["delim_id"]
+        new = synth.edit_tokens(2, doc[s:s + L], cfg["vocab"], cfg["delim_id"])
+        cache = model.prefill(doc)
+        ref = oracle.empty_cache(cfg, n)
+        ref.tokens[:] = doc
+        for policy, seed in (("random", 0), ("random", n), ("structural", 0),
+                             ("editlocal_boundary", 0), ("editlocal", 0)):
+            for K in (1, 32, n // 2, n - s - L):
+                got = model.select(cache, policy, K, s, new, seed)
+                want = oracle.select(cfg, None, ref, policy, K, s, new, seed)
+                assert got.tolist() == want.tolist(), (policy, every, K)
+        cache.close()
+    model.close()
