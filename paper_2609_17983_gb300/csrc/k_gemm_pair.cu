@@ -19,7 +19,7 @@
 // Work split, over the C clusters that fit at once: rounds of whole tiles, tile
 // R + c + kC to cluster c in round k (neighbouring clusters share weight or
 // token tiles and walk K in step, so each comes from DRAM once).  Of the R
-// tiles left over each goes to s <= C / R clusters, equal parts of K --
+// tiles left over each goes to s = floor(C / R) clusters, equal parts of K --
 // again in step -- that the tile's first cluster sums in part order from what
 // the others publish.  The parts come first, so that their sum runs beside
 // the MMAs of the whole tiles.  (Whole tiles alone: 2608 rows of a 4096-wide
@@ -33,7 +33,6 @@
 // epilogue.  Accumulators are double-buffered.  Every wait is bounded; a wait
 // that runs out sets the device error flag, the CTA's roles stop, the peer's
 // waits run out in turn, and both meet at the final cluster barrier.
-#include <algorithm>
 #include <cstdlib>
 #include <cuda.h>
 
@@ -60,7 +59,6 @@ constexpr int NT = 64 + EPI_THREADS;
 constexpr int PRE_WAIT_STAGES = 2;    // weight stages requested before the wait on the predecessor
 constexpr int MIN_UNITS = 4;          // units (of KS K blocks) a part of a tile has at least
 constexpr int MAX_PARTS = 8;          // clusters a left-over tile is split over at most
-constexpr double PART_CYCLES = 2500;  // what a part of a left-over tile costs beside its MMAs
 
 struct PairGemm {
   int M, N, KB, KU;   // K blocks, and units of KS of them (the last may be short)
@@ -415,33 +413,25 @@ size_t configure(PairGemm &p, int M, int N, int K, int clusters, int smem_limit)
   p.KB = K / BK;
   p.KU = (p.KB + KS - 1) / KS;
   p.n_tiles = (N + TM - 1) / TM;
-  // The token tile and split whose cost in cycles is least: per K block the longer
-  // of its MMAs (2 BN) and its operands' way from L2 (256 + BN at 64 bytes a cycle),
-  // and PART_CYCLES for each part that a left-over tile's owner adds, of which the
-  // MMAs of whole tiles behind it hide some (a twelfth of a tile's; both fitted to
-  // the projections of two shapes at 400 to 4096 rows).  With as many parts as
-  // there are clusters for, 2608 rows of 3584 x 3584 (two whole rounds and two
-  // tiles in seven parts) took 68 us against 59 (token tiles of 208, two parts),
-  // 4096 rows of 6144 x 4096 132 against 126.
+  // The token tile whose rounds cost least: per K block the longer of its MMAs
+  // (2 BN cycles) and its operands' way from L2 (256 + BN at 64 bytes a cycle).
   p.clusters = clusters;
   double best = -1;
   for (int bn = 256; bn >= 128; bn -= 16) {
     const long long mt = (M + bn - 1) / bn, tiles = mt * p.n_tiles;
     const int left = (int)(tiles % clusters);
-    const double tile = (double)p.KB * (2 * bn > 256 + bn ? 2 * bn : 256 + bn);
-    const int most = left ? std::min({clusters / left, MAX_PARTS, std::max(1, p.KU / MIN_UNITS)}) : 1;
-    for (int parts = 1; parts <= most; ++parts) {
-      const double sums = (parts - 1) * PART_CYCLES - (tiles >= clusters ? tile / 12 : 0.0);
-      const double c = (double)(tiles / clusters) * tile +
-                       (left ? tile / parts + std::max(sums, 0.0) : 0.0);
-      if (best < 0 || c < best) {
-        best = c;
-        p.BN = bn;
-        p.m_tiles = (int)mt;
-        p.left = left;
-        p.parts = parts;
-        p.rounds = (int)(tiles / clusters);
-      }
+    int parts = left ? clusters / left : 1;
+    if (parts > MAX_PARTS) parts = MAX_PARTS;
+    if (parts > p.KU / MIN_UNITS) parts = p.KU / MIN_UNITS > 1 ? p.KU / MIN_UNITS : 1;
+    const double rounds = (double)(tiles / clusters) + (left ? 1.0 / parts : 0.0);
+    const double c = rounds * (2 * bn > 256 + bn ? 2 * bn : 256 + bn);
+    if (best < 0 || c < best) {
+      best = c;
+      p.BN = bn;
+      p.m_tiles = (int)mt;
+      p.left = left;
+      p.parts = parts;
+      p.rounds = (int)(tiles / clusters);
     }
   }
   if (!p.rounds) p.clusters = p.left * p.parts;  // no more than have work
