@@ -2,6 +2,8 @@
 // embedding gather, RMSNorm, RoPE + K/V scatter into the paged cache,
 // and cache row readback / save / restore.
 #include <algorithm>
+#include <cooperative_groups.h>
+#include <utility>
 
 #include "kvr_internal.cuh"
 
@@ -577,13 +579,15 @@ __global__ void k_transplant(KVView dst, KVView src, const int32_t *pos, int n_p
   }
 }
 
-// out[i] = logits[i][target[i]] - logsumexp(logits[i]) for each row, one CTA a
-// row; out is page-locked host memory, and the device error flag goes with it
-// (copies of targets, results and flag took 30 us of a pass).  One pass: a thread
-// keeps its maximum and the sum of exponentials against it, LP_VEC float4 loads in flight (V % 4 == 0 keeps every row on a
-// 16-byte boundary; other widths load one at a time).  Two passes of scalar
-// loads by 256 threads took 49 us for 128256 logits.
-constexpr int LP_THREADS = 1024, LP_VEC = 4;
+// out[i] = logits[i][target[i]] - logsumexp(logits[i]) for each row; out is
+// page-locked host memory, and the device error flag goes with it (copies of
+// targets, results and flag took 30 us of a pass).  A cluster of LP_CTAS CTAs a
+// row, each with a slice of it, in one pass: a thread keeps its maximum and the
+// sum of exponentials against it, LP_VEC float4 loads in flight (V % 4 == 0
+// keeps every row on a 16-byte boundary; other widths load one at a time); the
+// first CTA adds the slices in order.  128256 logits: 5 us; one CTA a row 11,
+// two passes of scalar loads by 256 threads 49.
+constexpr int LP_THREADS = 1024, LP_VEC = 4, LP_CTAS = 8;
 struct AnswerIds {
   int32_t id[KVR_QUERY_RESERVE];
 };
@@ -593,12 +597,17 @@ __device__ __forceinline__ void lse_add(float &m, float &s, float m2, float s2) 
   s = s * expf(m - mm) + s2 * expf(m2 - mm);
   m = mm;
 }
-__global__ void __launch_bounds__(LP_THREADS)
+__global__ void __cluster_dims__(LP_CTAS, 1, 1) __launch_bounds__(LP_THREADS)
     k_row_logprob(const float *logits, int V, const __grid_constant__ AnswerIds target, float *out,
                   const int *flag_in, int *flag_out) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *flag_out = *flag_in;
-  const float *x = logits + (size_t)blockIdx.x * V;
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int row = blockIdx.x / LP_CTAS, part = blockIdx.x % LP_CTAS;
+  const float *x = logits + (size_t)row * V;
   __shared__ float2 red[LP_THREADS / 32];
+  __shared__ float2 slices[LP_CTAS];  // the first CTA's: every slice's maximum and sum
+  auto started = cluster.barrier_arrive();  // waited on before the first CTA's memory is written
   float m = -INFINITY, s = 0.f;
   // a batch of loaded values: its maximum first, then one rescale of the sum
   auto add = [&](const float *v, int n) {
@@ -612,8 +621,8 @@ __global__ void __launch_bounds__(LP_THREADS)
   };
   if (V % 4 == 0) {
     const float4 *x4 = (const float4 *)x;
-    const int n4 = V / 4;
-    for (int j0 = threadIdx.x; j0 < n4; j0 += LP_VEC * LP_THREADS) {
+    const int per = (V / 4 + LP_CTAS - 1) / LP_CTAS, n4 = min(V / 4, (part + 1) * per);
+    for (int j0 = part * per + threadIdx.x; j0 < n4; j0 += LP_VEC * LP_THREADS) {
       float4 v[LP_VEC];
 #pragma unroll
       for (int k = 0; k < LP_VEC; ++k) {
@@ -631,7 +640,8 @@ __global__ void __launch_bounds__(LP_THREADS)
       add(w, 4 * LP_VEC);
     }
   } else {
-    for (int j = threadIdx.x; j < V; j += LP_THREADS) {
+    const int per = (V + LP_CTAS - 1) / LP_CTAS, n = min(V, (part + 1) * per);
+    for (int j = part * per + threadIdx.x; j < n; j += LP_THREADS) {
       const float w[1] = {x[j]};
       add(w, 1);
     }
@@ -644,12 +654,20 @@ __global__ void __launch_bounds__(LP_THREADS)
   };
   fold();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(m, s);
+  cluster.barrier_wait(std::move(started));
   __syncthreads();
   if (threadIdx.x < 32) {
     m = red[threadIdx.x].x;
     s = red[threadIdx.x].y;
     fold();
-    if (threadIdx.x == 0) out[blockIdx.x] = x[target.id[blockIdx.x]] - (m + logf(s));
+    if (threadIdx.x == 0) cluster.map_shared_rank(slices, 0)[part] = make_float2(m, s);
+  }
+  cluster.sync();
+  if (part == 0 && threadIdx.x == 0) {
+    m = slices[0].x;
+    s = slices[0].y;
+    for (int k = 1; k < LP_CTAS; ++k) lse_add(m, s, slices[k].x, slices[k].y);
+    out[row] = x[target.id[row]] - (m + logf(s));
   }
 }
 
@@ -841,7 +859,7 @@ void launch_row_logprob(const float *logits, int rows, int V, const int32_t *tar
                         const int *flag_in, int *flag_out, cudaStream_t s) {
   AnswerIds t;
   std::copy(target, target + rows, t.id);
-  k_row_logprob<<<rows, LP_THREADS, 0, s>>>(logits, V, t, out, flag_in, flag_out);
+  k_row_logprob<<<rows * LP_CTAS, LP_THREADS, 0, s>>>(logits, V, t, out, flag_in, flag_out);
 }
 
 void launch_rows_copy(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,

@@ -104,9 +104,10 @@ def test_gemm_pairs_of_ctas(M):
     m.close()
 
 
-@pytest.mark.parametrize("vocab", [1024, 1021])
+@pytest.mark.parametrize("vocab", [1024, 1021, 20, 18])
 def test_answer_logprob_row_widths(vocab):
-    # rows on 16-byte boundaries, and rows that are not
+    # rows on 16-byte boundaries and rows that are not, and rows with fewer
+    # entries than a cluster's CTAs have slices
     cfg = synth.preset("tiny", vocab=vocab)
     W = synth.weights(cfg, 0)
     model = kv.Model(cfg, None, seed=0, max_context=256, max_rows=256)
