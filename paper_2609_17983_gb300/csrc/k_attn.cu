@@ -26,15 +26,16 @@ struct SimtAttn {
 // A CTA takes NQ queries of one kv head -- consecutive (row, query head) slots,
 // gp = H / G of them per row; with several documents gp is H / G rounded up to
 // NQ, so that a CTA's queries are of one row -- and its warps deal out the keys
-// in blocks of 32: a lane scores one key for every query (a key's row is read
-// once for all of them), the softmax folds a block at a time, then the lanes
-// split head_dim and add the block's values.  The warps' partial outputs are
-// merged in warp order.  (A warp per query that walked its keys one after
-// another, a shuffle reduction and two exponentials each, took 207 us for 36
-// rows over 240 keys and 441 us for 512 rows.)
+// in blocks of 32: four lanes score a key for every query (a key's row is read
+// once for all of them, 64 bytes at a time), the softmax folds a block at a
+// time, then the lanes split head_dim and add the block's values.  The warps'
+// partial outputs are merged in warp order.  Latency-bound: 7 us for 36 rows over
+// 240 keys, 17 for 512 rows.  (A lane per key, whose loads of one instruction lay
+// on 32 lines, took 11 and 25; a warp per query that walked its keys one after
+// another, a shuffle reduction and two exponentials each, 207 and 441.)
 constexpr int AW = 8;  // warps per CTA
 template <int VPL, int NQ>
-__global__ void __launch_bounds__(32 * AW) k_attn_simt(const SimtAttn p) {
+__global__ void __launch_bounds__(32 * AW, NQ * VPL <= 8 ? 3 : 2) k_attn_simt(const SimtAttn p) {
   constexpr int DH = 32 * VPL;
   __shared__ float4 sq4[NQ * DH / 4];          // queries, scaled
   __shared__ float so[AW][NQ][DH];             // warps' outputs
@@ -76,18 +77,37 @@ __global__ void __launch_bounds__(32 * AW) k_attn_simt(const SimtAttn p) {
   for (int b = warp; b <= kmax / 32; b += AW) {
     // a block lies in one page (its slots past the last key hold finite values)
     const float *kp = c + v.offset(p.layer, 0, g, 32 * b), *vp = c + v.offset(p.layer, 1, g, 32 * b);
-    const int key = 32 * b + lane;
-    float s[NQ];
+    // four lanes a key, each with every fourth float4 of it; of eight keys at a
+    // time, a lane keeps the sum of the one in the pass of its own number
+    const int part = lane & 3, kr = lane >> 2, key = 32 * b + 8 * part + kr;
+    const float4 *row4 = (const float4 *)(kp + (size_t)kr * DH) + part;
+    float s[NQ], t[4][NQ];
 #pragma unroll
-    for (int a = 0; a < NQ; ++a) s[a] = 0.f;
-#pragma unroll 8
-    for (int d = 0; d < DH / 4; ++d) {
-      const float4 k = *(const float4 *)(kp + (size_t)lane * DH + 4 * d);
+    for (int k8 = 0; k8 < 4; ++k8)
+#pragma unroll
+      for (int a = 0; a < NQ; ++a) t[k8][a] = 0.f;
+#pragma unroll(NQ == 1 ? 4 : 1)
+    for (int d = 0; d < DH / 16; ++d) {
+      float4 k[4];
+#pragma unroll
+      for (int k8 = 0; k8 < 4; ++k8) k[k8] = row4[8 * k8 * (DH / 4) + 4 * d];
 #pragma unroll
       for (int a = 0; a < NQ; ++a) {
-        const float4 x = sq4[a * (DH / 4) + d];
-        s[a] = fmaf(x.x, k.x, fmaf(x.y, k.y, fmaf(x.z, k.z, fmaf(x.w, k.w, s[a]))));
+        const float4 x = sq4[a * (DH / 4) + 4 * d + part];
+#pragma unroll
+        for (int k8 = 0; k8 < 4; ++k8)
+          t[k8][a] = fmaf(x.x, k[k8].x,
+                          fmaf(x.y, k[k8].y, fmaf(x.z, k[k8].z, fmaf(x.w, k[k8].w, t[k8][a]))));
       }
+    }
+#pragma unroll
+    for (int a = 0; a < NQ; ++a) {
+#pragma unroll
+      for (int k8 = 0; k8 < 4; ++k8) {
+        t[k8][a] += __shfl_xor_sync(0xffffffffu, t[k8][a], 1);
+        t[k8][a] += __shfl_xor_sync(0xffffffffu, t[k8][a], 2);
+      }
+      s[a] = part & 2 ? (part & 1 ? t[3][a] : t[2][a]) : (part & 1 ? t[1][a] : t[0][a]);
     }
 #pragma unroll
     for (int a = 0; a < NQ; ++a) {
@@ -116,7 +136,7 @@ __global__ void __launch_bounds__(32 * AW) k_attn_simt(const SimtAttn p) {
       const float *x = (const float *)&xv;
 #pragma unroll
       for (int a = 0; a < NQ; ++a) {
-        const float w = __shfl_sync(0xffffffffu, s[a], j);
+        const float w = __shfl_sync(0xffffffffu, s[a], (j & 7) * 4 + (j >> 3));
         if (whole || 32 * b + j <= lim[a])
 #pragma unroll
           for (int e = 0; e < VPL; ++e) o[a][e] = fmaf(w, x[e], o[a][e]);
