@@ -298,11 +298,13 @@ __device__ __forceinline__ void rope_dst(const RopeArgs &a, int hh, int i, int p
   }
 }
 
-// A pair rotated, with the rounding written out: a row's bits do not depend on how
-// many rows share its pass (kvr_margin runs two answers in one).
+// A pair rotated, with the rounding written out (x1 cos - x2 sin fused with its first
+// product, x2 cos + x1 sin with its second): left to the compiler it depended on
+// the kernel, and a row's bits must not depend on how many rows share its pass
+// (kvr_margin runs two answers in one).
 __device__ __forceinline__ void rotate(float x1, float x2, float c, float s, float &y1, float &y2) {
   y1 = __fmaf_rn(x1, c, -__fmul_rn(x2, s));  // x1, x2: copies, y may name the same pair
-  y2 = __fmaf_rn(x2, c, __fmul_rn(x1, s));
+  y2 = __fmaf_rn(x1, s, __fmul_rn(x2, c));
 }
 
 // A few rows: grid (M, ceil((H + 2G) / ROPE_HEADS)), block ROPE_HEADS * dh/2, a

@@ -4,6 +4,8 @@ attention (odd tile counts, ragged tiles, split and unsplit key ranges,
 several documents), pairs of CTAs per tile in the GEMM (ragged token tiles, a
 feature count that is an odd multiple of 128, few K blocks), vector row
 kernels."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -184,4 +186,30 @@ def test_norm_of_many_rows(d):
         _, v = model.prefill(doc).read(np.arange(n))
         err = np.abs(v[:, 0].reshape(n, -1) - want).max()
         assert err <= 8 * d * 2.0 ** -24 * np.abs(want).max(), n
+    model.close()
+
+
+def test_rope_rounding():
+    # The rotation's rounding is part of what a cache holds (saved rows are compared
+    # bit by bit): each half with one product rounded and one fused.  A document of
+    # one repeated token has the same unrotated K row everywhere, and position 0
+    # shows it; few rows, and the kernel of many
+    # (exact sums go to fp32 through float64: a double rounding would need 29 bits
+    # that happen to be a tie).
+    cfg = synth.preset("tiny", n_layers=2)
+    model = kv.Model(cfg, None, seed=0, max_context=1024, max_rows=512)
+    half = cfg["head_dim"] // 2
+    F = lambda v: Fraction(float(v))  # noqa: E731
+    for n in (40, 200):
+        k, _ = model.prefill(np.full(n, 17, np.int32)).read(np.arange(n))
+        x = k[0, 0]
+        for p in (1, 13, n - 1):
+            for t in range(0, half, 5):
+                a = p * cfg["rope_theta"] ** (-2.0 * t / cfg["head_dim"])
+                c, s = np.float32(np.cos(a)), np.float32(np.sin(a))
+                for g in range(cfg["n_kv_heads"]):
+                    x1, x2 = x[g, t], x[g, t + half]
+                    y1 = np.float32(float(F(x1) * F(c) - F(x2 * s)))
+                    y2 = np.float32(float(F(x1) * F(s) + F(x2 * c)))
+                    assert (k[p, 0, g, t], k[p, 0, g, t + half]) == (y1, y2), (n, p, t, g)
     model.close()
