@@ -121,8 +121,8 @@ kvr_status stage_flush(kvr_model *m) {
   return KVR_OK;
 }
 
-// Room for one more segment.  Those of a launch run in no order: one that
-// overwrites another goes behind it.
+// Room for one more segment (fewer than 2^32 words).  Those of a launch run in no
+// order: one that overwrites another goes behind it.
 kvr_status stage_room(kvr_model *m, const int32_t *dst, size_t count) {
   bool flush = m->staged.size() == UPLOAD_MAX;
   for (const Upload &u : m->staged) flush = flush || (dst < u.dst + u.words && u.dst < dst + count);
@@ -133,11 +133,13 @@ kvr_status stage_room(kvr_model *m, const int32_t *dst, size_t count) {
 kvr_status stage_copy(kvr_model *m, int32_t *dst, const int32_t *src, size_t count) {
   if (count == 0) return KVR_OK;
   KVR_TRY(stage_room(m, dst, count));
-  m->staged.push_back({dst, src, count});
+  m->staged.push_back({dst, src, (uint32_t)count, 0});
   return KVR_OK;
 }
 
-kvr_status stage_add(kvr_model *m, int32_t *dst, const int32_t *src, size_t count) {
+// tensor_maps: the data holds CUtensorMaps.
+kvr_status stage_add(kvr_model *m, int32_t *dst, const int32_t *src, size_t count,
+                     bool tensor_maps = false) {
   if (count == 0) return KVR_OK;
   if (count > m->stage_cap) return fail(KVR_E_UNSUPPORTED, "staging overflow (%zu)", count);
   KVR_TRY(stage_room(m, dst, count));
@@ -148,7 +150,7 @@ kvr_status stage_add(kvr_model *m, int32_t *dst, const int32_t *src, size_t coun
   }
   int32_t *h = m->stage_h + m->stage_off;
   memcpy(h, src, count * sizeof(int32_t));
-  m->staged.push_back({dst, h, count});
+  m->staged.push_back({dst, h, (uint32_t)count, tensor_maps ? 1u : 0u});
   m->stage_off += (count + 31) / 32 * 32;
   return KVR_OK;
 }
@@ -1589,7 +1591,7 @@ kvr_status kvr_repair_batch(kvr_model *m, const kvr_repair_req *reqs, int32_t n_
   KVR_TRY(grow_scratch(m, m->batch_scratch, m->batch_scratch_bytes, host.size() * 4,
                        "batch tables"));
   char *tab = (char *)m->batch_scratch;
-  kvr_status st = stage_add(m, (int32_t *)tab, host.data(), host.size());
+  kvr_status st = stage_add(m, (int32_t *)tab, host.data(), host.size(), all_tm);
   if (!st) st = stage_add(m, m->pos_d, P.data(), M);
   if (!st) st = stage_add(m, m->rowdoc_d, rowdoc.data(), M);
   if (!st) {
@@ -2008,7 +2010,7 @@ static kvr_status margin_one_pass(kvr_model *m, const kvr_cache *c,
   for (int i = 0; i < c->n_pages; ++i)
     ((int32_t *)(hb + mb + vb + pb))[i] = i < tail ? i : c->n_pages + i - tail;
   const StageScope scope{m};
-  KVR_TRY(stage_add(m, (int32_t *)dev, host.data(), host.size()));
+  KVR_TRY(stage_add(m, (int32_t *)dev, host.data(), host.size(), true));
   const size_t page_b = dm.page_elems() * dm.es();
   if (c->n % KVR_PAGE)
     KVR_TRY(stage_copy(m, (int32_t *)((char *)c->pages + c->n_pages * page_b),

@@ -118,6 +118,9 @@ __global__ void k_embed_rows(const T *embed, const int32_t *tokens,
 // Bound by a round trip to the host.  A copy engine takes
 // 3.2 us a segment, one after another, and more to hand over to the kernels:
 // the 68 segments of 64 edits in 16 documents took 230 us, k_upload 2.7.
+// Tensor maps are read through the tensor-map proxy: every thread that stores part
+// of one releases its stores to it, the other half of the fence that the attention
+// kernels execute before they use a map.  Each call overwrites the last one's maps.
 constexpr int UP_THREADS = 256, UP_WORDS = 4;
 template <int N>
 struct UploadList {
@@ -134,6 +137,7 @@ __global__ void __launch_bounds__(UP_THREADS) k_upload(const __grid_constant__ U
 #pragma unroll
   for (int k = 0; k < UP_WORDS; ++k)
     if (i0 + k * UP_THREADS < u.words) u.dst[i0 + k * UP_THREADS] = v[k];
+  if (u.tensor_maps) asm volatile("fence.proxy.tensormap::generic.release.gpu;" ::: "memory");
 }
 
 // One block per row (d <= 8192, d % 4 == 0), each load issued before its
@@ -694,7 +698,7 @@ void launch_fill_f32(float *dst, float v, size_t n, cudaStream_t s) {
 
 void launch_upload(const Upload *u, int n, cudaStream_t s) {
   size_t most = 1;
-  for (int i = 0; i < n; ++i) most = std::max(most, u[i].words);
+  for (int i = 0; i < n; ++i) most = std::max<size_t>(most, u[i].words);
   const dim3 grid((unsigned)((most + UP_THREADS * UP_WORDS - 1) / (UP_THREADS * UP_WORDS)), n);
   auto go = [&](auto list) {  // few segments: a launch without the larger list's bytes
     std::copy(u, u + n, list.u);

@@ -204,7 +204,8 @@ struct TcWorkspace {
 struct Upload {
   int32_t *dst;
   const int32_t *src;
-  size_t words;
+  uint32_t words;
+  uint32_t tensor_maps;  // 1: the segment holds CUtensorMaps, which TMA reads
 };
 constexpr int UPLOAD_MAX = 128;  // segments of one launch (3 KB of arguments)
 

@@ -82,6 +82,38 @@ def test_attention_pairs_of_several_documents():
     model.close()
 
 
+@pytest.mark.parametrize("rows", [20, 500])
+def test_batches_of_other_documents_in_turn(rows):
+    # every batch, and a margin, puts its documents' tensor maps where the last one's
+    # were: documents of other lengths and in another order, without a pause between
+    cfg = small_cfg(n_heads=8, n_kv_heads=2, head_dim=128)
+    W = synth.weights(cfg, 0)
+    model = kv.Model(cfg, None, seed=0, max_context=4096, max_rows=4096)
+    docs = [loaded(model, cfg, n, 30 + n) for n in (2300, 1501, 700, 1100)]
+    rng = np.random.default_rng(rows)
+    done = []
+    for pick in ((0, 1), (2, 3, 0), (1, 0), (3, 2)):
+        reqs = []
+        for i in pick:
+            cache, ref = docs[i]
+            s = int(rng.integers(0, 100))
+            new = synth.edit_tokens(3 + s, ref.tokens[s:s + 5], cfg["vocab"])
+            A = np.sort(rng.permutation(np.arange(s + 5, cache.n))[:rows])
+            reqs.append((cache, [(s, new)], A))
+            docs[i] = (cache, oracle.repair(cfg, W, ref, new, s, A))
+            done.append((i, np.concatenate([np.arange(s, s + 5), A])))
+        model.repair_batch(reqs)
+    prompt, a, b = (synth.fill_tokens(7 + i, c, cfg["vocab"], 13) for i, c in enumerate((9, 5, 3)))
+    for i in (1, 2):
+        got = model.margin(docs[i][0], prompt, a, b)
+        want = (oracle.answer_logprob(cfg, W, docs[i][1], prompt, a)
+                - oracle.answer_logprob(cfg, W, docs[i][1], prompt, b))
+        assert abs(got - want) <= TOL * max(1.0, abs(want))
+    for i, P in done:
+        check_rows(cfg, *docs[i], P)
+    model.close()
+
+
 @pytest.mark.parametrize("M", [961, 1537])
 def test_gemm_pairs_of_ctas(M):
     # 7040, 4224 and 8576 output features: odd multiples of 128, so the last
