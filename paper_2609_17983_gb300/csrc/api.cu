@@ -18,6 +18,7 @@
 #include <string>
 #include <vector>
 
+#include "host_rules.cuh"
 #include "kvr_internal.cuh"
 
 using namespace kvr;
@@ -710,22 +711,46 @@ kvr_status grow_scratch(kvr_model *m, void *&buf, size_t &have, size_t need, con
   return KVR_OK;
 }
 
+// The driver's view of a host address (all false where it knows none).
+HostRange host_range(const void *p) {
+  using Fn = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+  static const Fn fn = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return (Fn)f;
+  }();
+  uint64_t type = 0, managed = 0, access = 0;  // of one to eight bytes written
+  CUdeviceptr device = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute at[] = {
+      CU_POINTER_ATTRIBUTE_MEMORY_TYPE,      CU_POINTER_ATTRIBUTE_IS_MANAGED,
+      CU_POINTER_ATTRIBUTE_ACCESS_FLAGS,     CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+      CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void *out[] = {&type, &managed, &access, &device, &start, &size};
+  HostRange r;
+  if (!fn || fn(6, at, out, (CUdeviceptr)p) != CUDA_SUCCESS) return r;
+  r.page_locked = type == CU_MEMORYTYPE_HOST && !managed;
+  r.writable = access == CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE;
+  r.device = (uintptr_t)device;
+  r.start = (uintptr_t)start;
+  r.size = size;
+  return r;
+}
+
 // Whether n_pos rows (bytes of K, as many of V) go to the host by the kernel's own
 // stores (launch_cache_read_host): into page-locked memory that the device
-// writes directly.  Measured against gather, two copies and the flag's: 41 ->
-// 23 us for 1.3 MB, 48 -> 30 for 2.7, 142 -> 126 for 20, 488 -> 448 for 82; the
-// link (180 GB/s) bounds the large ones either way.
+// writes directly, all of it in one range.  Measured against gather, two copies and
+// the flag's: 41 -> 23 us for 1.3 MB, 48 -> 30 for 2.7, 142 -> 126 for 20, 488 -> 448
+// for 82; the link (180 GB/s) bounds the large ones either way.
 bool host_read_direct(int n_pos, int max_pos, size_t bytes, const void *k_out, const void *v_out) {
   if (n_pos > max_pos || bytes >= (size_t)1 << 35 || (((uintptr_t)k_out | (uintptr_t)v_out) & 15))
     return false;
-  for (const void *p : {k_out, v_out}) {
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (a.type != cudaMemoryTypeHost || a.devicePointer != p) return false;
-  }
+  for (const void *p : {k_out, v_out})
+    if (!device_stores_fit((uintptr_t)p, bytes, host_range(p))) return false;
   return true;
 }
 
