@@ -18,7 +18,6 @@
 #include <string>
 #include <vector>
 
-#include "host_rules.cuh"
 #include "kvr_internal.cuh"
 
 using namespace kvr;
@@ -190,7 +189,9 @@ kvr_status gemm(kvr_model *m, int cls, const void *X, const void *W, const CUten
     return launch_check(m, 1);
   }
   GemmArgs g{X, W, bias, Y, M, N, K, K, ldy, dm.dtype, epi == GEMM_EPI_ACCUM};
-  launch_gemm_simt(g, epi == GEMM_EPI_SWIGLU ? m->act : nullptr, m->num_sms, m->stream);
+  if (const char *e =
+          launch_gemm_simt(g, epi == GEMM_EPI_SWIGLU ? m->act : nullptr, m->num_sms, m->stream))
+    return fail(KVR_E_CUDA, "FFMA GEMM (M=%d N=%d K=%d): %s", M, N, K, e);
   return launch_check(m, 1);
 }
 

@@ -515,13 +515,8 @@ __global__ void __launch_bounds__(NT, 1)
 template <int DH>
 const char *run(const CUtensorMap &tm, const PairParams &p, int n_pairs, cudaStream_t s) {
   constexpr size_t smem = 1024 + (2 * QV + NSLOT * CH) * (size_t)DH * 2;
-  static bool set = false;
-  if (!set) {
-    cudaError_t e = cudaFuncSetAttribute(k_attn_pair<DH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cudaGetErrorString(e);
-    set = true;
-  }
+  static PerDevice<size_t> limit;
+  if (const char *e = smem_opt_in(limit, k_attn_pair<DH>, smem)) return e;
   dim3 grid(p.n_splits, p.G, n_pairs);
   launch_pdl(k_attn_pair<DH>, grid, NT, smem, s, tm, p);
   cudaError_t e = cudaGetLastError();

@@ -396,13 +396,8 @@ template <int DH>
 const char *run(const AttnTcParams &p, int max_mq, cudaStream_t s) {
   constexpr int smem = MAXQ * DH * 2 + 4 * CHUNK * DH * 2;
   const int warps = (max_mq + 15) / 16;
-  static bool set = false;
-  if (!set) {
-    cudaError_t e = cudaFuncSetAttribute(k_attn_tc<DH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return cudaGetErrorString(e);
-    set = true;
-  }
+  static PerDevice<size_t> limit;
+  if (const char *e = smem_opt_in(limit, k_attn_tc<DH>, smem)) return e;
   dim3 grid(p.n_splits, p.G, p.n_blocks);
   launch_pdl(k_attn_tc<DH>, grid, warps * 32, smem, s, p);
   if (p.n_splits > 1) {

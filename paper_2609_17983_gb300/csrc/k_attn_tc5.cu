@@ -539,13 +539,8 @@ constexpr size_t smem_bytes() {
 template <int DH>
 const char *run(const CUtensorMap &tm, const Attn5Params &p, cudaStream_t s) {
   constexpr size_t smem = smem_bytes<DH>();
-  static bool set = false;
-  if (!set) {
-    cudaError_t e = cudaFuncSetAttribute(k_attn_tc5<DH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cudaGetErrorString(e);
-    set = true;
-  }
+  static PerDevice<size_t> limit;
+  if (const char *e = smem_opt_in(limit, k_attn_tc5<DH>, smem)) return e;
   dim3 grid(p.n_splits, p.G, p.n_blocks);
   launch_pdl(k_attn_tc5<DH>, grid, NT5, smem, s, tm, p);
   cudaError_t e = cudaGetLastError();

@@ -463,7 +463,6 @@ bool gemm_pair_takes(int M, int N, int K, int epi) {
 
 const char *launch_gemm_pair(const GemmArgs &g, const CUtensorMap &tmW, int epi, void *out2,
                              int ld2, const TcWorkspace &ws, cudaStream_t s) {
-  static int smem_limit = -1, max_clusters = 0;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
@@ -474,27 +473,31 @@ const char *launch_gemm_pair(const GemmArgs &g, const CUtensorMap &tmW, int epi,
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (smem_limit < 0) {
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa{};
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (cudaFuncGetAttributes(&fa, k_gemm_pair) != cudaSuccess) return "kernel attributes";
-    const int lim = optin - (int)fa.sharedSizeBytes;
-    if (cudaFuncSetAttribute(k_gemm_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) !=
-        cudaSuccess)
-      return "cannot raise the dynamic shared memory limit";
-    // pairs that fit at once: stream-K's owners wait for other clusters' parts
+  // per device: the shared memory a CTA may use, and the pairs that fit at once
+  struct Fit {
+    int smem = 0, clusters = 0;
+  };
+  static PerDevice<size_t> limit;
+  static PerDevice<Fit> fits;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const Fit fit = fits.with(dev, [&](Fit &f) {
+    if (f.clusters > 0) return f;
+    Fit x;
+    x.smem = smem_opt_in_all(limit, k_gemm_pair);
     cfg.gridDim = dim3(ws.num_sms / 2 * 2);
-    cfg.dynamicSmemBytes = lim;
-    if (cudaOccupancyMaxActiveClusters(&max_clusters, (void *)k_gemm_pair, &cfg) != cudaSuccess ||
-        max_clusters < 1)
-      return "no cluster of two CTAs fits";
-    smem_limit = lim;
-  }
+    cfg.dynamicSmemBytes = x.smem;
+    if (x.smem < 0 ||
+        cudaOccupancyMaxActiveClusters(&x.clusters, (void *)k_gemm_pair, &cfg) != cudaSuccess)
+      x.clusters = 0;
+    if (x.clusters > 0) f = x;
+    return x;
+  });
+  if (fit.smem < 0) return "cannot raise the dynamic shared memory limit";
+  if (fit.clusters < 1) return "no cluster of two CTAs fits";
   PairGemm p{};
-  const int clusters = max_clusters < ws.num_sms / 2 ? max_clusters : ws.num_sms / 2;
-  cfg.dynamicSmemBytes = configure(p, g.M, g.N, g.K, clusters, smem_limit);
+  const int clusters = fit.clusters < ws.num_sms / 2 ? fit.clusters : ws.num_sms / 2;
+  cfg.dynamicSmemBytes = configure(p, g.M, g.N, g.K, clusters, fit.smem);
   cfg.gridDim = dim3(2 * p.clusters);
   p.Y = g.Y;
   p.ldy = g.ldy;

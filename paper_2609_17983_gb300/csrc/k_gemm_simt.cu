@@ -168,41 +168,33 @@ __global__ void __launch_bounds__(NTH) k_gemm_simt(const SimtGemm p) {
 }
 
 template <typename T, int BM, int BN, int KS, int KC>
-void run(const SimtGemm &p, cudaStream_t s) {
+const char *run(const SimtGemm &p, cudaStream_t s) {
   constexpr int st = 2 * (BM + BN) * (KC + 4) * 4, red = KS > 1 ? KS * BM * BN * 4 : 0;
   constexpr int smem = st > red ? st : red;
-  static bool set = false;
-  if (!set) {  // above 48 KB only by opt-in
-    cudaFuncSetAttribute(k_gemm_simt<T, BM, BN, KS, KC>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    set = true;
-  }
+  static PerDevice<size_t> limit;  // above 48 KB only by opt-in
+  if (const char *e = smem_opt_in(limit, k_gemm_simt<T, BM, BN, KS, KC>, smem)) return e;
   launch_pdl(k_gemm_simt<T, BM, BN, KS, KC>, dim3((p.N + BN - 1) / BN, (p.M + BM - 1) / BM), NTH,
              smem, s, p);
+  return nullptr;
 }
 
 template <typename T>
-void pick(const SimtGemm &p, int num_sms, cudaStream_t s) {
+const char *pick(const SimtGemm &p, int num_sms, cudaStream_t s) {
   auto tiles = [&](int bm, int bn) {
     return (long long)((p.M + bm - 1) / bm) * ((p.N + bn - 1) / bn);
   };
-  if (tiles(64, 64) >= 2 * num_sms)
-    run<T, 64, 64, 1, 32>(p, s);
-  else if (tiles(32, 32) >= num_sms)
-    run<T, 32, 32, 4, 128>(p, s);
-  else
-    run<T, 16, 32, 8, 128>(p, s);
+  if (tiles(64, 64) >= 2 * num_sms) return run<T, 64, 64, 1, 32>(p, s);
+  if (tiles(32, 32) >= num_sms) return run<T, 32, 32, 4, 128>(p, s);
+  return run<T, 16, 32, 8, 128>(p, s);
 }
 
 }  // namespace
 
-void launch_gemm_simt(const GemmArgs &g, void *act, int num_sms, cudaStream_t s) {
-  if (g.M <= 0 || g.N <= 0) return;
+const char *launch_gemm_simt(const GemmArgs &g, void *act, int num_sms, cudaStream_t s) {
+  if (g.M <= 0 || g.N <= 0) return nullptr;
   SimtGemm p{g.X, g.W, g.bias, g.Y, act, g.M, g.N, g.K, g.ldx, g.ldy, g.accumulate};
-  if (g.dtype == KVR_DTYPE_BF16)
-    pick<__nv_bfloat16>(p, num_sms, s);
-  else
-    pick<float>(p, num_sms, s);
+  return g.dtype == KVR_DTYPE_BF16 ? pick<__nv_bfloat16>(p, num_sms, s)
+                                   : pick<float>(p, num_sms, s);
 }
 
 }  // namespace kvr

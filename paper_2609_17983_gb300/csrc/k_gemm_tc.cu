@@ -978,10 +978,13 @@ int choose_cluster(int M, int N, int num_sms, size_t smem) {
   int P = num_sms / T;
   if (P > 8) P = 8;
   if (P < 2 || T * P * 4 < num_sms * 3) return 0;
-  static int cache_p[16] = {0}, cache_ok[16] = {0};
-  static size_t cache_smem[16] = {0};
-  for (int i = 0; i < 16; ++i)
-    if (cache_p[i] == P && cache_smem[i] == smem) return cache_ok[i] >= T ? P : 0;
+  struct Known {  // clusters of p CTAs with this much shared memory that fit at once
+    int p[16] = {0}, fit[16] = {0};
+    size_t smem[16] = {0};
+  };
+  static PerDevice<Known> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(T * P);
   cfg.blockDim = dim3(NTHREADS);
@@ -993,18 +996,22 @@ int choose_cluster(int M, int N, int num_sms, size_t smem) {
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  int nc = 0;
-  if (cudaOccupancyMaxActiveClusters(&nc, (void *)k_gemm_tc, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    nc = 0;
-  }
-  for (int i = 0; i < 16; ++i)
-    if (cache_p[i] == 0) {
-      cache_p[i] = P;
-      cache_smem[i] = smem;
-      cache_ok[i] = nc;
-      break;
+  const int nc = known.with(dev, [&](Known &c) {
+    int i = 0;
+    while (i < 16 && c.p[i] && (c.p[i] != P || c.smem[i] != smem)) ++i;
+    if (i < 16 && c.p[i]) return c.fit[i];
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_gemm_tc, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
     }
+    if (i < 16) {
+      c.p[i] = P;
+      c.smem[i] = smem;
+      c.fit[i] = n;
+    }
+    return n;
+  });
   return nc >= T ? P : 0;
 }
 }  // namespace
@@ -1022,20 +1029,14 @@ namespace {
 // Dynamic shared memory this kernel may use (opt-in limit minus static);
 // < 0 on failure.
 int dyn_smem_limit() {
-  static int max_dyn = -1;
-  if (max_dyn < 0) {
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa{};
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (cudaFuncGetAttributes(&fa, k_gemm_tc) != cudaSuccess) return -1;
-    int lim = optin - (int)fa.sharedSizeBytes;
-    if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) !=
-        cudaSuccess)
-      return -1;
-    max_dyn = lim;
-  }
-  return max_dyn;
+  static PerDevice<size_t> limit;
+  static PerDevice<int> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return known.with(dev, [](int &lim) {
+    if (lim <= 0) lim = smem_opt_in_all(limit, k_gemm_tc);
+    return lim;
+  });
 }
 
 // Tiling, pipeline depth and split of an M x N x K GEMM: fills the shape
@@ -1234,13 +1235,8 @@ const char *launch_gemm_chain(const ChainStep *st, int n, const TcWorkspace &ws,
   if (st[0].norm && (n < 2 || st[1].norm)) return "a chain's first norm feeds no GEMM";
   if (nn > 0 && M > ws.num_sms) return "chain norm rows above the SM count";
   c.M = M;
-  static int set_smem = -1;
-  if (set_smem < (int)smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_chain, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return cudaGetErrorString(e);
-    set_smem = (int)smem;
-  }
+  static PerDevice<size_t> limit;
+  if (const char *e = smem_opt_in(limit, k_gemm_chain, smem)) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(ws.num_sms);
   cfg.blockDim = dim3(NTHREADS);

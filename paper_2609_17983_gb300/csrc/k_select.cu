@@ -671,9 +671,8 @@ const char *launch_topk(const unsigned long long *keys, int n, int s_end, int K,
   if (c < 0) c = 0;
   size_t smem = (size_t)c * sizeof(unsigned long long);
   if (smem >= 32 * 1024) {  // the default 48 KB limit also covers static shared memory
-    cudaError_t e = cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return cudaGetErrorString(e);
+    static PerDevice<size_t> limit;
+    if (const char *e = smem_opt_in(limit, k_topk, smem)) return e;
   }
   k_topk<<<1, TOPK_THREADS, smem, s>>>(keys, c, s_end, K, nonzero_only, out, count, gen,
                                        flag_in, flag_out);
@@ -743,7 +742,8 @@ int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_
                            : (bf16 ? k_attn_select_logits<__nv_bfloat16, 64>
                                    : k_attn_select_logits<float, 64>);
   // fp32 at dh 128, plus the trace build's static shared memory, passes 48 KB
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static PerDevice<size_t> limit[2][2];  // (an error shows at the launch)
+  smem_opt_in(limit[bf16][dm.dh == 128], kern, smem);
   // one wave: the chunks spread evenly over the CTAs that fit at once
   const int nch = sel_chunks(c), fit = (bf16 ? 6 : 4) * num_sms / (dm.G * nqt * layers);
   const int per = fit < 1 ? nch : (nch + fit - 1) / fit;

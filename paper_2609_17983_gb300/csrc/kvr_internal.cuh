@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "../../include/kvrepair.h"
+#include "host_rules.cuh"
 
 namespace kvr {
 
@@ -447,6 +448,33 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Opts the kernel into `bytes` of dynamic shared memory on the current device (models
+// of one process may live on several); null, or what failed.  One `state` per kernel.
+template <typename... KArgs>
+inline const char *smem_opt_in(PerDevice<size_t> &state, void (*kernel)(KArgs...), size_t bytes) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = (cudaError_t)raise_to(state, dev, bytes, [&](size_t b) {
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+    });
+  return e == cudaSuccess ? nullptr : cudaGetErrorString(e);
+}
+
+// The opt-in limit of the current device less the kernel's static shared memory, opted
+// into; negative when that fails.
+template <typename... KArgs>
+inline int smem_opt_in_all(PerDevice<size_t> &state, void (*kernel)(KArgs...)) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa{};
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaFuncGetAttributes(&fa, kernel) != cudaSuccess)
+    return -1;
+  const int lim = optin - (int)fa.sharedSizeBytes;
+  return smem_opt_in(state, kernel, (size_t)lim) ? -1 : lim;
+}
+
 // Message returned by kvr_last_error() on the calling thread.
 void set_last_error(const char *msg);
 
@@ -517,8 +545,9 @@ struct GemmArgs {
   int accumulate;  // 1: Y += result
 };
 // FFMA GEMM; act (optional): W's rows are interleaved gate/up and the SwiGLU of
-// their products goes to act [M][N / 2] in the model dtype instead of Y.
-void launch_gemm_simt(const GemmArgs &g, void *act, int num_sms, cudaStream_t s);
+// their products goes to act [M][N / 2] in the model dtype instead of Y.  Null, or
+// what failed.
+const char *launch_gemm_simt(const GemmArgs &g, void *act, int num_sms, cudaStream_t s);
 
 // Tensor-core GEMM (bf16, N % 128 == 0, K % 64 == 0).  Epilogues:
 enum { GEMM_EPI_STORE = 0, GEMM_EPI_ACCUM = 1, GEMM_EPI_SWIGLU = 2 };

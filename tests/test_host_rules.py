@@ -1,4 +1,4 @@
-"""The host side's rules, compiled alone from csrc/host_rules.cuh (no GPU needed)."""
+"""The host side's rules, compiled alone from csrc (no GPU needed)."""
 import os
 import shutil
 import subprocess
@@ -50,3 +50,54 @@ int main() {
 }
 """)
     assert out == ["1", "1"] + ["0"] * 10
+
+
+def test_settings_are_raised_on_each_device_and_never_lowered(tmp_path):
+    out = run(tmp_path, r"""
+#include <atomic>
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "host_rules.cuh"
+using namespace kvr;
+int main() {
+  PerDevice<size_t> s;
+  std::vector<std::pair<int, size_t>> calls;
+  auto raise = [&](int dev, size_t bytes, int err = 0) {
+    const int e = raise_to(s, dev, bytes, [&](size_t b) { calls.push_back({dev, b}); return err; });
+    std::printf("%d:%zu ", e, calls.size());
+  };
+  raise(0, 100);     // set
+  raise(0, 100);     // known
+  raise(1, 100);     // another device: set there too
+  raise(0, 60);      // a smaller request lowers nothing
+  raise(2, 100, 7);  // a failure is reported
+  raise(2, 100);     // and not remembered
+  raise(MAX_DEVICES, 100);
+  raise(MAX_DEVICES, 100);
+  // threads with different requests: each finds its own granted when it returns
+  PerDevice<size_t> t;
+  std::atomic<size_t> granted{0};
+  std::atomic<int> low{0};
+  std::vector<std::thread> th;
+  for (size_t i = 1; i <= 8; ++i)
+    th.emplace_back([&, i] {
+      for (size_t k = 0; k < 2000; ++k) {
+        const size_t want = i * 1000 + k;
+        raise_to(t, 0, want, [&](size_t b) { granted = b; return 0; });
+        if (granted < want) ++low;
+      }
+    });
+  for (auto &x : th) x.join();
+  std::printf("%d", low.load());
+}
+""")
+    assert out == ["0:1", "0:1", "0:2", "0:2", "7:3", "0:4", "0:5", "0:6", "0"]
+
+
+def test_kernels_take_shared_memory_through_that_rule():
+    # a process-wide "already set" would leave a model on a second device without it
+    for name in sorted(os.listdir(CSRC)):
+        text = open(os.path.join(CSRC, name)).read()
+        uses = text.count("cudaFuncSetAttribute(")
+        assert uses == (1 if name == "kvr_internal.cuh" else 0), name
