@@ -20,9 +20,9 @@
 // R + c + kC to cluster c in round k (neighbouring clusters share weight or
 // token tiles and walk K in step, so each comes from DRAM once).  Of the R
 // tiles left over each goes to s = floor(C / R) clusters, equal parts of K --
-// again in step -- that the tile's first cluster sums in part order from what
-// the others publish.  The parts come first, so that their sum runs beside
-// the MMAs of the whole tiles.  (Whole tiles alone: 2608 rows of a 4096-wide
+// again in step -- that the cluster of the last part sums in part order from what
+// the others publish (the waits: pair_split.cuh).  The parts come first, so that
+// their sum runs beside the MMAs of the whole tiles.  (Whole tiles alone: 2608 rows of a 4096-wide
 // projection leave 24 of 76 clusters' slots of the last round in use.  Stream-K
 // ranges over the left tiles, each cluster at K blocks of its own, re-read
 // operands from DRAM: 66 us there, and 106 against a floor of 55 us for 904
@@ -38,6 +38,7 @@
 
 #include "gemm_epilogue.cuh"
 #include "kvr_internal.cuh"
+#include "pair_split.cuh"
 #include "tc_ptx.cuh"
 
 namespace kvr {
@@ -60,12 +61,9 @@ constexpr int PRE_WAIT_STAGES = 2;    // weight stages requested before the wait
 constexpr int MIN_UNITS = 4;          // units (of KS K blocks) a part of a tile has at least
 constexpr int MAX_PARTS = 8;          // clusters a left-over tile is split over at most
 
-struct PairGemm {
-  int M, N, KB, KU;   // K blocks, and units of KS of them (the last may be short)
-  int BN, n_tiles, m_tiles;
-  int clusters;       // clusters of the grid
-  int left, parts;    // tiles 0 .. left - 1 go to `parts` clusters each
-  int rounds;         // whole tiles per cluster after them
+struct PairGemm : PairSplit {  // its units: KS K blocks (the last may be short)
+  int M, N, KB;       // K blocks
+  int BN, n_tiles;
   int stages;
   float *Y;
   int ldy;
@@ -76,35 +74,6 @@ struct PairGemm {
   float *ws;      // [CTA][2][256][128] fp32 parts (the first slot of each CTA is used)
   int *ready;     // [2 * left] published parts per split tile and CTA rank (self-resetting)
   int *dev_flag;
-};
-
-// One accumulator's worth of work of a cluster: units [ku0, ku1) of a tile.
-struct Segment {
-  int tile, ntile, mtile, ku0, ku1;
-};
-// Segments of cluster c in order: its part of a left-over tile (part c / left of
-// tile c % left), then its whole tiles.
-struct Walk {
-  int k, c;
-  __device__ Walk(const PairGemm &p, int cluster)
-      : k(cluster < p.left * p.parts ? -1 : 0), c(cluster) {}
-  __device__ bool next(const PairGemm &p, Segment &s) {
-    if (k >= p.rounds) return false;
-    s.ku0 = 0;
-    s.ku1 = p.KU;
-    if (k < 0) {
-      const int j = c / p.left;
-      s.tile = c - j * p.left;
-      s.ku0 = (int)((long long)j * p.KU / p.parts);
-      s.ku1 = (int)((long long)(j + 1) * p.KU / p.parts);
-    } else {
-      s.tile = p.left + c + k * p.clusters;
-    }
-    ++k;
-    s.ntile = s.tile / p.m_tiles;
-    s.mtile = s.tile - s.ntile * p.m_tiles;
-    return true;
-  }
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -328,13 +297,13 @@ __global__ void __launch_bounds__(NT, 1)
       const uint32_t buf = seg & 1u;
       const int t0 = g.mtile * p.BN, mv = min(p.BN, p.M - t0);
       const int n = g.ntile * TM + rank * BM + f;
-      // a part of a tile: the first cluster sums the others' parts
+      // a part of a tile: the last part's cluster sums the others' parts and its own
       const int parts = g.ku1 - g.ku0 < p.KU ? p.parts : 1;
-      const bool owner = parts == 1 || cluster < p.left;
+      const bool owner = parts == 1 || sums_parts(p, cluster);
       int *ready = p.ready + 2 * g.tile + rank;
       if (owner && parts > 1) {
-        // Every cluster's part is its first segment, waits on nothing and is
-        // published at its end; all clusters are resident.
+        // Every other cluster's part is its first segment, waits on nothing and
+        // is published at its end.
         if (et == 0) {
           volatile int *r = ready;
           const uint64_t t0w = gtime_ns();
@@ -369,14 +338,20 @@ __global__ void __launch_bounds__(NT, 1)
             if (c + j < mv) dst[(size_t)j * BM] = v[j];
           continue;
         }
-        for (int k = 1; k < parts; ++k) {  // in part order
-          const float *src =
-              p.ws + ((size_t)(2 * (cluster + k * p.left) + rank) * 2 * 256 + c) * BM + f;
-          float x[CC];
+        if (parts > 1) {  // in part order, this cluster's own last
+          float s[CC];
+          for (int k = 0; k < parts - 1; ++k) {
+            const float *src =
+                p.ws +
+                ((size_t)(2 * part_cluster(p, g.tile, k) + rank) * 2 * 256 + c) * BM + f;
+            float x[CC];
 #pragma unroll
-          for (int j = 0; j < CC; ++j) x[j] = c + j < mv ? __ldcg(src + (size_t)j * BM) : 0.f;
+            for (int j = 0; j < CC; ++j) x[j] = c + j < mv ? __ldcg(src + (size_t)j * BM) : 0.f;
 #pragma unroll
-          for (int j = 0; j < CC; ++j) v[j] += x[j];
+            for (int j = 0; j < CC; ++j) s[j] = k ? s[j] + x[j] : x[j];
+          }
+#pragma unroll
+          for (int j = 0; j < CC; ++j) v[j] = s[j] + v[j];
         }
         if (n < p.N) {
           epilogue16(p, t0 + c, n, v, mv - c);

@@ -101,3 +101,63 @@ def test_kernels_take_shared_memory_through_that_rule():
         text = open(os.path.join(CSRC, name)).read()
         uses = text.count("cudaFuncSetAttribute(")
         assert uses == (1 if name == "kvr_internal.cuh" else 0), name
+
+
+def test_paired_gemm_waits_only_for_clusters_before_the_waiting_one(tmp_path):
+    # every split of a launch's tiles: each unit of K of each tile is computed once,
+    # the parts of a tile by clusters in part order, the last of which sums them --
+    # one of a higher number than all it waits for, so dispatched after them
+    out = run(tmp_path, r"""
+#include <cstdio>
+#include <map>
+#include <vector>
+#include "pair_split.cuh"
+using namespace kvr;
+int main() {
+  int checked = 0;
+  for (int clusters : {1, 2, 3, 7, 70, 76})
+    for (int tiles = 1; tiles <= 3 * clusters; tiles += 1 + clusters / 9)
+      for (int KU : {1, 4, 9, 33, 112})
+        for (int most = 1; most <= 8; ++most) {
+          PairSplit p{KU, 3, clusters, tiles % clusters, 1, tiles / clusters};
+          if (p.left) p.parts = clusters / p.left < most ? clusters / p.left : most;
+          if (p.parts > KU) p.parts = KU;
+          if (!p.rounds) p.clusters = p.left * p.parts;
+          std::map<int, std::vector<int>> units;   // of a tile: times computed
+          std::map<int, int> sum;                  // of a split tile: its summing cluster
+          for (int c = 0; c < p.clusters; ++c) {
+            Walk w(p, c);
+            Segment s;
+            for (bool first = true; w.next(p, s); first = false) {
+              auto &u = units[s.tile];
+              u.resize(KU);
+              for (int k = s.ku0; k < s.ku1; ++k) ++u[k];
+              if (s.ku1 - s.ku0 == KU) continue;
+              if (!first || s.ntile * 3 + s.mtile != s.tile) return std::puts("order"), 0;
+              if (sums_parts(p, c)) {
+                if (sum.count(s.tile) || s.ku1 != KU) return std::puts("sums"), 0;
+                sum[s.tile] = c;
+              }
+            }
+          }
+          if ((int)units.size() != tiles) return std::puts("tiles"), 0;
+          for (auto &u : units)
+            for (int n : u.second)
+              if (n != 1) return std::puts("units"), 0;
+          if (p.parts > 1)
+            for (int t = 0; t < p.left; ++t)
+              for (int k = 0; k < p.parts; ++k) {
+                const int c = part_cluster(p, t, k);
+                Walk w(p, c);
+                Segment s;
+                if (!w.next(p, s) || s.tile != t || s.ku0 != k * KU / p.parts)
+                  return std::puts("parts"), 0;
+                if (!sum.count(t) || (k + 1 < p.parts ? c >= sum[t] : c != sum[t]))
+                  return std::puts("waits"), 0;
+                ++checked;
+              }
+        }
+  std::puts(checked > 1000 ? "ok" : "few");
+}
+""")
+    assert out == ["ok"]
