@@ -599,7 +599,10 @@ struct AnswerIds {
 };
 __device__ __forceinline__ void lse_add(float &m, float &s, float m2, float s2) {
   const float mm = fmaxf(m, m2);
-  if (mm == -INFINITY) return;  // both empty
+  if (mm == -INFINITY) {  // both empty, or NaN (which the maximum passes over)
+    s += s2;
+    return;
+  }
   s = s * expf(m - mm) + s2 * expf(m2 - mm);
   m = mm;
 }
@@ -619,8 +622,12 @@ __global__ void __cluster_dims__(LP_CTAS, 1, 1) __launch_bounds__(LP_THREADS)
   auto add = [&](const float *v, int n) {
     float mx = m;
     for (int j = 0; j < n; ++j) mx = fmaxf(mx, v[j]);
-    if (mx == -INFINITY) return;
     float t = 0.f;
+    if (mx == -INFINITY) {  // nothing above the lowest value, but perhaps a NaN
+      for (int j = 0; j < n; ++j) t += v[j] == -INFINITY ? 0.f : v[j];
+      s += t;
+      return;
+    }
     for (int j = 0; j < n; ++j) t += expf(v[j] - mx);
     s = s * expf(m - mx) + t;
     m = mx;

@@ -153,6 +153,21 @@ def test_answer_logprob_row_widths(vocab):
     model.close()
 
 
+@pytest.mark.parametrize("vocab,ids", [(1021, [0]), (1021, [1020]), (1024, [8, 9, 10, 11]),
+                                       (1024, [700]), (18, [17])])
+def test_answer_logprob_of_a_nan(vocab, ids):
+    # a NaN among the logits, also where a thread sees nothing else: the
+    # log-softmax of the row is NaN
+    cfg = synth.preset("tiny", vocab=vocab)
+    W = synth.weights(cfg, 0)
+    W["lm_head"] = W["lm_head"].copy()
+    W["lm_head"][ids] = np.nan
+    model = kv.Model(cfg, W, max_context=256, max_rows=256)
+    cache = model.prefill(np.arange(2, 82, dtype=np.int32) % vocab)
+    assert np.isnan(model.answer_logprob(cache, np.array([3, 4], np.int32), np.array([5], np.int32)))
+    model.close()
+
+
 @pytest.mark.parametrize("policy,edit,n", [("attention", 3, 1500), ("attention", 220, 1500),
                                            ("cacheblend", 3, 1500), ("cacheblend", 3, 700)])
 def test_model_selectors_over_layer_groups(policy, edit, n):
