@@ -115,8 +115,9 @@ __global__ void __launch_bounds__(32 * AW, NQ * VPL <= 8 ? 3 : 2) k_attn_simt(co
       float mx = s[a];
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-      if (mx == -INFINITY) {  // no key of the block is this query's
-        s[a] = 0.f;
+      if (mx == -INFINITY) {  // no key of the block is this query's, or its scores are NaN
+        s[a] = isnan(s[a]) ? s[a] : 0.f;
+        l[a] += s[a];
         continue;
       }
       const float mn = fmaxf(m[a], mx), corr = expf(m[a] - mn);

@@ -90,3 +90,23 @@ def test_fp32_attention_of_several_documents(H, G, rows):
     for (cache, _, A), ref in zip(reqs, want):
         check_rows(cfg, cache, ref, np.concatenate([np.arange(7, 10), A]))
     model.close()
+
+
+@pytest.mark.parametrize("rows", [1, 60, 120])
+def test_attention_keeps_a_lone_nan(rows):
+    # fresh keys are NaN (their projection holds one), stale keys are finite: a row at
+    # the start of a block of 32 keys sees no other key of that block, and its output,
+    # so the next layer's values, is NaN; rows for each number of queries per CTA
+    cfg = synth.preset("tiny", n_layers=2)
+    W = synth.weights(cfg, 0)
+    W["layers"][0]["wk"] = W["layers"][0]["wk"].copy()
+    W["layers"][0]["wk"][:, 3] = np.nan
+    model = kv.Model(cfg, W, max_context=4096, max_rows=512)
+    n = 32 * 121
+    cache, _ = loaded(model, cfg, n, 5)
+    at = 32 * np.arange(1, rows + 1)
+    cache.repair(np.zeros(0, np.int32), 0, at)
+    k, v = cache.read(at)
+    assert np.isnan(k[:, 0]).all() and np.isnan(v[0, 1]).all()
+    assert np.isnan(v[:, 1]).all() and np.isfinite(v[:, 0]).all()
+    model.close()
