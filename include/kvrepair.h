@@ -235,6 +235,9 @@ kvr_status kvr_answer_logprob(kvr_model *model, const kvr_cache *cache, const in
  * teacher-forced log-probability (kvr_answer_logprob) of the answer a_new
  * minus that of a_old, both after the same prompt.  MR (Eq. 2) is
  * (m_repaired - m_stale) / (m_oracle - m_stale) over three cache states.
+ * Where both answers run in one pass, the second one's K/V take two pages of the
+ * model's, allocated with its first such margin (without room for them the
+ * answers run one after the other, with the same result).
  * Errors as kvr_answer_logprob, and KVR_E_INVAL for a NULL margin_out. */
 kvr_status kvr_margin(kvr_model *model, const kvr_cache *cache, const int32_t *prompt,
                       int32_t m_prompt, const int32_t *a_new, int32_t m_new,

@@ -212,6 +212,7 @@ struct Rows {
   int n_pairs = 0;
   const CUtensorMap *tm_kv = nullptr;        // TMA view of the single document's pages
   const CUtensorMap *tmaps = nullptr;        // device [docs]: TMA views of a batch's pages
+  int tail_page = NO_TAIL, tail_docs = 0;    // launch_attention_tc5's
   bool tc5 = false;                          // attention on tcgen05 (set by plan_attention)
   // kvr_repair_read: RoPE also writes the rows' K/V to rows_out (K then V,
   // [M][L][G][dh]); after every rd_every layers an event marks them ready
@@ -459,7 +460,7 @@ kvr_status attention(kvr_model *m, const Rows &r, int l) {
                   : launch_attention_tc5(m->qb, r.pos, r.blocks, r.n_blocks, r.n_splits, dm, l,
                                          r.single.pages, r.single.table, tm, m->attn_ws_o,
                                          m->attn_ws_ml, m->attn, m->dev_flag, m->stream, views,
-                                         r.tmaps);
+                                         r.tmaps, r.tail_page, r.tail_docs);
       if (!e)
         e = launch_attention_combine(r.blocks, r.n_blocks, r.max_block_rows, r.n_splits, dm,
                                      m->attn_ws_o, m->attn_ws_ml, m->attn, m->stream,
@@ -936,6 +937,7 @@ void kvr_model_free(kvr_model *m) {
   if (m->rd_cap) cudaStreamDestroy(m->rd_cap);
   dev_free(m->sel_scratch);
   dev_free(m->batch_scratch);
+  dev_free(m->spare_pages);
   dev_free(m->tcw.counters);
   dev_free(m->blocks_d);
   dev_free(m->attn_ws_o);
@@ -1296,9 +1298,7 @@ static kvr_status check_context(const kvr_model *m, const int32_t *tokens, int32
 // unless they are written before they are first read (slots never written
 // hold finite values, so a masked key meets probability 0 and never 0 * NaN),
 // the identity block table, the device copy of the tokens and, for bf16, the
-// TMA view of the page pool.  Behind the table's pages the pool holds
-// KVR_SPARE_PAGES more, for a second continuation past n (kvr_margin).
-// Enqueued on the model's stream.
+// TMA view of the page pool.  Enqueued on the model's stream.
 static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_cache **out) {
   const Dims &dm = m->dims;
   kvr_cache *c = new kvr_cache();
@@ -1308,8 +1308,7 @@ static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_
   c->cap = (n + KVR_QUERY_RESERVE + KVR_PAGE - 1) / KVR_PAGE * KVR_PAGE;
   c->n_pages = c->cap / KVR_PAGE;
   size_t page_bytes = dm.page_elems() * dm.es();
-  const int pool_pages = c->n_pages + KVR_SPARE_PAGES;
-  c->pages = dev_alloc((size_t)pool_pages * page_bytes);
+  c->pages = dev_alloc((size_t)c->n_pages * page_bytes);
   c->table = (int32_t *)dev_alloc((size_t)c->n_pages * 4);
   c->tokens_d = (int32_t *)dev_alloc((size_t)c->cap * 4);
   if (!c->pages || !c->table || !c->tokens_d) {
@@ -1322,12 +1321,12 @@ static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_
   // from n on hold slots that are read unwritten.
   const int clean = dm.max_rows % KVR_PAGE == 0 ? n / KVR_PAGE : 0;
   if (cudaMemsetAsync((char *)c->pages + (size_t)clean * page_bytes, 0,
-                      (size_t)(pool_pages - clean) * page_bytes, m->stream)) {
+                      (size_t)(c->n_pages - clean) * page_bytes, m->stream)) {
     kvr_cache_free(c);
     return fail(KVR_E_CUDA, "cache clear");
   }
   if (dm.dtype == KVR_DTYPE_BF16) {
-    const long long rows = (long long)pool_pages * dm.L * 2 * dm.G * KVR_PAGE;
+    const long long rows = (long long)c->n_pages * dm.L * 2 * dm.G * KVR_PAGE;
     c->tm_kv_ok = rows < (1ll << 31) && make_tmap_bf16(&c->tm_kv, c->pages, (int)rows, dm.dh, KVR_PAGE);
   }
   std::vector<int32_t> tab(c->n_pages);
@@ -2004,62 +2003,92 @@ static int margin_splits(const kvr_model *m, const kvr_cache *c, size_t rows0, s
   return splits[0] == splits[1] ? splits[0] : 0;
 }
 
-// Both answers in one pass, as two documents that share every page below n: the
-// second one's table ends in the cache's spare pages (the first of them a
-// copy of the page that n falls into), so that its rows' K/V past n have a
-// place of their own.  The pass streams the weights and lm_head once for both
-// (two 29-row answers on four 8B-shape layers: 1.25 -> 0.71 ms).
+// Both answers in one pass, as two documents that share every page below n: from
+// the page that n falls into on, the second one's lie in the model's spare pages
+// (copies of the cache's own, so their unwritten slots are as finite), and its
+// rows' K/V past n have a place of their own.  The pass streams the weights and
+// lm_head once for both (two 29-row answers on four 8B-shape layers: 1.25 -> 0.71
+// ms).  The tables, in the model's batch scratch: entries 0 and 1 of tensor maps,
+// views and token pointers are the documents' shared pages, 2 and 3 their tails.
+struct MarginTables {
+  size_t views, tokens, table, head, total;  // byte offsets; what is staged; all
+  explicit MarginTables(const kvr_cache *c) {
+    auto al = [](size_t x) { return (x + 255) / 256 * 256; };
+    views = al(4 * sizeof(CUtensorMap));
+    tokens = views + al(4 * sizeof(KVView));
+    table = tokens + al(4 * sizeof(void *));
+    head = table + al((size_t)c->n_pages * 4);
+    total = head + al((size_t)c->cap * 4);  // the second document's tokens, from n on
+  }
+};
+
+static kvr_status margin_scratch(kvr_model *m, const kvr_cache *c) {
+  const Dims &dm = m->dims;
+  KVR_TRY(grow_scratch(m, m->batch_scratch, m->batch_scratch_bytes, MarginTables(c).total,
+                       "margin tables"));
+  if (m->spare_pages) return KVR_OK;
+  KVR_TRY(grow_scratch(m, m->spare_pages, m->spare_bytes,
+                       KVR_SPARE_PAGES * dm.page_elems() * dm.es(), "margin pages"));
+  if (!make_tmap_bf16(&m->tm_spare, m->spare_pages,
+                      KVR_SPARE_PAGES * dm.L * 2 * dm.G * KVR_PAGE, dm.dh, KVR_PAGE)) {
+    dev_free(m->spare_pages);
+    m->spare_pages = nullptr;
+    m->spare_bytes = 0;
+    return fail(KVR_E_CUDA, "margin pages: TMA descriptor rejected");
+  }
+  return KVR_OK;
+}
+
+// After margin_scratch.
 static kvr_status margin_one_pass(kvr_model *m, const kvr_cache *c,
                                   const std::vector<int32_t> (&feed)[2], int32_t mp,
                                   const int32_t *const *answer, const int32_t *ma, int splits,
                                   double *lp) {
   const Dims &dm = m->dims;
-  auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-  const size_t tab_b = al((size_t)c->n_pages * 4), tok_b = al((size_t)c->cap * 4);
-  const size_t mb = al(2 * sizeof(CUtensorMap));
-  const size_t vb = al(2 * sizeof(KVView)), pb = al(2 * sizeof(void *));
-  // scratch: tensor maps, views, token pointers, the second document's table,
-  // its tokens (those from n on are read)
-  const size_t head = mb + vb + pb + tab_b;
-  KVR_TRY(grow_scratch(m, m->batch_scratch, m->batch_scratch_bytes, head + tok_b, "margin tables"));
+  const MarginTables mt(c);
   char *dev = (char *)m->batch_scratch;
-  int32_t *table1 = (int32_t *)(dev + mb + vb + pb), *tokens1 = (int32_t *)(dev + head);
-  std::vector<int32_t> host(head / 4);
+  std::vector<int32_t> host(mt.head / 4);
   char *hb = (char *)host.data();
-  KVView views[2] = {c->view(), c->view()};
-  views[1].table = table1;
-  const int32_t *tokens[2] = {c->tokens_d, tokens1};
-  for (int k = 0; k < 2; ++k) memcpy(hb + k * sizeof(CUtensorMap), &c->tm_kv, sizeof c->tm_kv);
-  memcpy(hb + mb, views, sizeof views);
-  memcpy(hb + mb + vb, tokens, sizeof tokens);
+  const CUtensorMap maps[4] = {c->tm_kv, c->tm_kv, c->tm_kv, m->tm_spare};
+  const KVView own = c->view();
+  const KVView views[4] = {
+      own, own, own, {m->spare_pages, (int32_t *)(dev + mt.table), dm.L, dm.G, dm.dh}};
+  int32_t *const tokens[4] = {c->tokens_d, c->tokens_d, c->tokens_d, (int32_t *)(dev + mt.head)};
+  memcpy(hb, maps, sizeof maps);
+  memcpy(hb + mt.views, views, sizeof views);
+  memcpy(hb + mt.tokens, tokens, sizeof tokens);
   const int tail = c->n / KVR_PAGE;  // the page that position n falls into
-  for (int i = 0; i < c->n_pages; ++i)
-    ((int32_t *)(hb + mb + vb + pb))[i] = i < tail ? i : c->n_pages + i - tail;
+  for (int i = tail; i < c->n_pages; ++i) ((int32_t *)(hb + mt.table))[i] = i - tail;
   const StageScope scope{m};
   KVR_TRY(stage_add(m, (int32_t *)dev, host.data(), host.size(), true));
   const size_t page_b = dm.page_elems() * dm.es();
-  if (c->n % KVR_PAGE)
-    KVR_TRY(stage_copy(m, (int32_t *)((char *)c->pages + c->n_pages * page_b),
-                       (const int32_t *)((const char *)c->pages + tail * page_b), page_b / 4));
-  std::vector<int32_t> P, doc;
+  const int pages = (c->n + (int)feed[1].size() - 1) / KVR_PAGE - tail + 1;  // its rows reach
+  KVR_TRY(stage_copy(m, (int32_t *)m->spare_pages,
+                     (const int32_t *)((const char *)c->pages + tail * page_b),
+                     pages * page_b / 4));
+  std::vector<int32_t> P, doc, tail_doc;
   for (int k = 0; k < 2; ++k) {
-    KVR_TRY(stage_add(m, (int32_t *)tokens[k] + c->n, feed[k].data(), feed[k].size()));
+    KVR_TRY(stage_add(m, tokens[2 + k] + c->n, feed[k].data(), feed[k].size()));
     for (size_t i = 0; i < feed[k].size(); ++i) {
       P.push_back(c->n + (int)i);
       doc.push_back(k);
+      tail_doc.push_back(2 + k);  // every row is past n
     }
   }
   KVR_TRY(stage_add(m, m->pos_d, P.data(), P.size()));
-  KVR_TRY(stage_add(m, m->rowdoc_d, doc.data(), doc.size()));
+  KVR_TRY(stage_add(m, m->rowdoc_d, tail_doc.data(), tail_doc.size()));
   Rows r;
   r.M = (int)P.size();
   r.pos = m->pos_d;
   r.rowdoc = m->rowdoc_d;
-  r.views = (const KVView *)(dev + mb);
-  r.doc_tokens = (const int32_t *const *)(dev + mb + vb);
+  r.views = (const KVView *)(dev + mt.views);
+  r.doc_tokens = (const int32_t *const *)(dev + mt.tokens);
   r.tmaps = (const CUtensorMap *)dev;
+  r.tail_page = tail;
+  r.tail_docs = 2;
   r.max_pos = c->n + (int)std::max(feed[0].size(), feed[1].size()) - 1;
   KVR_TRY(plan_attention(m, r, P.data(), doc.data(), splits));
+  if (!r.tc5 || r.pairs) return fail(KVR_E_CUDA, "a margin's pass without its attention");
   KVR_TRY(run_pass(m, r, false));
   const int first[2] = {mp - 1, (int)feed[0].size() + mp - 1};
   return answers_logprob(m, 2, first, answer, ma, lp);
@@ -2074,11 +2103,13 @@ kvr_status kvr_margin(kvr_model *m, const kvr_cache *c, const int32_t *prompt, i
   KVR_TRY(check_answer(m, c, prompt, mp, a_old, m_old, feed[1]));
   KVR_TRY(use_device(m));
   double lp[2] = {0.0, 0.0};
-  // one pass where its rows fit the pass and the answers' rows the logits
-  const int splits = (int)(feed[0].size() + feed[1].size()) <= m->dims.max_rows &&
-                             m_new + m_old <= KVR_QUERY_RESERVE
-                         ? margin_splits(m, c, feed[0].size(), feed[1].size())
-                         : 0;
+  // one pass where its rows fit the pass, the answers' rows the logits, and there is
+  // room for what it needs beside the cache
+  int splits = (int)(feed[0].size() + feed[1].size()) <= m->dims.max_rows &&
+                       m_new + m_old <= KVR_QUERY_RESERVE
+                   ? margin_splits(m, c, feed[0].size(), feed[1].size())
+                   : 0;
+  if (splits && margin_scratch(m, c)) splits = 0;
   if (splits) {
     const int32_t *answer[2] = {a_new, a_old};
     const int32_t ma[2] = {m_new, m_old};

@@ -79,6 +79,8 @@ struct Attn5Params {
   // (device memory, 64-byte aligned), indexed by the block's document
   const KVView *views;
   const CUtensorMap *tmaps;
+  // pages from tail_page on: entries tail_docs further of both arrays
+  int tail_page, tail_docs;
   int H, G, grp, layer, L;
   int n_splits, n_blocks;
   float *ws_o;    // [n_splits][n_blocks][G][WS_MAXQ][dh]
@@ -163,8 +165,8 @@ __global__ void __launch_bounds__(NT5, 1)
   const uint32_t base = (su32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sKV = base;
   volatile int *abort_v = &abort_f;
-  auto page_row = [&](int c, int kv) {  // first row of (chunk c, kv) in the pool's 2D view
-    const long long pg = table[c];
+  auto page_row = [&](int c, int kv) {  // first row of (chunk c, kv) in its pool's 2D view
+    const long long pg = (c < p.tail_page ? table : p.views[bd.w + p.tail_docs].table)[c];
     return (int)((((pg * p.L + p.layer) * 2 + kv) * p.G + g) * CH);
   };
   const bool rows_cached = nch <= 64;
@@ -196,7 +198,10 @@ __global__ void __launch_bounds__(NT5, 1)
     const int i = t >> 1, kv = t & 1;
     const int row = page_row(c0 + i, kv);
     if (rows_cached) sprow[t] = row;
-    const __nv_bfloat16 *pg = pages + (size_t)row * DH;
+    const __nv_bfloat16 *pg =
+        (c0 + i < p.tail_page ? pages
+                              : (const __nv_bfloat16 *)p.views[bd.w + p.tail_docs].pages) +
+        (size_t)row * DH;
     if (nch <= PREFETCH_MAX_CHUNKS)
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(pg), "r"(TBYTES)
                    : "memory");
@@ -219,10 +224,15 @@ __global__ void __launch_bounds__(NT5, 1)
     // ------------------------------------------------------------ TMA
     if (lane == 0) {
       // a tensor map in global memory is read through the tensor-map proxy
+      auto acquire = [](const CUtensorMap *t) {
+        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(t) : "memory");
+        tma_prefetch_desc(t);
+      };
       if (p.tmaps)
-        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tmap)
-                     : "memory");
-      tma_prefetch_desc(tmap);
+        acquire(tmap);
+      else
+        tma_prefetch_desc(tmap);
+      if (c1 > p.tail_page) acquire(tmap + p.tail_docs);
       pdl_wait();
       ts.waited();
       int issued = 0;
@@ -235,12 +245,13 @@ __global__ void __launch_bounds__(NT5, 1)
         mbar_expect_tx(&kv_full[b], KVBYTES);
         const int rk = rows_cached ? sprow[2 * i] : page_row(c0 + i, 0);
         const int rv = rows_cached ? sprow[2 * i + 1] : page_row(c0 + i, 1);
+        const CUtensorMap *tm = c0 + i < p.tail_page ? tmap : tmap + p.tail_docs;
         if (i == 0) trace_mark(1);
 #pragma unroll
         for (int h = 0; h < HALVES; ++h) {
-          tma_load_2d((void *)__cvta_shared_to_generic(sk + h * CH * 128), tmap, &kv_full[b],
+          tma_load_2d((void *)__cvta_shared_to_generic(sk + h * CH * 128), tm, &kv_full[b],
                       h * 64, rk);
-          tma_load_2d((void *)__cvta_shared_to_generic(sv + h * CH * 128), tmap, &kv_full[b],
+          tma_load_2d((void *)__cvta_shared_to_generic(sv + h * CH * 128), tm, &kv_full[b],
                       h * 64, rv);
         }
         ++issued;
@@ -559,12 +570,15 @@ const char *launch_attention_tc5(const void *q, const int32_t *pos, const int4 *
                                  const void *pages, const int32_t *table, const CUtensorMap &tm_kv,
                                  float *ws_o, float2 *ws_ml, void *out, int *dev_flag,
                                  cudaStream_t s, const KVView *views,
-                                 const CUtensorMap *tmaps) {
+                                 const CUtensorMap *tmaps, int tail_page, int tail_docs) {
   if (n_blocks <= 0) return nullptr;
   if ((views == nullptr) != (tmaps == nullptr)) return "document views without tensor maps";
+  if (!views && tail_page != NO_TAIL) return "a tail without document views";
   Attn5Params p{};
   p.views = views;
   p.tmaps = tmaps;
+  p.tail_page = tail_page;
+  p.tail_docs = tail_docs;
   p.q = (const __nv_bfloat16 *)q;
   p.qk_scale = (float)(1.4426950408889634 / std::sqrt((double)dm.dh));
   p.pos = pos;

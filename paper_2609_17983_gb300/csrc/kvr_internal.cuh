@@ -35,7 +35,7 @@ namespace kvr {
 constexpr int KVR_PAGE = 64;          // positions per KV page
 constexpr int KVR_RD_GROUPS = 8;      // layer groups of kvr_repair_read's overlapped copies
 constexpr int KVR_QUERY_RESERVE = 64; // positions past n reserved for fresh queries
-constexpr int KVR_SPARE_PAGES = 2;    // pages for a second continuation past n (reserve and n's page)
+constexpr int KVR_SPARE_PAGES = 2;    // pages a continuation past n spans at most (reserve and n's page)
 constexpr int GU_BLOCK = 16;          // gate/up interleave block (rows)
 
 struct Dims {
@@ -267,6 +267,10 @@ struct kvr_model {
   size_t sel_scratch_bytes = 0;
   void *batch_scratch = nullptr; // batched repair: documents' TMA views, cache views, tokens
   size_t batch_scratch_bytes = 0;
+  // kvr_margin: KVR_SPARE_PAGES pages for the second answer's rows past n
+  void *spare_pages = nullptr;
+  size_t spare_bytes = 0;
+  CUtensorMap tm_spare;  // their TMA view
   int *dev_flag = nullptr;     // device error flag (bounded waits)
   kvr::TraceBuf trace{};       // attached device timeline buffer, if any
   kvr::SplitView pending{};    // split tiles of h not yet added (next RMSNorm adds them)
@@ -635,15 +639,18 @@ const char *launch_attention_combine(const int4 *blocks, int n_blocks, int max_r
 // attn_tc5_rows_per_block(grp) rows of one document each; partials in the
 // same workspace layout as launch_attention_tc.  One document: pages, table
 // and tm_kv (its TMA view).  Several: views and tmaps, device arrays indexed
-// by a block's document (blocks[].w), tmaps 64-byte aligned.
+// by a block's document (blocks[].w), tmaps 64-byte aligned.  tail_page: logical pages
+// from it on lie in another pool, with view and TMA view tail_docs entries further.
 int attn_tc5_rows_per_block(int grp);
 int attn_tc5_ctas_per_sm(int dh);
+constexpr int NO_TAIL = 0x7fffffff;
 const char *launch_attention_tc5(const void *q, const int32_t *pos, const int4 *blocks,
                                  int n_blocks, int n_splits, const Dims &dm, int layer,
                                  const void *pages, const int32_t *table, const CUtensorMap &tm_kv,
                                  float *ws_o, float2 *ws_ml, void *out, int *dev_flag,
                                  cudaStream_t s, const KVView *views = nullptr,
-                                 const CUtensorMap *tmaps = nullptr);
+                                 const CUtensorMap *tmaps = nullptr, int tail_page = NO_TAIL,
+                                 int tail_docs = 0);
 
 // The same over many rows: the blocks are tiles of at most
 // attn_tc5_rows_per_block(grp) rows, and each CTA takes a pair (device int4:
