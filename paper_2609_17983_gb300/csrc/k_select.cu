@@ -7,6 +7,8 @@
 // positions ascending.
 #include <math.h>
 
+#include <algorithm>
+
 #include "kvr_internal.cuh"
 
 namespace kvr {
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(TOPK_THREADS)
 
 // Attention selector, a group of layers, in two kernels over a workspace.  The
 // stale pool keys are written by no kernel of the pass and the span's queries
-// of every layer are kept, so the scores of many layers run in one launch,
+// of a group's layers are kept, so the scores of many layers run in one launch,
 // where one layer's fill the chip for a few us and wait out their latencies
 // for twenty.  The queries of kv group g are the span rows' heads hh with
 // hh / (H/G) == g; within the group a query is ql = r * (H/G) + (hh mod H/G),
@@ -686,17 +688,19 @@ struct SelLayout {
   int group;                                 // layers scored per launch
 };
 // The logits of a group of layers stay within SEL_GROUP_BYTES (about half of
-// L2, from which the next kernel reads them), at least one layer.
+// L2, from which the next kernel reads them), and so do its queries; at least one
+// layer.
 constexpr size_t SEL_GROUP_BYTES = (size_t)64 << 20;
 SelLayout sel_layout(int S, const Dims &dm, int c) {
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t NQ = (size_t)S * dm.H, nqt = ((size_t)S * (dm.H / dm.G) + SEL_QT - 1) / SEL_QT;
-  const size_t cs = sel_stride(c), fit = SEL_GROUP_BYTES / (NQ * cs * sizeof(float));
+  const size_t cs = sel_stride(c);
+  const size_t fit = SEL_GROUP_BYTES / (NQ * std::max<size_t>(cs, dm.dh) * sizeof(float));
   SelLayout o;
   o.group = fit < 1 ? 1 : fit < (size_t)dm.L ? (int)fit : dm.L;
   while (o.group > 1 && (size_t)o.group * nqt > 65535) --o.group;  // grid z
   o.q = 0;
-  o.tot = o.q + al((size_t)dm.L * NQ * dm.dh * sizeof(float));
+  o.tot = o.q + al((size_t)o.group * NQ * dm.dh * sizeof(float));
   o.logit = o.tot + al((size_t)dm.L * c * sizeof(float));
   o.ml = o.logit + al(o.group * NQ * cs * sizeof(float));
   o.mz = o.ml + al(o.group * NQ * sel_chunks(c) * sizeof(float2));
@@ -712,7 +716,9 @@ size_t attn_select_ws_bytes(int S, const Dims &dm, int n_pool) {
 
 float *attn_select_queries(void *ws_base, int S, const Dims &dm, int n_pool, int layer) {
   const SelLayout o = sel_layout(S, dm, n_pool);
-  return (float *)((char *)ws_base + o.q) + (size_t)layer * S * dm.H * dm.dh;
+  // a group's queries take the last one's place: RoPE, which writes them, runs behind
+  // that group's kernels
+  return (float *)((char *)ws_base + o.q) + (size_t)(layer % o.group) * S * dm.H * dm.dh;
 }
 
 int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_end, int n,

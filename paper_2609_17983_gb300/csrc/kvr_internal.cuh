@@ -675,8 +675,9 @@ struct SimpleKeys {
 };
 // Attention selector over the workspace ws_base (attn_select_ws_bytes(S, dm,
 // n - s_end) bytes).  The pass leaves layer l's span queries (fp32 [S][H*dh])
-// in attn_select_queries(.., l) and calls launch_attn_select_scores after each
-// layer's: a group of layers is scored at its last one, and after the last
+// in attn_select_queries(.., l), where they stay until its group of layers is
+// scored, and calls launch_attn_select_scores after each layer's: a group is
+// scored at its last one, and after the last
 // layer keys[j - s_end] are the top-K keys of the sums over the layers, in
 // layer order, of the pool-softmax probabilities of key j.  Returns the
 // kernels launched.

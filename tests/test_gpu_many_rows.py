@@ -169,10 +169,12 @@ def test_answer_logprob_of_a_nan(vocab, ids):
 
 
 @pytest.mark.parametrize("policy,edit,n", [("attention", 3, 1500), ("attention", 220, 1500),
+                                           ("attention", 700, 1110),
                                            ("cacheblend", 3, 1500), ("cacheblend", 3, 700)])
 def test_model_selectors_over_layer_groups(policy, edit, n):
     # Attention: 220 span rows' logits of 14 layers are more than one launch takes
-    # (groups of 6, 6 and 2 layers), 3 rows' are one launch; CacheBlend:
+    # (groups of 6, 6 and 2 layers), 700 rows' queries (13 and 1), 3 rows' are one
+    # launch; CacheBlend:
     # head-wise projections of many and of fewer rows
     cfg = small_cfg(n_heads=14, n_kv_heads=2, head_dim=128, n_layers=14)
     W = synth.weights(cfg, 0)

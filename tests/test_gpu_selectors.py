@@ -8,6 +8,7 @@ import pytest
 
 import oracle
 from paper_2609_17983_gb300 import synth
+from tests.test_gpu_margin import Allocator
 
 try:
     from paper_2609_17983_gb300 import kvrepair as kv
@@ -68,3 +69,22 @@ def test_simple_policies_match_the_oracle(n):
                 assert got.tolist() == want.tolist(), (policy, every, K)
         cache.close()
     model.close()
+
+
+def test_attention_selector_scratch_of_a_long_span():
+    # 1000 span rows of 24 layers over a pool of 24: the queries kept are one
+    # group's (64 MB, as its logits), not all layers' (197 MB)
+    mem, model = Allocator(), None
+    try:
+        cfg = synth.preset("tiny", dtype="bf16", d_model=512, ffn=512, n_heads=32, n_kv_heads=8,
+                           head_dim=64, n_layers=24)
+        model = kv.Model(cfg, None, seed=0, max_context=1100, max_rows=1024)
+        cache = model.prefill(synth.document(3, 1034, cfg["vocab"]))
+        a0 = mem.asked
+        model.select(cache, "attention", 8, 10, synth.fill_tokens(4, 1000, cfg["vocab"], 13))
+        saved_rows = 1000 * 24 * 2 * 8 * 64 * 2
+        assert mem.asked - a0 < saved_rows + 2 * (64 << 20) + (1 << 20)
+    finally:
+        if model is not None:
+            model.close()
+        kv.use_cuda_allocator()
