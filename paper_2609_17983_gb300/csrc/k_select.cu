@@ -8,6 +8,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "kvr_internal.cuh"
 
@@ -539,36 +540,43 @@ __global__ void __launch_bounds__(SEL_THREADS, sizeof(T) == 2 ? 6 : 4)
 }
 
 // tot[layer][t] = sum over the S*H queries of exp(logit - max) / sum, in a fixed
-// order: a CTA takes ACC_KEYS keys of a layer, four a thread; its ACC_SLICES
+// order: a CTA takes 16 * VEC keys of a layer, VEC a thread; its ACC_SLICES
 // thread slices sum interleaved sets of the queries, then one thread per key
-// adds the slice sums in slice order.
-constexpr int ACC_KEYS = 64, ACC_SLICES = 32;
-__global__ void __launch_bounds__(ACC_KEYS / 4 * ACC_SLICES)
+// adds the slice sums in slice order (the same for every VEC).  Bound by the
+// exponentials' latency, so by the warps on the chip: VEC 4 reads logits and
+// statistics in a quarter of the loads where a group's launch fills the SMs
+// (4 layers, 10,900 keys, 8 rows of 32 heads: a selection 464 us, 475 with VEC 1), but of
+// one layer's 2,000 or 2,500 keys it has 32 or 39 CTAs (4 layers, 200 rows: 1013 and
+// 1100 us, 963 and 1054 with VEC 1).
+constexpr int ACC_LANES = 16, ACC_SLICES = 32;
+template <int VEC>
+__global__ void __launch_bounds__(ACC_LANES * ACC_SLICES)
     k_attn_select_accum(const float *logit, const float2 *mz, int NQ, int c, int cs, float *tot) {
+  using V = std::conditional_t<VEC == 4, float4, std::conditional_t<VEC == 2, float2, float>>;
+  constexpr int KEYS = ACC_LANES * VEC;
   TraceScope ts(TK_SELECT_ACC);
   pdl_trigger();
-  __shared__ float4 part[ACC_SLICES][ACC_KEYS / 4];
-  const int kq = threadIdx.x % (ACC_KEYS / 4), sl = threadIdx.x / (ACC_KEYS / 4);
-  const int t = blockIdx.x * ACC_KEYS + 4 * kq;
+  __shared__ V part[ACC_SLICES][ACC_LANES];
+  const int kq = threadIdx.x % ACC_LANES, sl = threadIdx.x / ACC_LANES;
+  const int t = blockIdx.x * KEYS + VEC * kq;
   logit += (size_t)blockIdx.y * NQ * cs;
   mz += (size_t)blockIdx.y * NQ;
   pdl_wait();  // logits and softmax statistics of the kernel before
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  alignas(16) float s[VEC] = {};
   if (t < c) {  // a row's last quad may end in its padding: sums that nobody takes
 #pragma unroll 8
     for (int qg = sl; qg < NQ; qg += ACC_SLICES) {
       const float2 st = mz[qg];
-      const float4 l = *(const float4 *)(logit + (size_t)qg * cs + t);
-      s.x += expf(l.x - st.x) * st.y;
-      s.y += expf(l.y - st.x) * st.y;
-      s.z += expf(l.z - st.x) * st.y;
-      s.w += expf(l.w - st.x) * st.y;
+      const V lv = *(const V *)(logit + (size_t)qg * cs + t);
+      const float *l = (const float *)&lv;
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) s[e] += expf(l[e] - st.x) * st.y;
     }
   }
-  part[sl][kq] = s;
+  part[sl][kq] = *(const V *)s;
   __syncthreads();
-  const int k = threadIdx.x, tk = blockIdx.x * ACC_KEYS + k;
-  if (k < ACC_KEYS && tk < c) {
+  const int k = threadIdx.x, tk = blockIdx.x * KEYS + k;
+  if (k < KEYS && tk < c) {
     float sum = 0.f;
 #pragma unroll
     for (int i = 0; i < ACC_SLICES; ++i) sum += ((const float *)part[i])[k];
@@ -757,9 +765,15 @@ int launch_attn_select_scores(int S, const Dims &dm, int layer, KVView v, int s_
   launch_pdl(kern, grid, SEL_THREADS, smem, s,
              (const float *)attn_select_queries(ws_base, S, dm, c, layer0), S, dm.H, dm.G,
              layer0, nqt, v, s_end, c, cs, scale, ws);
-  launch_pdl(k_attn_select_accum, dim3((c + ACC_KEYS - 1) / ACC_KEYS, layers),
-             ACC_KEYS / 4 * ACC_SLICES, 0, s, (const float *)ws.logit, (const float2 *)ws.mz,
-             S * dm.H, c, cs, tot + (size_t)layer0 * c);
+  auto accum = [&](auto kernel, int keys) {
+    launch_pdl(kernel, dim3((c + keys - 1) / keys, layers), ACC_LANES * ACC_SLICES, 0, s,
+               (const float *)ws.logit, (const float2 *)ws.mz, S * dm.H, c, cs,
+               tot + (size_t)layer0 * c);
+  };
+  if ((c + 63) / 64 * layers >= num_sms)  // an SM each at least
+    accum(k_attn_select_accum<4>, 64);
+  else
+    accum(k_attn_select_accum<1>, 16);
   if (layer + 1 < dm.L) return 2;
   launch_pdl(k_layer_sum_keys, grid_for(c, 256), 256, 0, s, (const float *)tot, dm.L, c, keys);
   return 3;
