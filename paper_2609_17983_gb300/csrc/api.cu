@@ -137,27 +137,40 @@ kvr_status stage_copy(kvr_model *m, int32_t *dst, const int32_t *src, size_t cou
   return KVR_OK;
 }
 
-// tensor_maps: the data holds CUtensorMaps.
-kvr_status stage_add(kvr_model *m, int32_t *dst, const int32_t *src, size_t count,
-                     bool tensor_maps = false) {
-  if (count == 0) return KVR_OK;
+// The next slot (*h), filled.
+kvr_status stage_slot(kvr_model *m, const int32_t *src, size_t count, int32_t **h) {
   if (count > m->stage_cap) return fail(KVR_E_UNSUPPORTED, "staging overflow (%zu)", count);
-  KVR_TRY(stage_room(m, dst, count));
-  if (m->stage_off + count > m->stage_cap) KVR_TRY(stage_flush(m));
   if (m->stage_off + count > m->stage_cap) {
+    KVR_TRY(stage_flush(m));
     CUDA_TRY(cudaEventSynchronize(m->stage_ev));
     m->stage_off = 0;
   }
-  int32_t *h = m->stage_h + m->stage_off;
-  memcpy(h, src, count * sizeof(int32_t));
-  m->staged.push_back({dst, h, (uint32_t)count, tensor_maps ? 1u : 0u});
+  *h = m->stage_h + m->stage_off;
+  memcpy(*h, src, count * sizeof(int32_t));
   m->stage_off += (count + 31) / 32 * 32;
   return KVR_OK;
 }
 
+// tensor_maps: the data holds CUtensorMaps.
+kvr_status stage_add(kvr_model *m, int32_t *dst, const int32_t *src, size_t count,
+                     bool tensor_maps = false) {
+  if (count == 0) return KVR_OK;
+  int32_t *h;
+  KVR_TRY(stage_room(m, dst, count));
+  KVR_TRY(stage_slot(m, src, count, &h));
+  m->staged.push_back({dst, h, (uint32_t)count, tensor_maps ? 1u : 0u});
+  return KVR_OK;
+}
+
+// One array alone, at once, by a copy engine: it starts sooner than a kernel.
 kvr_status stage_h2d(kvr_model *m, int32_t *dst, const int32_t *src, size_t count) {
-  KVR_TRY(stage_add(m, dst, src, count));
-  return stage_flush(m);
+  if (count == 0) return KVR_OK;
+  int32_t *h;
+  KVR_TRY(stage_flush(m));
+  KVR_TRY(stage_slot(m, src, count, &h));
+  CUDA_TRY(cudaMemcpyAsync(dst, h, count * sizeof(int32_t), cudaMemcpyHostToDevice, m->stream));
+  CUDA_TRY(cudaEventRecord(m->stage_ev, m->stream));
+  return KVR_OK;
 }
 
 // Nothing stays staged when a call returns, whichever way it does.
