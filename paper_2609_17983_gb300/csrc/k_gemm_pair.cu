@@ -418,22 +418,32 @@ size_t configure(PairGemm &p, int M, int N, int K, int clusters, int smem_limit)
 
 }  // namespace
 
-// Where the pairs win (both kernels measured inside a pass, us a launch): with
-// one token tile the few-row kernel splits K over all SMs and leaves the sums to
-// the next kernel, and only gate/up, which sums its own tiles, gains by pairs
-// (192 rows and below equal, 256 rows 63 -> 57).  Above 256 rows its CTAs walk
-// several token tiles (gate/up of 300 rows 107 -> 67), and the sums it leaves
-// cost the next kernel more (with its RoPE, 6144 x 4096: 300 rows 81 -> 73, 600
-// rows 116 -> 87); against that stand the pairs' launch and tail, about 8 us:
-// 4096 x 4096 with its RMSNorm, 300 rows 46 against 52, 600 rows 57 against 59.
-bool gemm_pair_takes(int M, int N, int K, int epi) {
+// Where the pairs win (both kernels measured inside a pass, us a launch).  Above 256
+// rows the few-row kernel's CTAs walk several token tiles (gate/up of 300 rows 107
+// -> 67), and the sums it leaves cost the next kernel more (with its RoPE,
+// 6144 x 4096: 300 rows 81 -> 73, 600 rows 116 -> 87); against that stand the pairs'
+// launch and tail, about 8 us, so small products stay: 4096 x 4096 with its
+// RMSNorm, 300 rows 46 against 52, 600 rows 57 against 59.
+// With one token tile the few-row kernel splits K over all SMs and leaves the sums
+// to the next kernel; only gate/up, which sums its own tiles, gains by pairs, where
+// their rounds are full and no tile is in more than two parts (193 to 256 rows, a
+// layer's GEMMs, RoPE and norms before over after: 4096 x 28672, 112 tiles for 76
+// clusters, 1.01 to 1.03; 3584 x 37888, 148 tiles, 1.00 to 1.03; 8192 x 57344 1.00
+// to 1.04; but 4096 x 22016, 10 of its 86 tiles in seven parts, 0.94 to 0.96, 4096 x
+// 32768, 128 tiles, 0.98 to 1.01) and the product is large (2304 x 18432, 72 tiles,
+// 0.97, 2560 x 19456, 76 tiles, 0.95).  192 rows and below: equal at best.
+bool gemm_pair_takes(int M, int N, int K, int epi, int num_sms) {
   static const bool off = [] {
     const char *e = getenv("KVR_DISABLE_PAIR_GEMM");
     return e && e[0] == '1';
   }();
-  const double flops = 2.0 * M * N * K;
-  if (off) return false;
-  return M > 256 ? flops >= 12e9 : M > 192 && epi == GEMM_EPI_SWIGLU && flops >= 32.5e9;
+  if (off || 2.0 * M * N * K < 12e9) return false;
+  if (M > 256) return true;
+  if (M <= 192 || epi != GEMM_EPI_SWIGLU || 2.0 * M * N * K < 40e9) return false;
+  const int clusters = num_sms / 2, tiles = (N + TM - 1) / TM, left = tiles % clusters;
+  const int parts = left ? clusters / left : 1;
+  const double rounds = tiles / clusters + (left ? 1.0 / parts : 0.0);
+  return parts <= 2 && tiles >= 0.9 * rounds * clusters;
 }
 
 const char *launch_gemm_pair(const GemmArgs &g, const CUtensorMap &tmW, int epi, void *out2,

@@ -1078,7 +1078,8 @@ const char *launch_gemm_tc(const GemmArgs &g, const CUtensorMap &tmW, int epi, v
                            int ld2, const TcWorkspace &ws, cudaStream_t s, SplitView *defer) {
   if (defer) *defer = SplitView{};
   if (g.M <= 0) return nullptr;
-  if (gemm_pair_takes(g.M, g.N, g.K, epi)) return launch_gemm_pair(g, tmW, epi, out2, ld2, ws, s);
+  if (gemm_pair_takes(g.M, g.N, g.K, epi, ws.num_sms))
+    return launch_gemm_pair(g, tmW, epi, out2, ld2, ws, s);
   bool dfr = defer != nullptr && epi != GEMM_EPI_SWIGLU;
   TcParams p{};
   size_t smem = 0;

@@ -602,7 +602,7 @@ const char *launch_gemm_chain(const ChainStep *steps, int n, const TcWorkspace &
                               cudaStream_t s, SplitView *last_defer);
 // Many rows (k_gemm_pair.cu): pairs of CTAs on 256-feature tiles; Y is always
 // complete.  launch_gemm_tc hands them over.
-bool gemm_pair_takes(int M, int N, int K, int epi);
+bool gemm_pair_takes(int M, int N, int K, int epi, int num_sms);
 const char *launch_gemm_pair(const GemmArgs &g, const CUtensorMap &tmW, int epi, void *out2,
                              int ld2, const TcWorkspace &ws, cudaStream_t s);
 const char *launch_gemm_tc(const GemmArgs &g, const CUtensorMap &tmW, int epi, void *out2,

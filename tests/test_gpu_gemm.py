@@ -63,12 +63,12 @@ def test_lm_head_matches_fp64_matmul(model):
     assert rel(got, f64(x) @ f64(lm).T) <= 1e-3
 
 
-@pytest.mark.parametrize("M", [512, 904, 4096])
+@pytest.mark.parametrize("M", [224, 300, 512, 904, 4096])
 def test_many_row_projections_match_fp64_matmul(M):
-    # a prefill chunk's row counts: pairs of CTAs on whole and split tiles, token
-    # tiles of up to 256 rows with a ragged last one (and stream-K over several
-    # token tiles where the work is small); the fp64 reference on a sample of
-    # rows from every token tile
+    # pairs of CTAs on whole and split tiles, token tiles of up to 256 rows with a
+    # ragged last one: all projections of a prefill chunk's row counts, gate/up of
+    # 224 rows; stream-K over one token tile (the others of 224 rows) and over two
+    # (O of 300 rows); the fp64 reference on a sample of rows from every token tile
     cfg = synth.preset("llama8b", n_layers=1)
     m = kv.Model(cfg, None, seed=0, max_context=512, max_rows=4096)
     d, F = cfg["d_model"], cfg["ffn"]

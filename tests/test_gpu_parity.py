@@ -553,9 +553,8 @@ def test_8b_shape_two_layer_parity(shape, chain, monkeypatch):
 
 
 def test_8b_shape_prefill_many_rows_parity():
-    # a prefill chunk of 600 rows: the gate/up and down GEMMs on pairs of CTAs,
-    # stream-K over several ragged token tiles for the others; every row's K/V
-    # at both layers against the oracle's prefill
+    # a prefill chunk of 600 rows: every projection on pairs of CTAs, over ragged
+    # token tiles; every row's K/V at both layers against the oracle's prefill
     cfg = synth.preset("llama8b", n_layers=2)
     n = 600
     doc = synth.document(4, n, cfg["vocab"])
