@@ -647,52 +647,60 @@ kvr_status run_pass(kvr_model *m, const Rows &r, bool kv_only) {
 // The repair pass through a CUDA graph: the launch sequence of a pass
 // depends only on the cache, the row count and the attention block/split
 // plan (positions, tokens and block contents are read from device memory),
-// so it is captured once per such key and replayed -- from the key's second
-// pass on: a replay saves 2.5% of a pass (3.24 -> 3.16 ms, 40 rows of 32 layers),
-// capturing and instantiating it cost 0.7 ms, which a document repaired once
-// never gets back (its pass: 3.88 -> 3.26 ms).  Only on a stream that can be
-// captured (not the legacy default stream) and with profiling off.
-kvr_status run_pass_graph(kvr_model *m, kvr_cache *c, const Rows &r) {
+// so it is captured once per such key and replayed from then on.  Capturing and
+// instantiating it takes the host 0.7 ms (40 rows of 32 layers; a replay saves
+// 2.5% of the 3.1 ms pass), which a document repaired once never gets back: the
+// first pass of a key only launches (3.74 -> 3.13 ms), and the second is captured
+// behind its own launches, while the device works (capture_pass).  Only on a
+// stream that can be captured (not the legacy default stream) and with profiling
+// off.  *capture: the caller is to call capture_pass once it has queued what
+// follows the pass, before it waits.
+kvr_status run_pass_graph(kvr_model *m, kvr_cache *c, const Rows &r, kvr_cache::Graph **capture) {
+  *capture = nullptr;
   if (!m->use_graphs || m->prof || m->stream == nullptr) return run_pass(m, r, true);
   KVR_TRY(stage_flush(m));  // not part of the graph
   auto g = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const auto &x) {
     return x.M == r.M && x.nb == r.n_blocks && x.np == r.n_pairs && x.ns == r.n_splits &&
            x.rows_out == r.rows_out;
   });
-  if (g == c->graphs.end()) {
-    // within a caller's own capture a pass is refused, as the capture below would be
-    cudaStreamCaptureStatus cs;
-    const cudaError_t e = cudaStreamIsCapturing(m->stream, &cs);
-    if (e != cudaSuccess || cs != cudaStreamCaptureStatusNone)
-      return fail(KVR_E_CUDA, "begin capture: %s",
-                  e != cudaSuccess ? cudaGetErrorString(e) : "the stream is being captured");
+  if (g != c->graphs.end() && g->exec) {
+    const cudaError_t e = cudaGraphLaunch(g->exec, m->stream);
+    if (e != cudaSuccess) return fail(KVR_E_CUDA, "graph launch: %s", cudaGetErrorString(e));
+    m->launches += g->kernels;
+    return KVR_OK;
+  }
+  // within a caller's own capture a pass is refused, as a capture of its own would be
+  cudaStreamCaptureStatus cs;
+  const cudaError_t e = cudaStreamIsCapturing(m->stream, &cs);
+  if (e != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+    return fail(KVR_E_CUDA, "begin capture: %s",
+                e != cudaSuccess ? cudaGetErrorString(e) : "the stream is being captured");
+  if (g == c->graphs.end())
     c->graphs.push_back({r.M, r.n_blocks, r.n_pairs, r.n_splits, r.rows_out, 0, nullptr});
-    return run_pass(m, r, true);
+  else if (!g->failed)
+    *capture = &*g;
+  return run_pass(m, r, true);
+}
+
+// Captures the pass that was just launched, for the next of its key.  Without its
+// graph a key's passes go on being launched.
+void capture_pass(kvr_model *m, const Rows &r, kvr_cache::Graph *g) {
+  const int64_t l0 = m->launches;
+  cudaGraph_t graph = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(m->stream, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    const kvr_status st = run_pass(m, r, true);
+    e = cudaStreamEndCapture(m->stream, &graph);
+    if (e == cudaSuccess && !st) e = cudaGraphInstantiate(&g->exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    if (e != cudaSuccess || st) g->exec = nullptr;
   }
   if (!g->exec) {
-    int64_t l0 = m->launches;
-    cudaError_t e = cudaStreamBeginCapture(m->stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return fail(KVR_E_CUDA, "begin capture: %s", cudaGetErrorString(e));
-    kvr_status st = run_pass(m, r, true);
-    cudaGraph_t graph = nullptr;
-    e = cudaStreamEndCapture(m->stream, &graph);
-    if (st || e != cudaSuccess) {
-      if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
-      return st ? st : fail(KVR_E_CUDA, "end capture: %s", cudaGetErrorString(e));
-    }
-    cudaGraphExec_t exec = nullptr;
-    e = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) return fail(KVR_E_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-    g->exec = exec;
-    g->kernels = m->launches - l0;
-    m->launches = l0;
+    g->failed = true;
+    cudaGetLastError();
   }
-  const cudaError_t e = cudaGraphLaunch(g->exec, m->stream);
-  if (e != cudaSuccess) return fail(KVR_E_CUDA, "graph launch: %s", cudaGetErrorString(e));
-  m->launches += g->kernels;
-  return KVR_OK;
+  g->kernels = m->launches - l0;
+  m->launches = l0;
 }
 
 // flag_queued: the stream's work already writes the device flag to m->flag_h.
@@ -1494,14 +1502,16 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
       r.rows_out = m->rows_scratch;
       r.rd_every = (dm.L + KVR_RD_GROUPS - 1) / KVR_RD_GROUPS;
     }
+    kvr_cache::Graph *capture = nullptr;
     if (!st) {
       launched = true;
-      st = run_pass_graph(m, c, r);
+      st = run_pass_graph(m, c, r, &capture);
     }
     if (!st && direct) {
-      launch_cache_read_host(r.single, dm.dtype, P.data(), nullptr, M, 0, dm.L, dm.G, dm.dh, k_out, v_out,
-                             m->dev_flag, m->flag_h, m->stream);
+      launch_cache_read_host(r.single, dm.dtype, P.data(), nullptr, M, 0, dm.L, dm.G, dm.dh, k_out,
+                             v_out, m->dev_flag, m->flag_h, m->stream);
       st = launch_check(m, 1);
+      if (!st && capture) capture_pass(m, r, capture);
       if (!st)
         st = sync_model(m, true);
       else
@@ -1519,10 +1529,13 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
                               cudaMemcpyDeviceToHost, m->rd_stream) != cudaSuccess)
           st = fail(KVR_E_CUDA, "row readback");
       }
+      if (!st && capture) capture_pass(m, r, capture);
       const kvr_status s2 = sync_model(m);
       if (!st) st = s2;
       if (cudaStreamSynchronize(m->rd_stream) != cudaSuccess && !st)
         st = fail(KVR_E_CUDA, "row readback");
+    } else if (!st && capture) {
+      capture_pass(m, r, capture);
     }
   }
   if (st && st != KVR_E_CUDA && !launched && edit_len) {

@@ -311,6 +311,7 @@ struct kvr_cache {
     const void *rows_out;  // kvr_repair_read's row buffer, or null
     int64_t kernels;
     cudaGraphExec_t exec;
+    bool failed = false;  // could not be captured
   };
   std::vector<Graph> graphs;  // repair passes of this cache: run once (exec null), then captured
   kvr::KVView view() const {

@@ -62,6 +62,31 @@ def test_single_repairs_reach_the_device_in_order():
     model.close()
 
 
+@pytest.mark.parametrize("read", [False, True])
+def test_every_pass_of_a_document_runs_once(read):
+    # the second pass of a row count is captured behind its own launches: it runs
+    # once (its edit lands, its launches count once), as the first and the replays
+    import torch
+    cfg = synth.preset("tiny", n_layers=9)
+    model = kv.Model(cfg, None, seed=0, max_context=2048, max_rows=256)
+    stream = torch.cuda.Stream()
+    model.set_stream(stream.cuda_stream)
+    doc = synth.document(9, 300, cfg["vocab"])
+    cache = model.prefill(doc)
+    used = []
+    for i in range(5):
+        new, A = np.arange(4, dtype=np.int32) + 11 * i, np.arange(104, 130 - i % 2)
+        l0 = model.launches()
+        rows = cache.repair_read(new, 100, A) if read else cache.repair(new, 100, A)
+        used.append(model.launches() - l0)
+        doc[100:104] = new
+        check_layer0(model, [cache], [doc], cfg["d_model"])
+        if read:
+            assert np.array_equal(rows[0], cache.read_raw(np.arange(100, 130 - i % 2))[0])
+    assert len(set(used)) == 1
+    model.close()
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 def test_rows_read_into_page_locked_memory(dtype):
     # the positions that a launch's arguments hold (512), one fewer and more, in
