@@ -245,6 +245,13 @@ bool use_tc_attention(const kvr_model *m) {
 // first), each range in `splits` parts.  One wave ends with its longest CTA;
 // more are dealt to the SMs as these fall free, longest first, so they end
 // about half a CTA after the mean.  A split pass also runs the combine.
+// Fitted to launches of 36 to 4096 rows over 500 to 12345 keys (4 and 7 query
+// heads a KV head) and good for the choice, not for the time: a few rows take
+// up to 30% longer than modelled, thousands up to 30% less.  Of 46 such plans it
+// takes the slower kernel in four, where equal CTAs fill little more than one
+// wave or two (600 scattered rows: pairs 84 us against 78; 1000: 119 against 116;
+// a 904-row prefill 28 against 26; 64 rows 24.0 against 23.4); in the others the
+// pairs take up to half of the time (2000 rows 119 against 233).
 struct AttnCost {
   int per_page, fixed;
 };
@@ -489,7 +496,7 @@ kvr_status attention(kvr_model *m, const Rows &r, int l) {
       KVR_TRY(launch_check(m, r.n_splits > 1 ? 2 : 1));
     } else {
       launch_attention_simt(r.q ? r.q : m->q, r.pos, r.M, dm, l, r.views, r.rowdoc, r.single,
-                            (float *)m->attn, m->stream);
+                            (float *)m->attn, m->num_sms, m->stream);
       KVR_TRY(launch_check(m, 1));
     }
   }
@@ -1348,7 +1355,8 @@ static kvr_status new_cache(kvr_model *m, const int32_t *tokens, int32_t n, kvr_
   }
   if (dm.dtype == KVR_DTYPE_BF16) {
     const long long rows = (long long)c->n_pages * dm.L * 2 * dm.G * KVR_PAGE;
-    c->tm_kv_ok = rows < (1ll << 31) && make_tmap_bf16(&c->tm_kv, c->pages, (int)rows, dm.dh, KVR_PAGE);
+    c->tm_kv_ok =
+        rows < (1ll << 31) && make_tmap_bf16(&c->tm_kv, c->pages, (int)rows, dm.dh, KVR_PAGE);
   }
   std::vector<int32_t> tab(c->n_pages);
   for (int i = 0; i < c->n_pages; ++i) tab[i] = i;
@@ -1491,12 +1499,14 @@ kvr_status repair_impl(kvr_cache *c, const int32_t *new_tokens, int32_t edit_sta
     st = plan_attention(m, r, P.data(), nullptr);
     const size_t row_b = (size_t)dm.L * dm.G * dm.dh * dm.es();  // one row, all layers
     // Few rows of few layers are read from the cache when the pass is over: below
-    // this the copies behind the layer groups cost more than they overlap (36
-    // fp32 rows of two layers 89 -> 84 us, 134 rows of four 8B-shape layers 454 ->
-    // 449; 40 rows of 32 layers, 2.6 MB, 3140 against 3153).
+    // this the copies behind the layer groups cost more than they overlap.  By the
+    // bytes of K, copies against stores: 36 fp32 rows of two layers (36 KB) 70.4 ->
+    // 60.0 us, 134 rows of four Qwen-shape layers (0.5 MiB) 433.6 -> 430.1, 100 rows
+    // of four 8B-shape layers (0.8 MiB) 402.7 -> 402.0; at 1.0 and 1.25 MiB equal; 250
+    // rows (2 MiB) 530 against 539, 40 rows of 32 layers (2.5 MiB) 3140 against 3156.
     constexpr size_t DIRECT_BYTES = (size_t)1 << 20;
-    const bool direct =
-        k_out && M * row_b <= DIRECT_BYTES && host_read_direct(M, HOST_READ_MAX_POS, M * row_b, k_out, v_out);
+    const bool direct = k_out && M * row_b <= DIRECT_BYTES &&
+                        host_read_direct(M, HOST_READ_MAX_POS, M * row_b, k_out, v_out);
     if (!st && k_out && !direct) {
       st = grow_scratch(m, m->rows_scratch, m->rows_scratch_bytes, 2 * M * row_b, "row buffer");
       r.rows_out = m->rows_scratch;

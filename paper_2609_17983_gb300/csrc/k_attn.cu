@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(32 * AW, NQ * VPL <= 8 ? 3 : 2) k_attn_simt(co
   }
   for (int b = warp; b <= kmax / 32; b += AW) {
     // a block lies in one page (its slots past the last key hold finite values)
-    const float *kp = c + v.offset(p.layer, 0, g, 32 * b), *vp = c + v.offset(p.layer, 1, g, 32 * b);
+    const float *kp = c + v.offset(p.layer, 0, g, 32 * b);
+    const float *vp = c + v.offset(p.layer, 1, g, 32 * b);
     // four lanes a key, each with every fourth float4 of it; of eight keys at a
     // time, a lane keeps the sum of the one in the pass of its own number
     const int part = lane & 3, kr = lane >> 2, key = 32 * b + 8 * part + kr;
@@ -175,11 +176,11 @@ __global__ void __launch_bounds__(32 * AW, NQ * VPL <= 8 ? 3 : 2) k_attn_simt(co
 }
 
 template <int VPL>
-void run(SimtAttn p, cudaStream_t s) {
+void run(SimtAttn p, int num_sms, cudaStream_t s) {
   const int grp = p.H / p.G;
   // queries per CTA: as many as share the reads of a key while the CTAs still
   // fill the SMs (about twice over)
-  constexpr int FILL = 304;
+  const int fill = 2 * num_sms;
   auto go = [&](auto nq) {
     constexpr int NQ = decltype(nq)::value;
     p.gp = p.views ? (grp + NQ - 1) / NQ * NQ : grp;
@@ -188,9 +189,9 @@ void run(SimtAttn p, cudaStream_t s) {
                p);
   };
   const long long q = (long long)p.M * p.H;
-  if (q >= 8 * FILL && !(p.views && grp < 8))
+  if (q >= 8 * fill && !(p.views && grp < 8))
     go(std::integral_constant<int, 8>{});
-  else if (q >= 4 * FILL && !(p.views && grp < 4))
+  else if (q >= 4 * fill && !(p.views && grp < 4))
     go(std::integral_constant<int, 4>{});
   else
     go(std::integral_constant<int, 1>{});
@@ -200,14 +201,14 @@ void run(SimtAttn p, cudaStream_t s) {
 
 void launch_attention_simt(const float *q, const int32_t *pos, int M, const Dims &dm, int layer,
                            const KVView *views, const int32_t *rowdoc, KVView single, float *out,
-                           cudaStream_t s) {
+                           int num_sms, cudaStream_t s) {
   if (M <= 0) return;
   SimtAttn p{q,     pos,    M,      dm.H, dm.G, dm.H / dm.G,
              layer, views,  rowdoc, single, out, (float)(1.0 / sqrt((double)dm.dh))};
   if (dm.dh == 64)
-    run<2>(p, s);
+    run<2>(p, num_sms, s);
   else
-    run<4>(p, s);
+    run<4>(p, num_sms, s);
 }
 
 }  // namespace kvr

@@ -27,7 +27,7 @@
 // 64-key chunk took 1.08 us, against 0.28 us of MMA, and nothing filled the
 // gaps.  Two tiles fill each other's, and a step of 128 keys halves the
 // hand-offs: 4096 rows over their own keys, 32 heads of 128, went from 236 to
-// 125 us (0.58 to 1.10 PFLOP/s), tensor pipe 20 to 40% active.  A step takes
+// 125 us (0.58 to 1.10 PFLOP/s), tensor pipe 20 to 51% active.  A step takes
 // about 2.0 us: its softmax 0.7 (MUFU 0.27 of it), the hand-offs and the issue
 // of 32 MMAs the rest.  Also measured, for the same rows: one thread per query
 // vector 155 us, a half row of scores held in registers throughout (92 bytes
@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(NT, 1)
       q_full, drain_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_f;
-  __shared__ float sx[2][QV];  // per tile: a row's maximum (a growing step), then its sum, handed over
+  // per tile: a row's maximum (a growing step), then its sum, handed over
+  __shared__ float sx[2][QV];
 
   TraceScope ts(TK_ATTN);
   const int split = blockIdx.x, g = blockIdx.y;
@@ -454,7 +455,9 @@ __global__ void __launch_bounds__(NT, 1)
       tc_fence_after();
       constexpr int RC = OC / 8;  // 16-byte pieces staged per row and warp
       uint8_t *st = (uint8_t *)__cvta_shared_to_generic(sQ + t * QBYTES) + part * OC * 2;
-      auto piece = [&](int r, int c) { return (uint4 *)(st + r * (DH * 2) + ((c ^ (r & (RC - 1))) << 4)); };
+      auto piece = [&](int r, int c) {
+        return (uint4 *)(st + r * (DH * 2) + ((c ^ (r & (RC - 1))) << 4));
+      };
       const size_t bs = ((size_t)split * p.n_blocks + blk) * p.G + g;
       if (p.n_splits == 1) {
         const float inv = lt > 0.f ? 1.f / lt : 0.f;

@@ -111,8 +111,9 @@ __global__ void __launch_bounds__(NTH) k_gemm_simt(const SimtGemm p) {
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          acc[i][j] = fmaf(a[i].x, b[j].x, fmaf(a[i].y, b[j].y,
-                                                fmaf(a[i].z, b[j].z, fmaf(a[i].w, b[j].w, acc[i][j]))));
+          acc[i][j] = fmaf(
+              a[i].x, b[j].x,
+              fmaf(a[i].y, b[j].y, fmaf(a[i].z, b[j].z, fmaf(a[i].w, b[j].w, acc[i][j]))));
     }
     if (c + 1 < chunks) {
       stage((c + 1) & 1);
@@ -128,7 +129,8 @@ __global__ void __launch_bounds__(NTH) k_gemm_simt(const SimtGemm p) {
   };
   auto out_act = [&](int m, int n, float gate, float up) {  // n: the gate row
     if (m >= p.M || n >= p.N) return;
-    put((T *)p.act + (size_t)m * (p.N / 2) + n / 32 * 16 + n % 16, gate / (1.0f + expf(-gate)) * up);
+    put((T *)p.act + (size_t)m * (p.N / 2) + n / 32 * 16 + n % 16,
+        gate / (1.0f + expf(-gate)) * up);
   };
   if constexpr (KS == 1) {
 #pragma unroll

@@ -496,8 +496,9 @@ struct HostReadPos {
   int32_t p[HOST_READ_MAX_POS];
 };
 __global__ void k_cache_read_host(KVView v, const __grid_constant__ HostReadPos pos,
-                                  const int32_t *many, int n_pos, int l0, int nl, int G, int vr, int es, uint4 *k_out,
-                                  uint4 *v_out, const int *flag_in, int *flag_out) {
+                                  const int32_t *many, int n_pos, int l0, int nl, int G, int vr,
+                                  int es, uint4 *k_out, uint4 *v_out, const int *flag_in,
+                                  int *flag_out) {
   pdl_trigger();
   pdl_wait();
   const unsigned total = (unsigned)n_pos * nl * G * vr;
@@ -839,13 +840,14 @@ void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, int n_pos,
 }
 
 void launch_cache_read_host(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d,
-                            int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out, const int *flag_in,
-                            int *flag_out, cudaStream_t s) {
+                            int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out,
+                            const int *flag_in, int *flag_out, cudaStream_t s) {
   const int es = dtype == KVR_DTYPE_BF16 ? 2 : 4, vr = dh * es / 16;
   HostReadPos p;
   if (!pos_d) std::copy(pos, pos + n_pos, p.p);
   launch_pdl(k_cache_read_host, grid_for((size_t)n_pos * (l1 - l0) * G * vr, 256), 256, 0, s, v, p,
-             pos_d, n_pos, l0, l1 - l0, G, vr, es, (uint4 *)k_out, (uint4 *)v_out, flag_in, flag_out);
+             pos_d, n_pos, l0, l1 - l0, G, vr, es, (uint4 *)k_out, (uint4 *)v_out, flag_in,
+             flag_out);
 }
 
 void launch_cache_scatter_raw(KVView v, int dtype, int p0, int n_pos, const void *k_in,

@@ -241,9 +241,9 @@ __global__ void __launch_bounds__(TOPK_THREADS)
 // chunk's keys are read once into shared memory and serve every query of the
 // tile (so a group's key rows leave L2 once per query tile, not once per query).
 // It stores the scaled logits, logit[qg * stride + (j - s_end)], and per query
-// the chunk's max and sum of exp(logit - max); the last CTA of (group, query tile) to finish folds the
-// chunk statistics into the pool softmax's max and 1 / sum.  Arrival is an
-// atomic count with no waiting: every other CTA just exits.  The contraction
+// the chunk's max and sum of exp(logit - max); the last CTA of (group, query tile)
+// to finish folds the chunk statistics into the pool softmax's max and 1 / sum.
+// Arrival is an atomic count with no waiting: every other CTA just exits.  The contraction
 // runs on mma.sync for bf16 caches and on FFMA micro-tiles for fp32 caches.
 // Eight layers of 8 span rows and 2,492 keys: 69 us for both kernels with a CTA
 // per chunk, run-time head sizes and scalar fragment loads, 45 now; mma.sync
@@ -298,7 +298,8 @@ __device__ __forceinline__ void sel_ldmatrix(uint32_t *r, const __nv_bfloat16 *r
 
 template <typename T, int DH>
 __global__ void __launch_bounds__(SEL_THREADS, sizeof(T) == 2 ? 6 : 4)
-    k_attn_select_logits(const float *q, int S, int H, int G, int layer0, int n_qt, KVView v, int s_end, int c, int cs, float scale, SelWs ws) {
+    k_attn_select_logits(const float *q, int S, int H, int G, int layer0, int n_qt, KVView v,
+                         int s_end, int c, int cs, float scale, SelWs ws) {
   constexpr bool BF16 = sizeof(T) == 2;
   TraceScope ts(TK_SELECT);
   pdl_trigger();

@@ -35,7 +35,7 @@ namespace kvr {
 constexpr int KVR_PAGE = 64;          // positions per KV page
 constexpr int KVR_RD_GROUPS = 8;      // layer groups of kvr_repair_read's overlapped copies
 constexpr int KVR_QUERY_RESERVE = 64; // positions past n reserved for fresh queries
-constexpr int KVR_SPARE_PAGES = 2;    // pages a continuation past n spans at most (reserve and n's page)
+constexpr int KVR_SPARE_PAGES = 2;    // pages that a continuation past n spans at most
 constexpr int GU_BLOCK = 16;          // gate/up interleave block (rows)
 
 struct Dims {
@@ -524,8 +524,8 @@ void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, int n_pos,
 // null, from the device, and the device error flag to *flag_out.
 constexpr int HOST_READ_MAX_POS = 512;
 void launch_cache_read_host(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d,
-                            int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out, const int *flag_in,
-                            int *flag_out, cudaStream_t s);
+                            int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out,
+                            const int *flag_in, int *flag_out, cudaStream_t s);
 // Rows [n_pos][L][G][dh] (cache dtype) of consecutive positions p0.. into the pages.
 void launch_cache_scatter_raw(KVView v, int dtype, int p0, int n_pos, const void *k_in,
                               const void *v_in, cudaStream_t s);
@@ -615,7 +615,7 @@ const char *launch_gemm_tc(const GemmArgs &g, const CUtensorMap &tmW, int epi, v
 // GQA head h -> kv head h / (H/G).  fp32 model; q, out [M][H*dh].
 void launch_attention_simt(const float *q, const int32_t *pos, int M, const Dims &dm, int layer,
                            const KVView *views, const int32_t *rowdoc, KVView single, float *out,
-                           cudaStream_t s);
+                           int num_sms, cudaStream_t s);
 
 // Tensor-core attention (bf16 cache, head_dim 64 or 128).  blocks: device
 // int4 (row0, nrows, kmax, doc) per query block (rows of one document, at

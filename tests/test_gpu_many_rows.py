@@ -164,7 +164,8 @@ def test_answer_logprob_of_a_nan(vocab, ids):
     W["lm_head"][ids] = np.nan
     model = kv.Model(cfg, W, max_context=256, max_rows=256)
     cache = model.prefill(np.arange(2, 82, dtype=np.int32) % vocab)
-    assert np.isnan(model.answer_logprob(cache, np.array([3, 4], np.int32), np.array([5], np.int32)))
+    prompt, answer = np.array([3, 4], np.int32), np.array([5], np.int32)
+    assert np.isnan(model.answer_logprob(cache, prompt, answer))
     model.close()
 
 
@@ -199,8 +200,9 @@ def test_model_selectors_over_layer_groups(policy, edit, n):
 
 @pytest.mark.parametrize("rows", [1, 512, 513])
 def test_read_into_page_locked_memory(rows):
-    # by the kernel's stores (up to 512 positions, 16-byte aligned), and by copies
-    # (more, or off the alignment): the same rows as into pageable memory
+    # by the kernel's stores (16-byte aligned; up to 512 positions come with the
+    # launch, more from device memory), and by copies (off the alignment): the same
+    # rows as into pageable memory
     import torch
     cfg = small_cfg(n_heads=8, n_kv_heads=2, head_dim=64)
     model = kv.Model(cfg, None, seed=0, max_context=1024, max_rows=1024)
