@@ -449,9 +449,15 @@ __global__ void __launch_bounds__(ROPE_THREADS, HPT > 1 ? 4 : 1) k_rope_rows(con
   }
 }
 
+// Positions of a readback: a few come with the launch (many: in device memory).
+struct HostReadPos {
+  int32_t p[HOST_READ_MAX_POS];
+};
+
 template <typename T>
-__global__ void k_cache_gather(KVView v, const int32_t *pos, int n_pos, int l0, int nl, int G,
-                               int dh, float *k_out, float *v_out) {
+__global__ void k_cache_gather(KVView v, const __grid_constant__ HostReadPos pos,
+                               const int32_t *many, int n_pos, int l0, int nl, int G, int dh,
+                               float *k_out, float *v_out) {
   size_t total = (size_t)n_pos * nl * G * dh;
   const T *c = (const T *)v.pages;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
@@ -460,18 +466,18 @@ __global__ void k_cache_gather(KVView v, const int32_t *pos, int n_pos, int l0, 
     size_t r = e / dh;
     int g = (int)(r % G);
     r /= G;
-    int l = (int)(r % nl);
-    int p = (int)(r / nl);
-    k_out[e] = ld(c, v.offset(l0 + l, 0, g, pos[p]) + i);
-    v_out[e] = ld(c, v.offset(l0 + l, 1, g, pos[p]) + i);
+    const int l = (int)(r % nl), p = many ? many[r / nl] : pos.p[r / nl];
+    k_out[e] = ld(c, v.offset(l0 + l, 0, g, p) + i);
+    v_out[e] = ld(c, v.offset(l0 + l, 1, g, p) + i);
   }
 }
 
 // K/V of the given positions, layers l0 .. l0+nl-1, as stored: 16-byte
 // pieces of the cache rows (a row is head_dim elements, a multiple of 16
 // bytes), vr pieces a row, output [n_pos][nl][G][row].
-__global__ void k_cache_gather_raw(KVView v, const int32_t *pos, int n_pos, int l0, int nl, int G,
-                                   int vr, int es, uint4 *k_out, uint4 *v_out) {
+__global__ void k_cache_gather_raw(KVView v, const __grid_constant__ HostReadPos pos,
+                                   const int32_t *many, int n_pos, int l0, int nl, int G, int vr,
+                                   int es, uint4 *k_out, uint4 *v_out) {
   const unsigned total = (unsigned)n_pos * nl * G * vr;
   const uint4 *c = (const uint4 *)v.pages;
   for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -480,21 +486,16 @@ __global__ void k_cache_gather_raw(KVView v, const int32_t *pos, int n_pos, int 
     unsigned r = e / vr;
     const int g = (int)(r % G);
     r /= G;
-    const int l = (int)(r % nl);
-    const int p = pos[r / nl];
+    const int l = (int)(r % nl), p = many ? many[r / nl] : pos.p[r / nl];
     k_out[e] = c[v.offset(l0 + l, 0, g, p) * es / 16 + i];
     v_out[e] = c[v.offset(l0 + l, 1, g, p) * es / 16 + i];
   }
 }
 
 // k_cache_gather_raw into page-locked host memory: the rows leave by the stores
-// themselves, without a gathered copy or a copy's set-up; a few positions come
-// with the launch (many: in device memory), and the device error flag goes with
-// the rows (everything queued before has run).  Bound by the link to the host:
-// 82 MB at 183 GB/s.
-struct HostReadPos {
-  int32_t p[HOST_READ_MAX_POS];
-};
+// themselves, without a gathered copy or a copy's set-up, and the device error flag
+// goes with the rows (everything queued before has run).  Bound by the link to the
+// host: 82 MB at 183 GB/s.
 __global__ void k_cache_read_host(KVView v, const __grid_constant__ HostReadPos pos,
                                   const int32_t *many, int n_pos, int l0, int nl, int G, int vr,
                                   int es, uint4 *k_out, uint4 *v_out, const int *flag_in,
@@ -812,20 +813,31 @@ void launch_rope_scatter(const float *qkv, const float2 *rope, const int32_t *po
     go((float *)nullptr);
 }
 
-void launch_cache_gather(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
-                         int G, int dh, float *k_out, float *v_out, cudaStream_t s) {
+namespace {
+HostReadPos launch_positions(const int32_t *pos, const int32_t *pos_d, int n_pos) {
+  HostReadPos p;
+  if (!pos_d) std::copy(pos, pos + n_pos, p.p);
+  return p;
+}
+}  // namespace
+
+void launch_cache_gather(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d, int n_pos,
+                         int l0, int l1, int G, int dh, float *k_out, float *v_out,
+                         cudaStream_t s) {
   size_t n = (size_t)n_pos * (l1 - l0) * G * dh;
   if (n == 0) return;
+  const HostReadPos p = launch_positions(pos, pos_d, n_pos);
   if (dtype == KVR_DTYPE_BF16)
-    k_cache_gather<__nv_bfloat16><<<grid_for(n, 256), 256, 0, s>>>(v, pos, n_pos, l0, l1 - l0, G,
-                                                                    dh, k_out, v_out);
+    k_cache_gather<__nv_bfloat16><<<grid_for(n, 256), 256, 0, s>>>(v, p, pos_d, n_pos, l0, l1 - l0,
+                                                                    G, dh, k_out, v_out);
   else
-    k_cache_gather<float><<<grid_for(n, 256), 256, 0, s>>>(v, pos, n_pos, l0, l1 - l0, G, dh,
+    k_cache_gather<float><<<grid_for(n, 256), 256, 0, s>>>(v, p, pos_d, n_pos, l0, l1 - l0, G, dh,
                                                             k_out, v_out);
 }
 
-void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
-                             int G, int dh, void *k_out, void *v_out, cudaStream_t s) {
+void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d,
+                             int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out,
+                             cudaStream_t s) {
   const int es = dtype == KVR_DTYPE_BF16 ? 2 : 4, vr = dh * es / 16;
   const size_t per_pos = (size_t)(l1 - l0) * G * vr;
   if (per_pos == 0) return;
@@ -834,8 +846,8 @@ void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, int n_pos,
   for (int p0 = 0; p0 < n_pos; p0 += chunk) {
     const int np = std::min(chunk, n_pos - p0);
     k_cache_gather_raw<<<grid_for(np * per_pos, 256), 256, 0, s>>>(
-        v, pos + p0, np, l0, l1 - l0, G, vr, es, (uint4 *)k_out + p0 * per_pos,
-        (uint4 *)v_out + p0 * per_pos);
+        v, launch_positions(pos + p0, pos_d, np), pos_d ? pos_d + p0 : nullptr, np, l0, l1 - l0, G,
+        vr, es, (uint4 *)k_out + p0 * per_pos, (uint4 *)v_out + p0 * per_pos);
   }
 }
 
@@ -843,11 +855,9 @@ void launch_cache_read_host(KVView v, int dtype, const int32_t *pos, const int32
                             int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out,
                             const int *flag_in, int *flag_out, cudaStream_t s) {
   const int es = dtype == KVR_DTYPE_BF16 ? 2 : 4, vr = dh * es / 16;
-  HostReadPos p;
-  if (!pos_d) std::copy(pos, pos + n_pos, p.p);
-  launch_pdl(k_cache_read_host, grid_for((size_t)n_pos * (l1 - l0) * G * vr, 256), 256, 0, s, v, p,
-             pos_d, n_pos, l0, l1 - l0, G, vr, es, (uint4 *)k_out, (uint4 *)v_out, flag_in,
-             flag_out);
+  launch_pdl(k_cache_read_host, grid_for((size_t)n_pos * (l1 - l0) * G * vr, 256), 256, 0, s, v,
+             launch_positions(pos, pos_d, n_pos), pos_d, n_pos, l0, l1 - l0, G, vr, es,
+             (uint4 *)k_out, (uint4 *)v_out, flag_in, flag_out);
 }
 
 void launch_cache_scatter_raw(KVView v, int dtype, int p0, int n_pos, const void *k_in,

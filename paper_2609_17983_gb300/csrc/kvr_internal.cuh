@@ -514,15 +514,18 @@ void launch_rope_scatter(const float *qkv, const float2 *rope, const int32_t *po
                          const Dims &dm, int layer, const KVView *views, const int32_t *rowdoc,
                          KVView single, float *q_out, void *qb_out, float qscale, bool write_kv,
                          cudaStream_t s, const SplitView *sv = nullptr, void *rows_out = nullptr);
-void launch_cache_gather(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
-                         int G, int dh, float *k_out, float *v_out, cudaStream_t s);
-// The same gather in the cache's element type (no widening).
-void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, int n_pos, int l0, int l1,
-                             int G, int dh, void *k_out, void *v_out, cudaStream_t s);
-// The same into page-locked host memory (16-byte aligned, fewer than 2^31 16-byte
-// pieces), positions from host memory (at most HOST_READ_MAX_POS) or, pos_d not
-// null, from the device, and the device error flag to *flag_out.
+// K/V rows of positions, widened to fp32.  Positions come from host memory, with the
+// launch (at most HOST_READ_MAX_POS), or, pos_d not null, from the device.
 constexpr int HOST_READ_MAX_POS = 512;
+void launch_cache_gather(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d, int n_pos,
+                         int l0, int l1, int G, int dh, float *k_out, float *v_out,
+                         cudaStream_t s);
+// The same gather in the cache's element type (no widening).
+void launch_cache_gather_raw(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d,
+                             int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out,
+                             cudaStream_t s);
+// The same into page-locked host memory (16-byte aligned, fewer than 2^31 16-byte
+// pieces), and the device error flag to *flag_out.
 void launch_cache_read_host(KVView v, int dtype, const int32_t *pos, const int32_t *pos_d,
                             int n_pos, int l0, int l1, int G, int dh, void *k_out, void *v_out,
                             const int *flag_in, int *flag_out, cudaStream_t s);
