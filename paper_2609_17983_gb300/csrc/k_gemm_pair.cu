@@ -60,6 +60,7 @@ constexpr int NT = 64 + EPI_THREADS;
 constexpr int PRE_WAIT_STAGES = 2;    // weight stages requested before the wait on the predecessor
 constexpr int MIN_UNITS = 4;          // units (of KS K blocks) a part of a tile has at least
 constexpr int MAX_PARTS = 8;          // clusters a left-over tile is split over at most
+constexpr int SUM_PARTS = 3;          // parts of a tile in flight while they are summed
 
 struct PairGemm : PairSplit {  // its units: KS K blocks (the last may be short)
   int M, N, KB;       // K blocks
@@ -325,34 +326,54 @@ __global__ void __launch_bounds__(NT, 1)
       tc_fence_after();
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + buf * ACC_COLS;
       for (int c = CC * eg; c < mv && !dead; c += CC * EPI_GROUPS) {
+        if (owner && parts > 1) {
+          // The others' parts in part order, then this cluster's own.  Sixteen rows of
+          // SUM_PARTS parts are in flight at once: with 32 rows of one part, seven parts
+          // took longer than the next tile's MMAs, and the tile after that waited for
+          // this buffer (4096 rows of 6144 x 4096, four tiles in eight parts: 133 -> 126
+          // us).  Four parts, 121 us, take 161 registers, and the next kernel no longer
+          // fits beside this one: passes were no faster.
+          for (int c2 = c; c2 < min(c + CC, mv); c2 += 16) {
+            float v[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = -0.f;  // exact: -0 + x = x
+            for (int k0 = 0; k0 < parts - 1; k0 += SUM_PARTS) {
+              float x[SUM_PARTS][16];
+#pragma unroll
+              for (int u = 0; u < SUM_PARTS; ++u) {
+                const size_t slot = 2 * part_cluster(p, g.tile, k0 + u) + rank;
+                const float *src = p.ws + (slot * 2 * 256 + c2) * BM + f;
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  x[u][j] = k0 + u < parts - 1 && c2 + j < mv ? __ldcg(src + (size_t)j * BM) : -0.f;
+              }
+#pragma unroll
+              for (int u = 0; u < SUM_PARTS; ++u)
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] += x[u][j];
+            }
+            uint32_t r[16];
+            tmem_ld16_nowait(taddr + c2, r);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] += __uint_as_float(r[j]);
+            if (n < p.N) epilogue16(p, t0 + c2, n, v, mv - c2);
+          }
+          continue;
+        }
         uint32_t r[CC];
-        float v[CC];
         tmem_ld32_nowait(taddr + c, r);
         tmem_wait_ld();
-#pragma unroll
-        for (int j = 0; j < CC; ++j) v[j] = __uint_as_float(r[j]);
         if (!owner) {
           float *dst = p.ws + ((size_t)blockIdx.x * 2 * 256 + c) * BM + f;
 #pragma unroll
           for (int j = 0; j < CC; ++j)
-            if (c + j < mv) dst[(size_t)j * BM] = v[j];
+            if (c + j < mv) dst[(size_t)j * BM] = __uint_as_float(r[j]);
           continue;
         }
-        if (parts > 1) {  // in part order, this cluster's own last
-          float s[CC];
-          for (int k = 0; k < parts - 1; ++k) {
-            const float *src =
-                p.ws +
-                ((size_t)(2 * part_cluster(p, g.tile, k) + rank) * 2 * 256 + c) * BM + f;
-            float x[CC];
+        float v[CC];
 #pragma unroll
-            for (int j = 0; j < CC; ++j) x[j] = c + j < mv ? __ldcg(src + (size_t)j * BM) : 0.f;
-#pragma unroll
-            for (int j = 0; j < CC; ++j) s[j] = k ? s[j] + x[j] : x[j];
-          }
-#pragma unroll
-          for (int j = 0; j < CC; ++j) v[j] = s[j] + v[j];
-        }
+        for (int j = 0; j < CC; ++j) v[j] = __uint_as_float(r[j]);
         if (n < p.N) {
           epilogue16(p, t0 + c, n, v, mv - c);
           if (c + 16 < mv) epilogue16(p, t0 + c + 16, n, v + 16, mv - c - 16);
