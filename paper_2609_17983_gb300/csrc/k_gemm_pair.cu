@@ -449,9 +449,9 @@ size_t configure(PairGemm &p, int M, int N, int K, int clusters, int smem_limit)
 // to the next kernel; only gate/up, which sums its own tiles, gains by pairs, where
 // their rounds are full and no tile is in more than two parts (193 to 256 rows, a
 // layer's GEMMs, RoPE and norms before over after: 4096 x 28672, 112 tiles for 76
-// clusters, 1.01 to 1.03; 3584 x 37888, 148 tiles, 1.00 to 1.03; 8192 x 57344 1.00
-// to 1.04; but 4096 x 22016, 10 of its 86 tiles in seven parts, 0.94 to 0.96, 4096 x
-// 32768, 128 tiles, 0.98 to 1.01) and the product is large (2304 x 18432, 72 tiles,
+// clusters, 1.00 to 1.03; 3584 x 37888, 148 tiles, 1.00 to 1.04; 8192 x 57344 1.01
+// to 1.04; but 4096 x 22016, 10 of its 86 tiles in seven parts, 0.97 to 0.99, 4096 x
+// 32768, 128 tiles, 0.98 to 1.02) and the product is large (2304 x 18432, 72 tiles,
 // 0.97, 2560 x 19456, 76 tiles, 0.95).  192 rows and below: equal at best.
 bool gemm_pair_takes(int M, int N, int K, int epi, int num_sms) {
   static const bool off = [] {
